@@ -23,7 +23,10 @@
  *  - A handle is not thread-safe: use one handle per host thread.  Work is enqueued on the
  *    handle's CUDA stream (its own by default, or the caller's via ch_set_stream); calls
  *    that return host data synchronise that stream only.
- *  - Precision: CH_FP64 keeps fields and all arithmetic in FP64.  CH_FP32 keeps fields,
+ *  - Precision: CH_FP64 keeps fields in FP64 and computes each step with at least FP64's
+ *    precision: by default in 64-bit fixed point scaled to the data (59 to 62 significant
+ *    bits; lines of 16 to 1024 points), in FP64 for other sizes, for values outside the
+ *    scaled range and whenever ch_tuning asks for a kernel shape.  CH_FP32 keeps fields,
  *    the stencil and the sweeps in FP32 (sweep coefficients computed in FP64, rounded
  *    once), while the F / dF/dt reductions, beta and its time average stay in FP64.
  */
@@ -175,7 +178,10 @@ int ch_launch_phase(ch_handle h, int phase);
 /*
  * Launch shape of a handle's kernels (no effect on results beyond round-off order within
  * a line's recurrence chunks; every choice is checked by the parity tests).  Fields <= 0
- * (split: -1) take the precision's default.
+ * (split: -1) take the precision's default.  With every field at its default, CH_FP64 members
+ * of 16 to 1024 points per axis and gamma dt / h^4 up to about 1e5 run in the fixed-point form,
+ * whose shapes follow from the member's size alone; setting a field (other than the CH_FP32
+ * ones, resident and resident_rows) selects the FP64 kernels described here.
  *   split       1: stencil and row sweep as separate kernels (default for CH_FP64: all
  *               threads of the stencil kernel do FP64 work, the sweeps run as many
  *               independent recurrences per SM); 0: one fused row kernel (default for

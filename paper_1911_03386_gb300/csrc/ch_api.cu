@@ -235,6 +235,111 @@ void seg_responses(double p1, double p2, int S, chk::SegTable* t) {
   }
 }
 
+// Fixed-point form (ch_fixed.cu): the scan tables of a line of n points in segments of S points
+// whose last one may be shorter (len points): A[d] = M^(S 2^d), P = M^len, B[l] = M^(S l) (I -
+// M^n)^-1 for segment l, B[32 + pos] = M^(distance of segment pos from the line's end) (I -
+// M^n)^-1, pos counted from the end.
+void fx_tables(double p1, double p2, int S, int n, chk::SegTable* t) {
+  std::memset(t, 0, sizeof *t);
+  const int G = (n + S - 1) / S, len = n - (G - 1) * S;
+  const double M[4] = {p1, p2, 1.0, 0.0};
+  double MS[4] = {1.0, 0.0, 0.0, 1.0}, ML[4] = {1.0, 0.0, 0.0, 1.0}, Mn[4] = {1.0, 0.0, 0.0, 1.0};
+  for (int k = 0; k < S; ++k) mat2_mul(M, MS, MS);
+  for (int k = 0; k < len; ++k) mat2_mul(M, ML, ML);
+  for (int k = 0; k + 1 < G; ++k) mat2_mul(MS, Mn, Mn);
+  mat2_mul(ML, Mn, Mn);
+  const double a = 1.0 - Mn[0], b = -Mn[1], c = -Mn[2], d = 1.0 - Mn[3], det = a * d - b * c;
+  const double P[4] = {d / det, -b / det, -c / det, a / det};
+  double Ad[4] = {MS[0], MS[1], MS[2], MS[3]};
+  for (int q = 0; q < 5 && (1 << q) < G; ++q) {
+    std::memcpy(t->A[q], Ad, sizeof Ad);
+    mat2_mul(Ad, Ad, Ad);
+  }
+  std::memcpy(t->P, ML, sizeof ML);
+  double F[4] = {P[0], P[1], P[2], P[3]}, R[4];
+  for (int l = 0; l < G; ++l) {
+    std::memcpy(t->B[l], F, sizeof F);
+    mat2_mul(MS, F, F);
+  }
+  std::memcpy(t->B[32], P, sizeof P);
+  mat2_mul(ML, P, R);
+  for (int pos = 1; pos < G; ++pos) {
+    std::memcpy(t->B[32 + pos], R, sizeof R);
+    mat2_mul(MS, R, R);
+  }
+}
+
+// v as h 2^32 + l with l signed (|v| < 2^63 - 2^31).
+chk::FxLimb fx_limb(double v) {
+  const long long q = std::llround(v);
+  chk::FxLimb r;
+  r.l = (int32_t)(uint32_t)(unsigned long long)q;
+  r.h = (int32_t)((q - r.l) >> 32);
+  return r;
+}
+
+// log2 bound of the gain of y_i = r_i + p1 y_{i-1} + p2 y_{i-2}: its impulse response's l1 norm.
+int fx_gain(double p1, double p2) {
+  double y1 = 1.0, y2 = 0.0, sum = 1.0;
+  for (int k = 0; k < 1000000; ++k) {
+    const double y = p1 * y1 + p2 * y2;
+    y2 = y1;
+    y1 = y;
+    sum += std::fabs(y);
+    if (std::fabs(y1) + std::fabs(y2) < 1e-18 * sum) break;
+  }
+  return (int)std::ceil(std::log2(sum * (1.0 + 1e-9)));
+}
+
+// Shapes of the fixed-point form: points per lane and rows per band of the row kernel, rows per
+// thread and columns per panel of the column kernel (256 threads).  Short lines take short
+// segments, whose serial chains set a small run's step time.
+int fx_seg_rows(int nx) { return nx <= 64 ? 8 : nx <= 128 ? 16 : 32; }
+int fx_class(int nx) { return nx <= 64 ? 0 : nx <= 128 ? 1 : nx <= 512 ? 2 : 3; }
+int fx_band(int nx) { return nx <= 64 || nx > 256 ? 8 : 16; }
+int fx_seg_cols(int ny) { return ny <= 64 ? 8 : ny <= 128 ? 16 : 32; }
+int fx_panel(int ny) { return ny <= 256 ? 32 : ny <= 512 ? 16 : 8; }
+
+// The member's constants of the fixed-point form; false where it does not apply: lines of 16 to
+// 1024 points whose recurrences gain at most 2^9 (s up to about 1e5: above, 64 bits minus the
+// gain's headroom would hold less than FP64).
+bool fx_params(MemberParams* p) {
+  if (p->nx < 16 || p->ny < 16 || p->nx > 1024 || p->ny > 1024) return false;
+  p->fx_gainx = fx_gain(p->p1x, p->p2x);
+  p->fx_gainy = fx_gain(p->p1y, p->p2y);
+  if (p->fx_gainx > 9 || p->fx_gainy > 9) return false;
+  p->fx_square = p->hx == p->hy;
+  // |C| < 2^E: |mu| / 2^E <= 3 + 4 (bx + by) for E <= 1 and |R'| <= 4 (1 + rho) |mu|, which has
+  // to fit 62 bits (60 where R' takes a product with rho)
+  const double bound = 4.0 * (1.0 + p->rho) * (3.0 + 4.0 * (p->bx + p->by));
+  p->fx_kmu = std::min(55, (p->fx_square ? 62 : 60) - (int)std::ceil(std::log2(bound)));
+  if (p->fx_kmu < 24) return false;
+  p->fx_su = 55 - p->fx_kmu;
+  int er = 0;
+  if (std::frexp(p->rho, &er) > 1.0 - 1e-9) ++er;  // rho < 2^er, not by rounding alone
+  p->fx_er = std::max(0, er + 1);
+  if (p->fx_er > 40) return false;
+  p->fx_rho = fx_limb(std::ldexp(p->rho, 64 - p->fx_er));
+  p->fx_bx = fx_limb(std::ldexp(p->bx, p->fx_kmu + 5));
+  p->fx_by = fx_limb(std::ldexp(p->by, p->fx_kmu + 5));
+  p->fx_cx = chk::FxCoef{fx_limb(std::ldexp(p->p1x, 61)), fx_limb(std::ldexp(p->p2x, 61))};
+  p->fx_cy = chk::FxCoef{fx_limb(std::ldexp(p->p1y, 61)), fx_limb(std::ldexp(p->p2y, 61))};
+  auto pow2 = [](int g) {
+    int w = 1;
+    while (w < g) w *= 2;
+    return w;
+  };
+  const int sx = fx_seg_rows(p->nx), sy = fx_seg_cols(p->ny);
+  p->fx_gx = (p->nx + sx - 1) / sx;
+  p->fx_gwx = pow2(p->fx_gx);
+  p->fx_gy = (p->ny + sy - 1) / sy;
+  p->fx_sx = sx;
+  p->fx_sy = sy;
+  p->fx_cw = fx_panel(p->ny);
+  p->fx_gwy = pow2(p->fx_gy);
+  return true;
+}
+
 bool is_pow2_upto32(int g) { return g >= 1 && g <= 32 && (g & (g - 1)) == 0; }
 
 }  // namespace chh
@@ -462,10 +567,17 @@ int build_tiles(ch_ensemble* h, const ch_tuning& t) {
   auto resident_rows = [&](const MemberParams& p) {
     return (t.resident_rows == 64 && p.nx == 256 && p.ny % 64 == 0) ? 64 : 32;
   };
+  // fixed-point form (CH_FP64): every member it applies to, unless the tuning asks for a shape
+  // of the other forms
+  const bool fx_on = f64 && (t.split < 0 || h->fx_fused) && t.stream < 0 && t.persist <= 0 && t.row_seg == 0 && t.col_seg == 0 &&
+                     t.rows_band == 0 && t.rows_p == 0 && t.sweep_band == 0 && t.cols_panel == 0 && t.cols_p == 0 &&
+                     t.threads == 0 && t.preroll_head == 0;
   int cwarps[4] = {8, 8, max_wp, max_wp};  // warps per CTA of each class
   for (int k = 0; k < h->m; ++k) {
-    if (!h->has(k) || resident(h->hp[k])) continue;
-    const MemberParams& p = h->hp[k];
+    if (!h->has(k)) continue;
+    MemberParams& p = h->hp[k];
+    p.fx = fx_on && fx_params(&p) ? 1 + fx_class(p.nx) : 0;
+    if (resident(p) || p.fx) continue;
     if (t.row_seg == 1 && !split && !rowT_fits(p))
       return fail(CH_EINVAL, "row_seg 1: some member's nx is not 32 times at most 16");
     if (t.row_seg > 1 && !row_fits(p, t.row_seg))
@@ -480,6 +592,7 @@ int build_tiles(ch_ensemble* h, const ch_tuning& t) {
   std::vector<Tile> rcl[chk::kResClasses];        // cluster-resident members by class
   std::vector<Tile> rtb;                          // stencil blocks of long rows (last)
   std::vector<Tile> rtT[17];                   // rows, transposed-block form, by nw
+  std::vector<Tile> fxr[chk::kFxRowClasses], fxc;  // fixed-point members: rows by class, columns
   chk::LaunchShape sh{};
   sh.split = split;
   sh.stream = stream;
@@ -508,6 +621,24 @@ int build_tiles(ch_ensemble* h, const ch_tuning& t) {
       seg_tables(p.p1x, p.p2x, p.nx / 16, 16, &h->hseg[k]);
       seg_tables(p.p1y, p.p2y, p.nx / 8, p.ny / (p.nx / 8), &h->hsegy[k]);
       seg_responses(p.p1y, p.p2y, p.nx / 8, &h->hsegy[k]);
+      continue;
+    }
+    if (p.fx) {
+      p.seg_g = p.row_t = p.col_s = 0;
+      p.kx32 = 0;
+      p.rows_p = p.cols_p = 1;
+      const int cr = fx_class(p.nx), br = std::min(p.ny, fx_band(p.nx)), cw = p.fx_cw;
+      fx_tables(p.p1x, p.p2x, fx_seg_rows(p.nx), p.nx, &h->hseg[k]);
+      fx_tables(p.p1y, p.p2y, fx_seg_cols(p.ny), p.ny, &h->hsegy[k]);
+      int b = 0;
+      for (int j0 = 0; j0 < p.ny; j0 += br, ++b) fxr[cr].push_back(Tile{k, j0, std::min(br, p.ny - j0), b, 0, 0});
+      sh.fx_smem[cr] = std::max(sh.fx_smem[cr], chk::fx_rows_smem(br, p.nx, fx_seg_rows(p.nx)));
+      sh.fx_cols_smem = std::max(sh.fx_cols_smem, chk::fx_cols_smem(p.fx_sy));
+      p.nbands = b;
+      p.partial_base = part;
+      part += b;
+      int q = 0;
+      for (int i0 = 0; i0 < p.nx; i0 += cw, ++q) fxc.push_back(Tile{k, i0, std::min(cw, p.nx - i0), q, 0, 0});
       continue;
     }
     const int rc = row_class(p), cc = col_class(p), ri = rc == 16 ? 0 : rc == 32 ? 1 : 2;
@@ -635,12 +766,19 @@ int build_tiles(ch_ensemble* h, const ch_tuning& t) {
   sh.rt_blk = (int)rtb.size();
   rt.insert(rt.end(), rtb.begin(), rtb.end());
   for (int c = 0; c < 4; ++c) cst.insert(cst.end(), csts[c].begin(), csts[c].end());
+  sh.fx_ct = (int)fxc.size();
+  cst.insert(cst.end(), fxc.begin(), fxc.end());
   std::vector<Tile> rest;
   for (int c = 0; c < chk::kResClasses; ++c) {
     sh.res_n[c] = (int)rcl[c].size();
     rest.insert(rest.end(), rcl[c].begin(), rcl[c].end());
   }
   sh.n_row_tiles = (int)rt.size();
+  for (int c = 0; c < chk::kFxRowClasses; ++c) {
+    sh.fx_rt[c] = (int)fxr[c].size();
+    sh.fx_tiles += sh.fx_rt[c];
+    rt.insert(rt.end(), fxr[c].begin(), fxr[c].end());
+  }
   sh.n_sweep_tiles = (int)st.size();
   sh.n_col_tiles = (int)ct.size();
   h->rest.swap(rest);
@@ -689,7 +827,8 @@ int upload_tiles(ch_ensemble* h) {
   if (!h->rest.empty())
     CH_CUDA(cudaMemcpyAsync(h->dres, h->rest.data(), sizeof(Tile) * h->rest.size(), cudaMemcpyHostToDevice, h->stream),
             "tiles");
-  if (h->shape.rt_seg[0] + h->shape.rt_seg[1] + h->shape.st_seg[0] + h->shape.st_seg[1] + n_rowT + h->rest.size())
+  if (h->shape.rt_seg[0] + h->shape.rt_seg[1] + h->shape.st_seg[0] + h->shape.st_seg[1] + n_rowT + h->rest.size() +
+      h->shape.fx_tiles)
     CH_CUDA(cudaMemcpyAsync(h->dseg, h->hseg.data(), sizeof(chk::SegTable) * h->m, cudaMemcpyHostToDevice, h->stream),
             "upload scan tables");
   if (!h->cst.empty())
@@ -736,7 +875,7 @@ int create_common(int m, const ch_member_desc* d, int precision, ch_handle* out)
   h->hp.resize(m);
   h->hseg.resize(m);
   h->hsegy.resize(m);
-  int64_t off = 0;
+  int64_t off = 0, rows = 0;
   for (int k = 0; k < m; ++k) {
     int rc = fill_params(d[k], precision, &h->hp[k]);
     if (rc) {
@@ -744,6 +883,8 @@ int create_common(int m, const ch_member_desc* d, int precision, ch_handle* out)
       return rc;
     }
     h->hp[k].offset = off;
+    h->hp[k].fx_wexp = rows;
+    rows += d[k].ny;
     const int64_t np = (int64_t)d[k].nx * d[k].ny;
     // keep every member's field 16-byte aligned
     off += (np + 3) & ~(int64_t)3;
@@ -757,6 +898,8 @@ int create_common(int m, const ch_member_desc* d, int precision, ch_handle* out)
       off += ((int64_t)d[k].nx * d[k].ny + 3) & ~(int64_t)3;
     }
   h->c_points = off;
+  h->w_points = h->total_points;
+  const size_t exp_bytes = precision == CH_FP64 ? sizeof(short2) * rows : 0;
   int rc = build_tiles(h, default_tuning());
   if (rc) {
     delete h;
@@ -773,7 +916,7 @@ int create_common(int m, const ch_member_desc* d, int precision, ch_handle* out)
   h->stream = h->own;
   auto alloc = [&](void** p, size_t bytes) -> cudaError_t { return chk::dev_malloc(p, bytes == 0 ? 16 : bytes); };
   if ((e = alloc(&h->C, h->elt * h->c_points)) != cudaSuccess ||
-      (e = alloc(&h->W, h->elt * h->total_points)) != cudaSuccess ||
+      (e = alloc(&h->W, h->elt * h->total_points + exp_bytes)) != cudaSuccess ||
       (e = alloc((void**)&h->dmp, sizeof(MemberParams) * m)) != cudaSuccess ||
       (e = alloc((void**)&h->dms, sizeof(MemberState) * m)) != cudaSuccess ||
       (e = alloc((void**)&h->dseg, sizeof(chk::SegTable) * m)) != cudaSuccess ||
@@ -787,7 +930,7 @@ int create_common(int m, const ch_member_desc* d, int precision, ch_handle* out)
                 std::string("device allocation: ") + cudaGetErrorString(e));
   }
   if ((e = chk::set_kernel_smem_limits(precision)) != cudaSuccess ||
-      (e = cudaMemsetAsync(h->W, 0, h->elt * h->total_points, h->stream)) != cudaSuccess) {
+      (e = cudaMemsetAsync(h->W, 0, h->elt * h->total_points + exp_bytes, h->stream)) != cudaSuccess) {
     int r = cuda_fail(e, "handle set-up");
     ch_destroy(h);
     return r;
@@ -816,7 +959,7 @@ int check_member(ch_handle h, int member) {
 // n single steps of the tiled kernels (every member outside the cluster-resident form).
 int launch_tiled_direct(ch_ensemble* h, int64_t n) {
   const chk::DevView v = h->view();
-  if (h->shape.n_row_tiles == 0) return CH_OK;
+  if (h->shape.n_row_tiles + h->shape.fx_tiles == 0) return CH_OK;
   for (int64_t i = 0; i < n; ++i) {
     cudaError_t e = chk::launch_step(v, h->precision, h->shape, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "step launch");
@@ -851,7 +994,7 @@ int fork_resident(ch_ensemble* h, int64_t n) {
   h->aux_used = 0;
   const int nc = chk::resident_classes(h->shape);
   if (nc == 0 || n <= 0) return CH_OK;
-  if (nc == 1 && h->shape.n_row_tiles == 0) {  // nothing to overlap with
+  if (nc == 1 && h->shape.n_row_tiles + h->shape.fx_tiles == 0) {  // nothing to overlap with
     CH_CUDA(chk::launch_resident(h->view(), h->precision, h->shape, n, &h->stream, 1), "resident step launch");
     return CH_OK;
   }
@@ -1025,7 +1168,7 @@ int ch_step(ch_handle h, int64_t nsteps) {
   // the other members' single steps on the handle's stream, replayed from a captured graph
   // where possible; the handle's stream then waits for both
   if (int rc = fork_resident(h, nsteps)) return rc;
-  if (h->shape.n_row_tiles > 0) {
+  if (h->shape.n_row_tiles + h->shape.fx_tiles > 0) {
     int64_t left = nsteps;
     if (can_graph && left >= kGraphSteps) {
       if (int rc = ensure_graph(h)) return rc;
@@ -1305,6 +1448,17 @@ int ch_debug_row_solve(ch_handle h, int member, double* out) {
   const double scale = p.dt / (p.hx * p.hx * p.cx);
   if (h->precision == CH_FP64) {
     if (int rc = copy_out(h, out, static_cast<double*>(h->W) + p.offset, sizeof(double) * np, "read W")) return rc;
+    if (p.fx) {  // 64-bit integers with an exponent per row (rows held in FP64: as they are)
+      std::vector<short2> ex(p.ny);
+      if (int rc = copy_out(h, ex.data(), h->view().wexp + p.fx_wexp, sizeof(short2) * ex.size(), "read W")) return rc;
+      for (int64_t i = 0; i < np; ++i) {
+        const short2 e = ex[i / p.nx];
+        if (e.y == chk::kBadRow) continue;
+        long long q;
+        std::memcpy(&q, out + i, sizeof q);
+        out[i] = std::ldexp((double)q, e.x);
+      }
+    }
     for (int64_t i = 0; i < np; ++i) out[i] *= scale;
     return CH_OK;
   }

@@ -1,0 +1,785 @@
+// ch_fixed.cu -- the CH_FP64 step in 64-bit fixed point (sm_103a).
+//
+// GB300's FP64 pipe takes 2 operations per SM and clock, so an FP64 recurrence step (2 FMA)
+// costs a warp 38 SM clocks; the same step in 64-bit fixed point (six 32 x 32 -> 64 bit
+// multiply-adds and a few adds) costs 8.7 (measured, 16 or more warps per SM).  The step of a
+// CH_FP64 member is therefore formed in 64-bit integers with power-of-two scales taken from
+// the data, which hold 59 to 63 significant bits where FP64 holds 53; the fields stay FP64 in
+// memory and the update C += kappa Z is one FP64 FMA.
+//
+//   fx_rows_kernel   a band of rows: C -> mu -> R' -> both row recurrences -> W (64-bit
+//                    integers, one exponent per row)
+//   fx_cols_kernel   a panel of up to 32 columns: both column recurrences of W, C += kappa Z
+//
+// Measured (us per step of a whole ensemble, the FP64 kernels before): 256 x 256^2 rows 207 +
+// columns 164 = 0.362 ms (stencil 0.334 + rows 0.196 + columns 0.241 = 0.762 ms); 16 x 1024^2
+// 0.432 ms (1.43 ms); 64^2 alone 20 us (70 us).  At 256^2 a point takes about 290 instructions of
+// the row kernel and 170 of the column kernel; both are bound by issue slots and the integer
+// multiply pipe (56 % and 44 % of the issue slots used), not by HBM (40 bytes per point, 0.1 ms).
+//
+// Scales.  x = C / 2^E with 2^E just above the band's largest |C| (E from an integer maximum
+// over the loaded values); C enters as x 2^59, mu as mu 2^(kmu - E), where kmu leaves room
+// for the largest R' the stencil can form from such a band (so mu's unit is a few bits below
+// the rounding of the FP64 formula, whose terms 4 (bx + by) C are as large), R' is formed
+// from mu exactly where hx = hy.  Each recurrence y_i = r_i + p1 y_{i-1} + p2 y_{i-2} then
+// runs on r shifted so that its row's (or panel's) largest value sits g bits below 2^62, 2^g
+// a bound of the recurrence's gain (the l1 norm of its impulse response), and its result is
+// shifted the same way before the backward one.
+//
+// A band whose largest |C| is outside [2^-200, 2), or not finite, is taken through the same
+// code in FP64 arithmetic (the Fp policy), its rows marked kBadRow; the columns of a member
+// with such a row run in FP64 too.
+//
+// Lines of n points are split into G = ceil(n / S) segments of S points (the last one may be
+// shorter), one lane (rows) or warp (columns) per segment.  Each recurrence is a pass from a
+// zero state over every segment, a Kogge-Stone scan of the end states in FP64 (its 24
+// operations per segment and pass overlap with the integer work) and a pass from the exact
+// periodic start state.
+#include <cstdint>
+#include <type_traits>
+
+#include <cuda_runtime.h>
+
+#include "ch_device.cuh"
+#include "ch_internal.h"
+
+namespace chk {
+namespace {
+
+using i64 = long long;
+constexpr unsigned kAll = 0xffffffffu;
+
+// -------------------------------------------------------------------------------------
+// 64-bit fixed point
+// -------------------------------------------------------------------------------------
+// a b + c, 32 x 32 -> 64 bits, signed.
+__device__ __forceinline__ i64 madw(int a, int b, i64 c) {
+  i64 d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+}
+
+// v = h 2^32 + l with l signed (so that every partial product is a signed one).
+__device__ __forceinline__ FxLimb limbs(i64 v) {
+  FxLimb q;
+  q.l = (int)v;
+  q.h = (int)(v >> 32) + (int)((unsigned)q.l >> 31);
+  return q;
+}
+
+// a b / 2^64 for |a| <= 2^62, |b| < 2^63, to about one unit: the product of the low limbs (at most
+// 1/4 unit) is left out, the middle products are rounded.
+__device__ __forceinline__ i64 mul_top(FxLimb a, FxLimb b) {
+  const i64 mid = madw(a.l, b.h, madw(a.h, b.l, 1ll << 31));
+  return madw(a.h, b.h, mid >> 32);
+}
+
+// v / 2^r (1 <= r <= 62), rounded to nearest, halves away from zero (a rounding that is not odd
+// in v would bias every point of a field the same way, and the mean is the mode that the solves
+// damp least).
+__device__ __forceinline__ i64 shift_down(i64 v, int r) { return (v + ((1ll << r) >> 1) + (v >> 63)) >> r; }
+
+// v 2^s for |s| <= 62: f(operation) with the operation for the sign of s (s the same in a warp).
+template <class F>
+__device__ __forceinline__ void with_shift(int s, const F& f) {
+  if (s >= 0)
+    f([s](i64 v) { return v << s; });
+  else
+    f([s](i64 v) { return shift_down(v, -s); });
+}
+
+// (double)v, truncated to 53 bits (it is the update of C, far below C itself), on the integer
+// pipes: the conversion instruction takes the FP64 pipe 16 SM clocks per warp, which the update
+// and the scans need.
+__device__ __forceinline__ double to_double(i64 v) {
+  const i64 s = v >> 63;
+  const unsigned long long m = (unsigned long long)((v ^ s) - s);
+  const int lz = __clzll((i64)m);
+  const unsigned long long q = (m << lz) >> 11;  // 53 bits, the leading one adds 1 to the exponent
+  const int hi = (int)(q >> 32) + ((1085 - lz) << 20) + ((int)(s >> 32) & 0x80000000);
+  return m == 0 ? 0.0 : __hiloint2double(hi, (int)q);
+}
+
+// x 2^(59 - E) for |x| < 2^E, E = emax - 1022, from the fields of the binary64 value: the
+// 53-bit significand moved up by 6 bits, then down by the distance of its exponent from emax.
+__device__ __forceinline__ i64 to_fixed(i64 bits, int emax) {
+  const int hi = (int)(bits >> 32);
+  const int e = (hi >> 20) & 0x7ff;
+  const i64 m = ((i64)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)bits) << 6;
+  const i64 v = m >> min(emax - e, 63);
+  const i64 s = hi >> 31;
+  return (v ^ s) - s;
+}
+
+// Asynchronous global -> shared copy of one value.
+__device__ __forceinline__ void copy8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+__device__ __forceinline__ i64 double_bits(double x) { return __double_as_longlong(x); }
+
+// Arithmetic of the recurrences: fixed point ...
+struct Fx {
+  using State = FxLimb;
+  FxLimb p1, p2;  // p / 8, times 2^64
+  unsigned top = 0;  // OR of the magnitudes' high words
+  __device__ __forceinline__ Fx(const FxCoef& c, double, double) : p1(c.p1), p2(c.p2) {}
+  static __device__ __forceinline__ State zero() { return FxLimb{0, 0}; }
+  // y = r + p1 a + p2 b to about one unit, for |a|, |b|, |y| < 2^62: the middle products are at most
+  // 2^61 (l p1.h), 2^60 (l p2.h) and 2^61 (h p.l), so their sum stays below 2^63.  They start at 2^63
+  // + 2^28, so that the sum is unsigned and its shift rounds; the high products take the 2^63 back.
+  __device__ __forceinline__ i64 step(State a, State b, i64 r) const {
+    i64 lo = madw(b.l, p2.h, (i64)((1ull << 63) + (1ull << 28)));
+    lo = madw(b.h, p2.l, lo);
+    i64 hi = madw(b.h, p2.h, -(1ll << 31));
+    lo = madw(a.l, p1.h, lo);
+    lo = madw(a.h, p1.l, lo);
+    hi = madw(a.h, p1.h, hi);
+    return r + (hi << 3) + (i64)((unsigned long long)lo >> 29);
+  }
+  static constexpr bool kFixed = true;
+  static __device__ __forceinline__ State state(i64 y) { return limbs(y); }
+  static __device__ __forceinline__ double value(State s) { return (double)(((i64)s.h << 32) + s.l); }
+  static __device__ __forceinline__ State start(double x) { return limbs(__double2ll_rn(x)); }
+  __device__ __forceinline__ void track(i64 y) {
+    const int h = (int)(y >> 32);
+    top |= (unsigned)(h ^ (h >> 31));
+  }
+};
+
+// ... and FP64 (values held as their bits).
+struct Fp {
+  using State = double;
+  double p1, p2;
+  unsigned top = 0;
+  __device__ __forceinline__ Fp(const FxCoef&, double q1, double q2) : p1(q1), p2(q2) {}
+  static __device__ __forceinline__ State zero() { return 0.0; }
+  __device__ __forceinline__ i64 step(State a, State b, i64 r) const {
+    return double_bits(fma(p1, a, fma(p2, b, __longlong_as_double(r))));
+  }
+  static constexpr bool kFixed = false;
+  static __device__ __forceinline__ State state(i64 y) { return __longlong_as_double(y); }
+  static __device__ __forceinline__ double value(State s) { return s; }
+  static __device__ __forceinline__ State start(double x) { return x; }
+  __device__ __forceinline__ void track(i64) {}
+};
+
+// One pass of a recurrence over a segment of len values in shared memory, `es` elements apart
+// (p: its first value in the pass's direction, es negative for the backward one), from the
+// state (a, b); the loads of four values are issued ahead of the chain.  PRE: each value is first
+// replaced by pre(value).  STORE: the solution replaces the values.
+template <bool STORE, bool PRE, class A, class Pre>
+__device__ __forceinline__ void pass(A& ar, i64* p, int es, int len, typename A::State& a, typename A::State& b,
+                                     const Pre& pre) {
+  auto one = [&](i64 r, i64* at) {
+    if constexpr (PRE) {
+      r = pre(r);
+      *at = r;
+    }
+    const i64 t = ar.step(a, b, r);
+    if constexpr (STORE) {
+      *at = t;
+      ar.track(t);
+    }
+    b = a;
+    a = A::state(t);
+  };
+  int k = 0;
+#pragma unroll 1
+  for (; k + 4 <= len; k += 4) {
+    i64 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = p[u * es];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) one(v[u], p + u * es);
+    p += 4 * es;
+  }
+#pragma unroll 1
+  for (; k < len; ++k) {
+    one(*p, p);
+    p += es;
+  }
+}
+// The zero-state pass over the values shifted by sl (FP64: unshifted), and the pass from a state.
+template <class A>
+__device__ __forceinline__ void pass_end(A& ar, i64* p, int es, int len, int sl, typename A::State& a,
+                                         typename A::State& b) {
+  a = A::zero();
+  b = A::zero();
+  if constexpr (A::kFixed)
+    with_shift(sl, [&](auto sh) { pass<false, true>(ar, p, es, len, a, b, sh); });
+  else
+    pass<false, false>(ar, p, es, len, a, b, 0);
+}
+template <class A>
+__device__ __forceinline__ void pass_full(A& ar, i64* p, int es, int len, typename A::State a, typename A::State b) {
+  ar.top = 0;
+  pass<true, false>(ar, p, es, len, a, b, 0);
+}
+
+// Start states of the segments of one line from their end states, one lane per segment (the
+// first G of gw consecutive lanes, gw a power of two; l = lane within them).  The line's last
+// segment may be shorter than the others; tab.A[d] = M^(S 2^d), tab.P = M^(length of the last
+// segment), tab.B[l] = M^(S l) P, tab.B[32 + pos] = M^(distance from the line's end) P with P
+// = (I - M^n)^-1, all in shared memory.  (a, b): end state in, start state out.
+struct ScanTab {
+  double A[5][4], P[4], B[64][4];
+};
+__device__ __forceinline__ void load_tab(ScanTab& t, const SegTable& g) {
+  const double* src = &g.A[0][0];
+  for (int k = threadIdx.x; k < 20; k += blockDim.x) (&t.A[0][0])[k] = src[k];
+  for (int k = threadIdx.x; k < 256; k += blockDim.x) (&t.B[0][0])[k] = (&g.B[0][0])[k];
+  if (threadIdx.x < 4) t.P[threadIdx.x] = g.P[threadIdx.x];
+}
+
+template <bool REV>
+__device__ __forceinline__ void scan_states(const ScanTab& tab, double& a, double& b, int l, int G, int gw) {
+  const int pos = REV ? G - 1 - l : l;
+  const double e0 = a, e1 = b;
+#pragma unroll
+  for (int d = 0; d < 5; ++d) {
+    const int delta = 1 << d;
+    if (delta < gw) {
+      const double ya = REV ? __shfl_down_sync(kAll, a, delta, gw) : __shfl_up_sync(kAll, a, delta, gw);
+      const double yb = REV ? __shfl_down_sync(kAll, b, delta, gw) : __shfl_up_sync(kAll, b, delta, gw);
+      if (pos >= delta) {
+        const double na = fma(tab.A[d][0], ya, fma(tab.A[d][1], yb, a));
+        b = fma(tab.A[d][2], ya, fma(tab.A[d][3], yb, b));
+        a = na;
+      }
+    }
+  }
+  double xa = REV ? __shfl_down_sync(kAll, a, 1, gw) : __shfl_up_sync(kAll, a, 1, gw);
+  double xb = REV ? __shfl_down_sync(kAll, b, 1, gw) : __shfl_up_sync(kAll, b, 1, gw);
+  if (pos == 0) xa = xb = 0.0;
+  double ta = a, tb = b;
+  if (!REV) {  // the last segment's own length
+    ta = fma(tab.P[0], xa, fma(tab.P[1], xb, e0));
+    tb = fma(tab.P[2], xa, fma(tab.P[3], xb, e1));
+  }
+  ta = __shfl_sync(kAll, ta, REV ? 0 : G - 1, gw);
+  tb = __shfl_sync(kAll, tb, REV ? 0 : G - 1, gw);
+  const double* B = tab.B[REV ? 32 + max(pos, 0) : min(l, 31)];
+  a = fma(B[0], ta, fma(B[1], tb, xa));
+  b = fma(B[2], ta, fma(B[3], tb, xb));
+}
+
+__device__ __forceinline__ int bit_length_hi(unsigned top) { return 64 - __clz((int)top); }  // >= 32
+
+// -------------------------------------------------------------------------------------
+// Rows
+// -------------------------------------------------------------------------------------
+// mu at c with neighbours e, w, n, s (SQ: hx = hy, one product for both directions).  The cubic
+// term: (C^2 - 1) 2^(60 - su) from C^2's product by one shift (sh = 2 E + 6 - su), times C.
+template <bool SQ, class Shift>
+struct MuFx {
+  FxLimb pbx, pby;
+  i64 one;
+  Shift sh;
+  __device__ __forceinline__ i64 operator()(i64 c, i64 e, i64 w, i64 n, i64 s) const {
+    const FxLimb cl = limbs(c);
+    const i64 u = mul_top(cl, limbs(sh(mul_top(cl, cl)) - one));
+    const i64 lx = e + w - 2 * c, ly = n + s - 2 * c;
+    if (SQ) return u - mul_top(limbs(lx + ly), pbx);
+    return u - mul_top(limbs(lx), pbx) - mul_top(limbs(ly), pby);
+  }
+};
+struct MuFp {
+  double a, bx, by;
+  __device__ __forceinline__ i64 operator()(i64 c_, i64 e_, i64 w_, i64 n_, i64 s_) const {
+    const double c = __longlong_as_double(c_), e = __longlong_as_double(e_), w = __longlong_as_double(w_),
+                 n = __longlong_as_double(n_), s = __longlong_as_double(s_);
+    return double_bits(fma(-by, s + n, fma(-bx, e + w, c * fma(c, c, -a))));
+  }
+};
+// R' at m with neighbours e, w, n, s (SQ: hx = hy, exact).
+template <bool SQ>
+struct RhsFx {
+  FxLimb rho;
+  int er;
+  __device__ __forceinline__ i64 operator()(i64 m, i64 e, i64 w, i64 n, i64 s) const {
+    const i64 dx = e + w - 2 * m, dy = n + s - 2 * m;
+    return SQ ? dx + dy : dx + mul_top(limbs(dy << er), rho);
+  }
+};
+struct RhsFp {
+  double rho, w0;
+  __device__ __forceinline__ i64 operator()(i64 m_, i64 e_, i64 w_, i64 n_, i64 s_) const {
+    const double m = __longlong_as_double(m_), e = __longlong_as_double(e_), w = __longlong_as_double(w_),
+                 n = __longlong_as_double(n_), s = __longlong_as_double(s_);
+    return double_bits(fma(w0, m, fma(rho, s + n, e + w)));
+  }
+};
+
+// One band of nr rows (up to TH / gw).  The band's C rows (with two halo rows on each side) go to
+// a shared-memory tile whose rows are padded by one value per segment of S, so that lanes S + 1
+// values apart fall in distinct banks.  Warps take strips of 32 columns down the rows, twice and
+// in place: mu from three C rows in registers and the neighbouring lanes, written over the C row
+// above, then R' from three mu rows the same way (strip edges of both through shared memory).
+// Then gw lanes take each row for both recurrences.  All of it runs in short loops over shared
+// memory: fully unrolled register forms of this kernel spent a third of their cycles fetching
+// instructions, and their registers held an SM to 16 warps.
+struct Band {
+  i64* tile;
+  int pitch, ls;       // tile pitch; log2 S: column i at i + (i >> ls)
+  int nx, ns, nr;      // columns, strips, band rows
+};
+
+// First element of an edge column (rows values) of a strip.
+__device__ __forceinline__ int edge_index(int rows, int strip, int side) { return (2 * strip + side) * rows; }
+
+// A walk of every strip down `rows` output rows: out row r = f(c, e, w, n, s) with n, c, s the
+// input rows r, r + 1, r + 2 (conv applied on entry), written over input row r.  Ein: edge columns
+// of the input rows; each output row goes to `sink` (value, row, valid lane) before it is stored.
+template <class Conv, class F, class Sink>
+__device__ __forceinline__ void walk_strips(const Band& b, int rows, const i64* Ein, const Conv& conv, const F& f,
+                                            const Sink& sink) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int s = threadIdx.x >> 5; s < b.ns; s += nw) {
+    const int last = min(31, b.nx - 1 - 32 * s);
+    const int i = 32 * s + min(lane, last);
+    i64* col = b.tile + i + (i >> b.ls);
+    // west edge of lane 0: right edge of the strip before; east edge of the last lane: left edge
+    // of the strip after
+    const i64* ew = Ein + edge_index(rows + 2, s == 0 ? b.ns - 1 : s - 1, 1) + 1;
+    const i64* ee = Ein + edge_index(rows + 2, s + 1 == b.ns ? 0 : s + 1, 0) + 1;
+    i64 n = conv(col[0]), c = conv(col[b.pitch]);
+#pragma unroll 2
+    for (int r = 0; r < rows; ++r) {
+      const i64 so = conv(col[2 * b.pitch]);
+      i64 w = __shfl_up_sync(kAll, c, 1), e = __shfl_down_sync(kAll, c, 1);
+      if (lane == 0) w = ew[r];
+      if (lane == last) e = ee[r];
+      const i64 m = f(c, e, w, n, so);
+      sink(m, s, r, lane, last);
+      if (lane <= last) col[0] = m;
+      col += b.pitch;
+      n = c;
+      c = so;
+    }
+  }
+}
+
+// mu, then R' (with the OR of its magnitudes in top), over the tile.
+template <bool FIXED, class Mu, class Rhs>
+__device__ __forceinline__ void band_rhs(const Band& b, i64* Es, i64* Em, unsigned& top, int emax, const Mu& mu,
+                                         const Rhs& rhs) {
+  walk_strips(
+      b, b.nr + 2, Es, [emax](i64 c) { return FIXED ? to_fixed(c, emax) : c; }, mu,
+      [&](i64 m, int s, int r, int lane, int last) {
+        if (lane == 0) Em[edge_index(b.nr + 2, s, 0) + r] = m;
+        if (lane == last) Em[edge_index(b.nr + 2, s, 1) + r] = m;
+      });
+  __syncthreads();
+  top = 0;
+  walk_strips(
+      b, b.nr, Em, [](i64 m) { return m; }, rhs,
+      [&](i64 m, int, int, int lane, int last) {
+        const int h = (int)(m >> 32);
+        if (FIXED && lane <= last) top |= (unsigned)(h ^ (h >> 31));
+      });
+}
+
+// OR of `top` over the CTA (slots: one per warp, not in use; ends with every thread past it).
+template <int NW>
+__device__ __forceinline__ unsigned cta_or(unsigned top, unsigned* slots) {
+  const int lane = threadIdx.x & 31;
+  top = __reduce_or_sync(kAll, top);
+  if (lane == 0) slots[threadIdx.x >> 5] = top;
+  __syncthreads();
+  return __reduce_or_sync(kAll, lane < NW ? slots[lane] : 0u);
+}
+
+// Both recurrences of a row: segment seg (len points) of lane l of gw, G of them in use; top: OR of
+// the band's |R'|.  The band shares its shifts, so a band of W has one exponent.
+template <int NW, class A>
+__device__ __forceinline__ void row_solve(i64* seg, int len, int l, int G, int gw, A ar, const ScanTab& tab, int gain,
+                                          unsigned top, unsigned* slots, int& e_lsb, int& e_top) {
+  const int sl = 62 - gain - bit_length_hi(cta_or<NW>(top, slots));
+  typename A::State a, b;
+  pass_end(ar, seg, 1, len, sl, a, b);
+  double ea = A::value(a), eb = A::value(b);
+  scan_states<false>(tab, ea, eb, l, G, gw);
+  pass_full(ar, seg, 1, len, A::start(ea), A::start(eb));
+  const int sl2 = 62 - gain - bit_length_hi(cta_or<NW>(ar.top, slots + NW));
+  i64* end = seg + max(len - 1, 0);
+  pass_end(ar, end, -1, len, sl2, a, b);
+  ea = A::value(a);
+  eb = A::value(b);
+  scan_states<true>(tab, ea, eb, l, G, gw);
+  pass_full(ar, end, -1, len, A::start(ea), A::start(eb));
+  e_lsb = -sl - sl2;
+  e_top = e_lsb + bit_length_hi(cta_or<NW>(ar.top, slots + 2 * NW));
+}
+
+template <int TH, int MINB>
+__global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_base) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ unsigned wtop[4 * (TH / 32)];
+  const Tile tl = v.row_tiles[tile_base + blockIdx.x];
+  const MemberParams& P = v.mp[tl.member];
+  MemberState* st = v.ms + tl.member;
+  bool sample;
+  if (!stencil_prologue(tl, st, P, sample)) return;
+  constexpr int NW = TH / 32;
+  const int nx = P.nx, ny = P.ny, j0 = tl.start, nr = tl.count, S = P.fx_sx, G = P.fx_gx, gw = P.fx_gwx;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  ScanTab& tab = *reinterpret_cast<ScanTab*>(smem);
+  Band b;
+  b.tile = reinterpret_cast<i64*>(smem + sizeof(ScanTab));
+  b.pitch = G * (S + 1);
+  b.ls = __ffs(S) - 1;
+  b.nx = nx;
+  b.ns = (nx + 31) >> 5;
+  b.nr = nr;
+  i64* Es = b.tile + (nr + 4) * b.pitch;
+  i64* Em = Es + 2 * b.ns * (nr + 4);
+  double* red = reinterpret_cast<double*>(Em + 2 * b.ns * (nr + 2));
+
+  // C rows j0 - 2 .. j0 + nr + 1 (periodic) into the tile
+  {
+    const i64* Cg = static_cast<const i64*>(v.C) + P.offset;
+    for (int s = warp; s < b.ns; s += NW) {
+      const int i = min(32 * s + lane, nx - 1);
+      i64* col = b.tile + i + (i >> b.ls);
+      int j = j0 - 2 < 0 ? j0 - 2 + ny : j0 - 2;
+      const i64* src = Cg + (int64_t)j * nx + i;
+#pragma unroll 4
+      for (int t = 0; t < nr + 4; ++t) {
+        copy8(col, src);
+        col += b.pitch;
+        src += nx;
+        if (++j == ny) {
+          j = 0;
+          src = Cg + i;
+        }
+      }
+    }
+  }
+  load_tab(tab, v.seg[tl.member]);
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  unsigned top = 0;
+  for (int s = warp; s < b.ns; s += NW) {  // this thread's own copies
+    const int i = min(32 * s + lane, nx - 1);
+    const int2* col = reinterpret_cast<const int2*>(b.tile + i + (i >> b.ls));
+#pragma unroll 4
+    for (int t = 0; t < nr + 4; ++t) top = max(top, (unsigned)col[t * b.pitch].y & 0x7fffffffu);
+  }
+  top = __reduce_max_sync(kAll, top);
+  if (lane == 0) wtop[warp] = top;
+  __syncthreads();
+  top = __reduce_max_sync(kAll, lane < NW ? wtop[lane] : 0u);
+  const int emax = (int)(top >> 20);  // biased exponent of the largest |C|
+  const bool bad = emax > 1023 || emax < 823;
+  // the strips' edge columns
+  for (int k = threadIdx.x; k < 2 * b.ns * (nr + 4); k += TH) {
+    const int e = k / (nr + 4), t = k - e * (nr + 4);
+    const int i = min(16 * (e & ~1) + 31 * (e & 1), nx - 1);
+    const i64 c = b.tile[t * b.pitch + i + (i >> b.ls)];
+    Es[k] = bad ? c : to_fixed(c, emax);
+  }
+  __syncthreads();
+  if (bad)
+    band_rhs<false>(b, Es, Em, top, emax, MuFp{P.a, P.bx, P.by}, RhsFp{P.rho, P.w0});
+  else
+    with_shift(2 * (emax - 1022) + 6 - P.fx_su, [&](auto sh) {
+      const i64 one = 1ll << (60 - P.fx_su);
+      if (P.fx_square)
+        band_rhs<true>(b, Es, Em, top, emax, MuFx<true, decltype(sh)>{P.fx_bx, P.fx_by, one, sh},
+                       RhsFx<true>{P.fx_rho, P.fx_er});
+      else
+        band_rhs<true>(b, Es, Em, top, emax, MuFx<false, decltype(sh)>{P.fx_bx, P.fx_by, one, sh},
+                       RhsFx<false>{P.fx_rho, P.fx_er});
+    });
+  if (sample)
+    band_partials_mu64<double>(v, tl, nx, nr, P, v.partials + P.partial_base + tl.index, red);
+
+  // rows: gw lanes per row (row_solve starts with a barrier: R' is complete)
+  const int l = lane & (gw - 1), row = threadIdx.x / gw, r = min(row, nr - 1);
+  const int len = l < G && row < nr ? min(S, nx - l * S) : 0;
+  i64* seg = b.tile + r * b.pitch + l * (S + 1);
+  int e_lsb, e_top;
+  if (bad)
+    row_solve<NW>(seg, len, l, G, gw, Fp(P.fx_cx, P.p1x, P.p2x), tab, 0, 0u, wtop + NW, e_lsb, e_top);
+  else
+    row_solve<NW>(seg, len, l, G, gw, Fx(P.fx_cx, 0.0, 0.0), tab, P.fx_gainx, top, wtop + NW, e_lsb, e_top);
+  if (row < nr && l == 0) {
+    const int eb = emax - 1022 - P.fx_kmu;
+    v.wexp[P.fx_wexp + j0 + row] = bad ? make_short2(0, kBadRow) : make_short2((short)(e_lsb + eb), (short)(e_top + eb));
+  }
+  // W to HBM as whole rows (row_solve ends with a barrier)
+  i64* Wg = static_cast<i64*>(v.W) + P.offset + (int64_t)j0 * nx;
+  for (int q = warp; q < nr; q += NW) {
+    const i64* src = b.tile + q * b.pitch;
+    i64* dst = Wg + q * nx;
+#pragma unroll 4
+    for (int i = lane; i < nx; i += 32) dst[i] = src[i + (i >> b.ls)];
+  }
+}
+
+// Observables of the current fields (ch_observables): the partials of one band.
+__global__ void __launch_bounds__(256) fx_observe_kernel(DevView v, int tile_base) {
+  __shared__ double red[16];
+  const Tile tl = v.row_tiles[tile_base + blockIdx.x];
+  const MemberParams& P = v.mp[tl.member];
+  band_partials_mu64<double>(v, tl, P.nx, tl.count, P, v.partials + P.partial_base + tl.index, red);
+}
+
+// -------------------------------------------------------------------------------------
+// Columns
+// -------------------------------------------------------------------------------------
+// A CTA of 256 threads takes a panel of cw columns (32, 16 or 8), thread = segment tid / cw of S
+// rows of column tid % cw, its values in shared memory (value u of thread t at u 256 + t: no bank
+// conflicts).  The first pass runs as W arrives, the last one updates C.
+constexpr int kColThreads = 256;
+constexpr int kXsMax = 32 * 9;  // state exchange: G x (cw + 1), G cw <= 256
+
+template <class A>
+__device__ __forceinline__ int col_solve(A& ar, i64* y, int len, const ScanTab& tab, double2* xs, unsigned* wtop, int G,
+                                         int gw, int cw, int gain, typename A::State& a, typename A::State& b) {
+  const int seg = threadIdx.x / cw, c = threadIdx.x - seg * cw;
+  const int l = threadIdx.x & (gw - 1), sc = threadIdx.x / gw;  // scan: segment l of column sc
+  auto exchange = [&](bool rev) {  // end state of this thread's segment in, its start state out
+    if (seg < G) xs[seg * (cw + 1) + c] = make_double2(A::value(a), A::value(b));
+    __syncthreads();
+    double2* p = xs + min(l, G - 1) * (cw + 1) + min(sc, cw - 1);
+    double2 e = *p;
+    if (rev)
+      scan_states<true>(tab, e.x, e.y, l, G, gw);
+    else
+      scan_states<false>(tab, e.x, e.y, l, G, gw);
+    if (l < G && sc < cw) *p = e;
+    __syncthreads();
+    e = xs[min(seg, G - 1) * (cw + 1) + c];
+    a = A::start(e.x);
+    b = A::start(e.y);
+  };
+  exchange(false);
+  pass_full(ar, y, kColThreads, len, a, b);
+  // the panel's largest |y| sets the shift before the backward recurrence
+  const int sl = 62 - gain - bit_length_hi(cta_or<kColThreads / 32>(ar.top, wtop));
+  pass_end(ar, y + max(len - 1, 0) * kColThreads, -kColThreads, len, sl, a, b);
+  exchange(true);
+  return sl;
+}
+
+// The backward pass from its start state and the update C += kap x (y, Cg: the segment's last row),
+// 4 rows at a time, the next 4 rows of C in flight.
+template <class A, class Conv>
+__device__ __forceinline__ void col_update(const A& ar, const i64* y, int len, double* Cg, int nx, double kap, bool cv,
+                                           typename A::State a, typename A::State b, Conv conv) {
+  double nc[4];
+  const double* q = Cg;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    if (u < len && cv) nc[u] = *q;
+    q -= nx;
+  }
+#pragma unroll 1
+  for (int k = len; k > 0; k -= 4) {
+    double cc[4];
+    i64 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      cc[u] = nc[u];
+      if (u < k) v[u] = y[-u * kColThreads];
+      if (u + 4 < k && cv) nc[u] = *q;
+      q -= nx;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (u < k) {
+        const i64 t = ar.step(a, b, v[u]);
+        b = a;
+        a = A::state(t);
+        if (cv) *Cg = fma(kap, conv(t), cc[u]);
+        Cg -= nx;
+      }
+    y -= 4 * kColThreads;
+  }
+}
+
+// The scaled forward pass from a zero state over W as its copies arrive, in 4 groups of S / 4 rows
+// per segment.  Rows come in bands of one exponent that start at multiples of 8 (ws: the segment's
+// row exponents).
+template <class A, class Scaled>
+__device__ __forceinline__ void col_first(const A& ar, i64* y, int len, int S, const short2* ws,
+                                          typename A::State& a, typename A::State& b, const Scaled& scaled) {
+  a = A::zero();
+  b = A::zero();
+  const int per = max(S >> 2, 8);
+#pragma unroll 1
+  for (int k = 0; k < S; k += 8) {
+    if (k == 0)
+      asm volatile("cp.async.wait_group 3;\n" ::: "memory");
+    else if (k == per)
+      asm volatile("cp.async.wait_group 2;\n" ::: "memory");
+    else if (k == 2 * per)
+      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    else
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();
+    if (k < len)
+      scaled(ws[k], [&](auto sh) {
+        i64 w[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (k + u < len) w[u] = y[u * kColThreads];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (k + u < len) {
+            const i64 r = sh(w[u]);
+            y[u * kColThreads] = r;
+            const i64 t = ar.step(a, b, r);
+            b = a;
+            a = A::state(t);
+          }
+      });
+    y += 8 * kColThreads;
+  }
+}
+
+__global__ void __launch_bounds__(kColThreads, 3) fx_cols_kernel(DevView v, int tile_base) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(16) double2 xs[kXsMax];
+  __shared__ ScanTab tab;
+  __shared__ unsigned wtop[kColThreads / 32];
+  const Tile tl = v.colseg_tiles[tile_base + blockIdx.x];
+  MemberState* st = v.ms + tl.member;
+  if (!st->active) return;
+  const MemberParams& P = v.mp[tl.member];
+  const int nx = P.nx, ny = P.ny, G = P.fx_gy, gw = P.fx_gwy, gain = P.fx_gainy, S = P.fx_sy, cw = P.fx_cw;
+  const int lane = threadIdx.x & 31;
+  const int seg = threadIdx.x / cw, c = threadIdx.x - seg * cw;
+  const bool cv = c < tl.count;
+  const int len = cv && seg < G ? min(S, ny - seg * S) : 0;  // 0: nothing to do, and no say in the panel's scale
+  const int64_t base = (int64_t)min(seg, G - 1) * S * nx + tl.start + (cv ? c : 0);
+  i64* y = reinterpret_cast<i64*>(smem) + threadIdx.x;
+  double* Cg = static_cast<double*>(v.C) + P.offset + base;
+  const short2* we = v.wexp + P.fx_wexp;
+  const short2* ws = we + min(seg, G - 1) * S;
+  // All of the panel's W in flight in up to 4 groups of rows of every segment (value u of segment g
+  // at u 256 + g cw, so a row piece of the panel is contiguous on both sides), in 16-byte pieces
+  // where the rows allow it; C on its way to L2 for the update.
+  {
+    i64* Y = reinterpret_cast<i64*>(smem);
+    const i64* Wm = static_cast<const i64*>(v.W) + P.offset + tl.start;
+    const bool wide = !((nx | tl.count) & 1);
+    const int E = wide ? 2 : 1, cols = wide ? tl.count >> 1 : tl.count, per = max(S >> 2, 8);
+    const int half = wide ? cw >> 1 : cw, rows_at_once = kColThreads / half;
+    const int tc = threadIdx.x % half, tr = threadIdx.x / half;
+    for (int g = 0; g < 4; ++g) {
+      // rows u0 .. u0 + per - 1 of every segment, numbered q = segment per + (u - u0)
+      const int u0 = g * per;
+      if (u0 < S && tc < cols)
+        for (int q = tr; q < G * per; q += rows_at_once) {
+          const int sq = q / per, u = u0 + q - sq * per, j = sq * S + u;
+          if (j < ny) {
+            const i64* src = Wm + (int64_t)j * nx + E * tc;
+            i64* dst = Y + u * kColThreads + sq * cw + E * tc;
+            if (wide)
+              copy16(dst, src);
+            else
+              copy8(dst, src);
+          }
+        }
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+    const char* Cm = static_cast<const char*>(v.C) + 8 * (P.offset + tl.start);
+    for (int j = threadIdx.x; j < ny; j += kColThreads) {
+      const char* p = Cm + (int64_t)j * nx * 8;
+      asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p));
+      asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p + 8 * (tl.count - 1)));
+      if (tl.count > 16) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p + 128));
+    }
+  }
+  load_tab(tab, v.segy[tl.member]);
+  int emax = -32768;
+  for (int j = lane; j < ny; j += 32) emax = max(emax, (int)we[j].y);
+  emax = __reduce_max_sync(kAll, emax);
+  const bool bad = emax == kBadRow;
+  i64* const ye = y + max(len - 1, 0) * kColThreads;
+  double* const Ce = Cg + (int64_t)max(len - 1, 0) * nx;
+  if (bad) {
+    Fp ar(P.fx_cy, P.p1y, P.p2y);
+    double a, b;
+    col_first(ar, y, len, S, ws, a, b, [](short2 e, auto f) {
+      f([e](i64 w) { return e.y == kBadRow ? w : double_bits(ldexp((double)w, e.x)); });
+    });
+    col_solve(ar, y, len, tab, xs, wtop, G, gw, cw, 0, a, b);
+    col_update(ar, ye, len, Ce, nx, P.kappa, cv, a, b, [](i64 t) { return __longlong_as_double(t); });
+  } else {
+    Fx ar(P.fx_cy, 0.0, 0.0);
+    FxLimb a, b;
+    const int up = 62 - gain - emax;
+    col_first(ar, y, len, S, ws, a, b, [up](short2 e, auto f) { with_shift(max(-62, min(62, up + (int)e.x)), f); });
+    const int sl = col_solve(ar, y, len, tab, xs, wtop, G, gw, cw, gain, a, b);
+    col_update(ar, ye, len, Ce, nx, P.kappa * ldexp(1.0, -up - sl), cv, a, b, [](i64 t) { return to_double(t); });
+  }
+  if (tl.index == 0 && threadIdx.x == 0) finalize_sample(v, tl.member, st, P);
+}
+
+template <int TH, int MINB>
+cudaError_t rows_limit() {
+  return cudaFuncSetAttribute(fx_rows_kernel<TH, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+}
+
+}  // namespace
+
+cudaError_t launch_fx_rows(const DevView& v, const LaunchShape& sh, cudaStream_t st) {
+  int base = sh.n_row_tiles;
+  const int* n = sh.fx_rt;
+  const size_t* sm = sh.fx_smem;
+  // Classes only set the CTA size (a row's arithmetic does not depend on it): where several of the
+  // short ones are present they share a launch, since a mix of small runs is bound by its launches
+  // (a burst of 24 requests of 64^2 to 256^2 takes 35.2 ms in separate launches, 24.2 ms in one).
+  if ((n[0] > 0) + (n[1] > 0) + (n[2] > 0) > 1) {
+    const int all = n[0] + n[1] + n[2];
+    fx_rows_kernel<256, 4><<<all, 256, max(sm[0], max(sm[1], sm[2])), st>>>(v, base);
+    base += all;
+    if (n[3] > 0) fx_rows_kernel<256, 2><<<n[3], 256, sm[3], st>>>(v, base);
+    return cudaGetLastError();
+  }
+  if (n[0] > 0) fx_rows_kernel<64, 14><<<n[0], 64, sm[0], st>>>(v, base);
+  base += n[0];
+  if (n[1] > 0) fx_rows_kernel<128, 7><<<n[1], 128, sm[1], st>>>(v, base);
+  base += n[1];
+  if (n[2] > 0) fx_rows_kernel<256, 4><<<n[2], 256, sm[2], st>>>(v, base);
+  base += n[2];
+  if (n[3] > 0) fx_rows_kernel<256, 2><<<n[3], 256, sm[3], st>>>(v, base);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fx_observe(const DevView& v, const LaunchShape& sh, cudaStream_t st) {
+  if (sh.fx_tiles > 0) fx_observe_kernel<<<sh.fx_tiles, 256, 0, st>>>(v, sh.n_row_tiles);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fx_cols(const DevView& v, const LaunchShape& sh, cudaStream_t st) {
+  const int base = sh.cst_n[0] + sh.cst_n[1] + sh.cst_n[2] + sh.cst_n[3];
+  if (sh.fx_ct > 0) fx_cols_kernel<<<sh.fx_ct, kColThreads, sh.fx_cols_smem, st>>>(v, base);
+  return cudaGetLastError();
+}
+
+size_t fx_rows_smem(int nr, int nx, int S) {
+  const int G = (nx + S - 1) / S, ns = (nx + 31) / 32;
+  return sizeof(ScanTab) + 8 * ((size_t)(nr + 4) * G * (S + 1) + (size_t)2 * ns * (2 * nr + 6) + 32);
+}
+
+size_t fx_cols_smem(int S) { return (size_t)S * kColThreads * 8; }
+
+cudaError_t set_fx_smem_limits() {
+  cudaError_t e;
+  if ((e = rows_limit<64, 14>()) != cudaSuccess || (e = rows_limit<128, 7>()) != cudaSuccess ||
+      (e = rows_limit<256, 4>()) != cudaSuccess || (e = rows_limit<256, 2>()) != cudaSuccess)
+    return e;
+  return cudaFuncSetAttribute(fx_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+}
+
+}  // namespace chk

@@ -30,6 +30,7 @@ struct ch_ensemble {
   std::vector<Tile> rest;         // members of the cluster-resident form (FP32), by class
   chk::LaunchShape shape{};
   ch_tuning tuning{};             // as requested (0 / -1 = default)
+  bool fx_fused = false;          // server: the fixed-point form beside the fused one
   int64_t total_points = 0, max_points = 0;
   int64_t c_points = 0;            // elements of C: the fields, then the lo blocks of compensated members
   int64_t total_bands = 0;
@@ -38,7 +39,8 @@ struct ch_ensemble {
   int64_t series_cap = 0;
   // device
   void* C = nullptr;
-  void* W = nullptr;
+  void* W = nullptr;               // then, CH_FP64: the row exponents of the fixed-point form
+  int64_t w_points = 0;            // elements of W before the row exponents
   MemberParams* dmp = nullptr;
   MemberState* dms = nullptr;
   chk::SegTable* dseg = nullptr;
@@ -84,6 +86,7 @@ struct ch_ensemble {
     v.segy = dsegy;
     v.colseg_tiles = dcst;
     v.res_tiles = dres;
+    v.wexp = reinterpret_cast<short2*>(static_cast<char*>(W) + elt * w_points);
     v.m = m;
     return v;
   }

@@ -9,7 +9,8 @@
 //   sweep_tiles Tile[]            one CTA of the row-sweep kernel per band (split form);
 //   col_tiles   Tile[]            one CTA of the column kernel per tile (a column panel);
 //   partials    double2[]         FP64 (sum F density, sum dF/dt density) per row band;
-//   series      double[m][cap][4] ring of (t, F, dF/dt, beta) samples per member.
+//   series      double[m][cap][4] ring of (t, F, dF/dt, beta) samples per member;
+//   wexp        short2[]          row exponents of W (fixed-point form, behind W).
 #pragma once
 
 #include <cstdint>
@@ -20,6 +21,16 @@ namespace chk {
 constexpr int64_t kUnbounded = INT64_MAX;
 
 constexpr int kBlockCols = 256;  // columns of a stencil block (long rows, FP64 split form)
+
+// 64-bit fixed-point constants of the CH_FP64 step (ch_fixed.cu): a value h 2^32 + l, l signed.
+struct FxLimb {
+  int h, l;
+};
+struct FxCoef {
+  FxLimb p1, p2;         // recurrence coefficients / 8, times 2^64
+};
+constexpr int kBadRow = 32767;    // row exponent of a row held in FP64
+constexpr int kFxRowClasses = 4;  // nx <= 64, 128, 512, 1024
 
 struct MemberParams {
   int64_t offset;        // first element of the member's field in C and W
@@ -55,6 +66,16 @@ struct MemberParams {
   // C at offset, lo in C at lo_offset); the update keeps the rounding error of hi in lo
   int comp;              // 1: compensated update (lo_offset valid)
   int64_t lo_offset;     // first element of the lo part in C, -1 if none
+  // fixed-point form (CH_FP64, default tuning, 16 <= nx, ny <= 1024): 1 + row class, or 0
+  int fx;
+  int fx_gx, fx_gwx, fx_gy, fx_gwy;  // segments per row / column, and the next power of two
+  int fx_sx, fx_sy, fx_cw;           // points per segment (powers of two), columns per panel
+  int fx_gainx, fx_gainy;            // log2 bound of the recurrences' gain
+  int fx_kmu, fx_su;                 // mu is held times 2^(kmu - E); su = 55 - kmu
+  int fx_er, fx_square;              // rho product: dy << er; square: hx = hy
+  FxCoef fx_cx, fx_cy;
+  FxLimb fx_bx, fx_by, fx_rho;       // bx, by times 2^(kmu + 5); rho times 2^(64 - er)
+  int64_t fx_wexp;                   // first row exponent in DevView::wexp
 };
 
 // Scan tables of the segment form of the row sweep (S points per lane, G lanes per row),
@@ -111,6 +132,7 @@ struct DevView {
   const SegTable* segy;  // [m] scan tables of the y recurrence (segment form of the column kernel)
   const Tile* colseg_tiles;  // CTAs of the segment-form column kernel
   const Tile* res_tiles;     // one per member of the cluster-resident form (FP32)
+  short2* wexp;              // fixed-point form: per row of W, the exponent of its unit and of its largest value
   int m;
 };
 
@@ -163,6 +185,11 @@ struct LaunchShape {
   size_t colseg_smem[4];
   // cluster-resident members (FP32): tiles per class (see res_class)
   int res_n[kResClasses];
+  // fixed-point members (FP64): row tiles by class after the n_row_tiles others, column tiles
+  // after the other segment-form ones
+  int fx_rt[kFxRowClasses], fx_ct;
+  size_t fx_smem[kFxRowClasses], fx_cols_smem;
+  int fx_tiles;          // row tiles of all classes
 };
 
 // Host-side fault injection (ch_fault.cu; armed by ch_set_fault or CH_FAULT).
@@ -200,6 +227,13 @@ int resident_classes(const LaunchShape& sh);
 // Dynamic shared memory of the cluster-resident kernel for rows of nx floats, nr per CTA.
 size_t resident_smem_bytes(int nx, int nr, int comp);
 cudaError_t set_kernel_smem_limits(int precision);
+// Fixed-point form (ch_fixed.cu): the row and column phases and the observables' partials.
+cudaError_t launch_fx_rows(const DevView& v, const LaunchShape& sh, cudaStream_t st);
+cudaError_t launch_fx_cols(const DevView& v, const LaunchShape& sh, cudaStream_t st);
+cudaError_t launch_fx_observe(const DevView& v, const LaunchShape& sh, cudaStream_t st);
+cudaError_t set_fx_smem_limits();
+size_t fx_rows_smem(int nr, int nx, int S);
+size_t fx_cols_smem(int S);
 // Resident CTAs per SM of the column kernel for a launch shape (0 on error).
 int cols_blocks_per_sm(int precision, int persist, int threads, size_t smem);
 // Resident CTAs per SM of the persistent segment row kernel (0 on error).

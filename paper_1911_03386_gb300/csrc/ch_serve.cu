@@ -38,6 +38,7 @@ namespace {
 using Clock = std::chrono::steady_clock;
 
 constexpr int64_t kAlignElems = 64;      // 256 B for FP32, 512 B for FP64
+constexpr int64_t kRowElems = 16;        // elements of W per row exponent (fixed-point runs: nx >= 16)
 constexpr int64_t kMaxChunk = 64;        // steps between retire/admit decisions
 constexpr int64_t kMaxQueue = 1 << 20;   // pending requests before CH_EBUSY
 constexpr int kDefaultEvery = 100;
@@ -150,6 +151,7 @@ int admit_slots(ch_server_s* S, const std::vector<int>& slots, const std::vector
     const Req& r = *reqs[i];
     if (int rc = chh::fill_params(r.d, h->precision, &h->hp[k])) return rc;
     h->hp[k].offset = r.offset;
+    h->hp[k].fx_wexp = r.offset / kRowElems;
     h->hp[k].lo_offset = r.comp ? r.lo_offset : -1;
     h->hp[k].every = r.every;
     h->hp[k].t1 = r.t1;
@@ -345,12 +347,14 @@ int ch_server_create(size_t hbm_budget_bytes, int precision, int max_members, ch
   h->hsegy.assign(max_members, chk::SegTable{});
   for (auto& p : h->hp) p.every = 1;
   h->present.assign(max_members, 0);
-  // Fused form for both precisions: segment-form rows and columns where a run's size
-  // allows (per run, so a result does not depend on the mix), streaming columns (FP64) or
-  // panels (FP32) for the others.  The split form's thread-per-line streams need many
-  // lines to fill the GPU, which a handful of served runs does not give.
+  // FP64: the fixed-point form; FP32, and FP64 runs it does not take: the fused form, with
+  // segment-form rows and columns where a run's size allows (per run, so a result does not
+  // depend on the mix), streaming columns (FP64) or panels (FP32) for the others.  The split
+  // form's thread-per-line streams need many lines to fill the GPU, which a handful of served
+  // runs does not give.
   h->tuning = chh::default_tuning();
   h->tuning.split = 0;
+  h->fx_fused = true;
   S->slot_req.assign(max_members, 0);
   S->arena.init(elems);
   cudaError_t e;
@@ -378,7 +382,10 @@ int ch_server_create(size_t hbm_budget_bytes, int precision, int max_members, ch
   if ((e = cudaStreamCreateWithFlags(&h->own, cudaStreamNonBlocking)) != cudaSuccess)
     return cleanup(CH_ECUDA, std::string("stream: ") + cudaGetErrorString(e));
   h->stream = h->own;
-  if ((e = chk::dev_malloc(&h->C, elt * elems)) != cudaSuccess || (e = chk::dev_malloc(&h->W, elt * elems)) != cudaSuccess ||
+  h->w_points = elems;
+  const size_t exp_bytes = precision == CH_FP64 ? sizeof(short2) * (elems / kRowElems) : 0;
+  if ((e = chk::dev_malloc(&h->C, elt * elems)) != cudaSuccess ||
+      (e = chk::dev_malloc(&h->W, elt * elems + exp_bytes)) != cudaSuccess ||
       (e = chk::dev_malloc((void**)&h->dmp, sizeof(MemberParams) * max_members)) != cudaSuccess ||
       (e = chk::dev_malloc((void**)&h->dms, sizeof(MemberState) * max_members)) != cudaSuccess ||
       (e = chk::dev_malloc((void**)&h->dseg, sizeof(chk::SegTable) * max_members)) != cudaSuccess ||
