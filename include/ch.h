@@ -158,7 +158,9 @@ int ch_set_field(ch_handle h, int member, const double* in);
 /*
  * Bulk transfer of every member's field: `in` / `out` hold the members in order, member
  * k as ny_k*nx_k doubles (total = sum of nx*ny).  With page-locked host buffers the FP64
- * copies are asynchronous DMA; FP32 fields are converted on the host.  Synchronises.
+ * copies are asynchronous DMA; FP32 fields are converted on the device, through a staging buffer
+ * of at most 32 MiB allocated on the first transfer (on the host if there is no room for it).
+ * Synchronises.
  */
 int ch_set_fields(ch_handle h, const double* in);
 int ch_get_fields(ch_handle h, double* out);

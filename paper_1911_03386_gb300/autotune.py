@@ -28,6 +28,7 @@ def candidates(precision):
         out.append(dict(split=0, resident=-1))
         out.append(dict(split=0, rows_band=8, threads=128, resident=-1))
     else:
+        out.append(dict())  # the fixed-point form where it applies
         out.append(dict(split=1, stream=1))
         for band in (8, 16):
             out.append(dict(split=1, stream=1, rows_band=band))

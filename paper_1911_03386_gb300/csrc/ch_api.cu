@@ -235,12 +235,22 @@ void seg_responses(double p1, double p2, int S, chk::SegTable* t) {
   }
 }
 
+// v as h 2^32 + l with l signed (|v| < 2^63 - 2^31).
+chk::FxLimb fx_limb(double v) {
+  const long long q = std::llround(v);
+  chk::FxLimb r;
+  r.l = (int32_t)(uint32_t)(unsigned long long)q;
+  r.h = (int32_t)((q - r.l) >> 32);
+  return r;
+}
+
 // Fixed-point form (ch_fixed.cu): the scan tables of a line of n points in segments of S points
 // whose last one may be shorter (len points): A[d] = M^(S 2^d), P = M^len, B[l] = M^(S l) (I -
 // M^n)^-1 for segment l, B[32 + pos] = M^(distance of segment pos from the line's end) (I -
-// M^n)^-1, pos counted from the end.
-void fx_tables(double p1, double p2, int S, int n, chk::SegTable* t) {
-  std::memset(t, 0, sizeof *t);
+// M^n)^-1, pos counted from the end.  False if an entry is too large for the scans' products (a
+// line short against the decay of M); t may be null.
+bool fx_tables(double p1, double p2, int S, int n, chk::SegTable* t, int* levels = nullptr) {
+  if (t) std::memset(t, 0, sizeof *t);
   const int G = (n + S - 1) / S, len = n - (G - 1) * S;
   const double M[4] = {p1, p2, 1.0, 0.0};
   double MS[4] = {1.0, 0.0, 0.0, 1.0}, ML[4] = {1.0, 0.0, 0.0, 1.0}, Mn[4] = {1.0, 0.0, 0.0, 1.0};
@@ -250,32 +260,39 @@ void fx_tables(double p1, double p2, int S, int n, chk::SegTable* t) {
   mat2_mul(ML, Mn, Mn);
   const double a = 1.0 - Mn[0], b = -Mn[1], c = -Mn[2], d = 1.0 - Mn[3], det = a * d - b * c;
   const double P[4] = {d / det, -b / det, -c / det, a / det};
+  bool ok = true;
+  auto put = [&](chk::FxLimb* to, const double* m) {
+    for (int i = 0; i < 4; ++i) {
+      if (!(std::fabs(m[i]) < 15.0))
+        ok = false;
+      else if (t)
+        to[i] = fx_limb(std::ldexp(m[i], 58));
+    }
+  };
+  chk::SegTable none;
+  chk::SegTable& T = t ? *t : none;
   double Ad[4] = {MS[0], MS[1], MS[2], MS[3]};
+  int lv = 0;
   for (int q = 0; q < 5 && (1 << q) < G; ++q) {
-    std::memcpy(t->A[q], Ad, sizeof Ad);
+    for (double x : Ad)
+      if (std::fabs(x) >= 0x1p-62) lv = q + 1;
+    put(T.Ax[q], Ad);
     mat2_mul(Ad, Ad, Ad);
   }
-  std::memcpy(t->P, ML, sizeof ML);
+  put(T.Px, ML);
   double F[4] = {P[0], P[1], P[2], P[3]}, R[4];
   for (int l = 0; l < G; ++l) {
-    std::memcpy(t->B[l], F, sizeof F);
+    put(T.Bx[l], F);
     mat2_mul(MS, F, F);
   }
-  std::memcpy(t->B[32], P, sizeof P);
+  put(T.Bx[32], P);
   mat2_mul(ML, P, R);
   for (int pos = 1; pos < G; ++pos) {
-    std::memcpy(t->B[32 + pos], R, sizeof R);
+    put(T.Bx[32 + pos], R);
     mat2_mul(MS, R, R);
   }
-}
-
-// v as h 2^32 + l with l signed (|v| < 2^63 - 2^31).
-chk::FxLimb fx_limb(double v) {
-  const long long q = std::llround(v);
-  chk::FxLimb r;
-  r.l = (int32_t)(uint32_t)(unsigned long long)q;
-  r.h = (int32_t)((q - r.l) >> 32);
-  return r;
+  if (levels) *levels = lv;
+  return ok;
 }
 
 // log2 bound of the gain of y_i = r_i + p1 y_{i-1} + p2 y_{i-2}: its impulse response's l1 norm.
@@ -300,6 +317,20 @@ int fx_band(int nx) { return nx <= 64 || nx > 256 ? 8 : 16; }
 int fx_seg_cols(int ny) { return ny <= 64 ? 8 : ny <= 128 ? 16 : 32; }
 int fx_panel(int ny) { return ny <= 256 ? 32 : ny <= 512 ? 16 : 8; }
 
+// Constants of mu in fixed point (any member whose stencil coefficients fit).
+void fx_mu_params(MemberParams* p) {
+  p->fx_square = p->hx == p->hy;
+  // |C| < 2^E: |mu| / 2^E <= 3 + 4 (bx + by) for E <= 1 and |R'| <= 4 (1 + rho) |mu|, which has
+  // to fit 62 bits (60 where R' takes a product with rho)
+  const double bound = 4.0 * (1.0 + p->rho) * (3.0 + 4.0 * (p->bx + p->by));
+  p->fx_mu = std::isfinite(bound) && bound < 1e9;
+  if (!p->fx_mu) return;
+  p->fx_kmu = std::min(55, (p->fx_square ? 62 : 60) - (int)std::ceil(std::log2(bound)));
+  p->fx_su = 55 - p->fx_kmu;
+  p->fx_bx = fx_limb(std::ldexp(p->bx, p->fx_kmu + 5));
+  p->fx_by = fx_limb(std::ldexp(p->by, p->fx_kmu + 5));
+}
+
 // The member's constants of the fixed-point form; false where it does not apply: lines of 16 to
 // 1024 points whose recurrences gain at most 2^9 (s up to about 1e5: above, 64 bits minus the
 // gain's headroom would hold less than FP64).
@@ -308,20 +339,12 @@ bool fx_params(MemberParams* p) {
   p->fx_gainx = fx_gain(p->p1x, p->p2x);
   p->fx_gainy = fx_gain(p->p1y, p->p2y);
   if (p->fx_gainx > 9 || p->fx_gainy > 9) return false;
-  p->fx_square = p->hx == p->hy;
-  // |C| < 2^E: |mu| / 2^E <= 3 + 4 (bx + by) for E <= 1 and |R'| <= 4 (1 + rho) |mu|, which has
-  // to fit 62 bits (60 where R' takes a product with rho)
-  const double bound = 4.0 * (1.0 + p->rho) * (3.0 + 4.0 * (p->bx + p->by));
-  p->fx_kmu = std::min(55, (p->fx_square ? 62 : 60) - (int)std::ceil(std::log2(bound)));
-  if (p->fx_kmu < 24) return false;
-  p->fx_su = 55 - p->fx_kmu;
+  if (!p->fx_mu) return false;
   int er = 0;
   if (std::frexp(p->rho, &er) > 1.0 - 1e-9) ++er;  // rho < 2^er, not by rounding alone
   p->fx_er = std::max(0, er + 1);
   if (p->fx_er > 40) return false;
   p->fx_rho = fx_limb(std::ldexp(p->rho, 64 - p->fx_er));
-  p->fx_bx = fx_limb(std::ldexp(p->bx, p->fx_kmu + 5));
-  p->fx_by = fx_limb(std::ldexp(p->by, p->fx_kmu + 5));
   p->fx_cx = chk::FxCoef{fx_limb(std::ldexp(p->p1x, 61)), fx_limb(std::ldexp(p->p2x, 61))};
   p->fx_cy = chk::FxCoef{fx_limb(std::ldexp(p->p1y, 61)), fx_limb(std::ldexp(p->p2y, 61))};
   auto pow2 = [](int g) {
@@ -337,7 +360,20 @@ bool fx_params(MemberParams* p) {
   p->fx_sy = sy;
   p->fx_cw = fx_panel(p->ny);
   p->fx_gwy = pow2(p->fx_gy);
-  return true;
+  return fx_tables(p->p1x, p->p2x, sx, p->nx, nullptr, &p->fx_lvx) &&
+         fx_tables(p->p1y, p->p2y, sy, p->ny, nullptr, &p->fx_lvy);
+}
+
+void fx_member_tables(const MemberParams& p, chk::SegTable* x, chk::SegTable* y) {
+  fx_tables(p.p1x, p.p2x, p.fx_sx, p.nx, x);
+  fx_tables(p.p1y, p.p2y, p.fx_sy, p.ny, y);
+}
+
+// Shared memory of the member's tiles into the launch shape (the largest of its class).
+void fx_shape(const MemberParams& p, chk::LaunchShape* sh) {
+  const int c = fx_class(p.nx);
+  sh->fx_smem[c] = std::max(sh->fx_smem[c], chk::fx_rows_smem(std::min(p.ny, fx_band(p.nx)), p.nx, p.fx_sx));
+  sh->fx_cols_smem = std::max(sh->fx_cols_smem, chk::fx_cols_smem(p.fx_sy));
 }
 
 bool is_pow2_upto32(int g) { return g >= 1 && g <= 32 && (g & (g - 1)) == 0; }
@@ -371,6 +407,8 @@ void free_device(ch_ensemble* h) {
   cudaFree(h->dpart);
   cudaFree(h->dseries);
   cudaFree(h->dobs);
+  cudaFree(h->stage);
+  h->stage = nullptr;
   h->C = h->W = nullptr;
   h->dmp = nullptr;
   h->dms = nullptr;
@@ -418,6 +456,8 @@ int fill_params(const ch_member_desc& d, int precision, MemberParams* p) {
   p->seed = d.seed;
   p->counter_base = d.counter_base;
   const double hx2 = p->hx * p->hx, hy2 = p->hy * p->hy;
+  p->ihx2 = 1.0 / hx2;
+  p->ihy2 = 1.0 / hy2;
   p->a = 1.0 - 2.0 * d.gamma / hx2 - 2.0 * d.gamma / hy2;
   p->bx = d.gamma / hx2;
   p->by = d.gamma / hy2;
@@ -444,10 +484,14 @@ int fill_params(const ch_member_desc& d, int precision, MemberParams* p) {
   p->fkappa = (float)p->kappa;
   p->comp = precision == CH_FP32 && std::max(sx, sy) > kCompS ? 1 : 0;
   p->lo_offset = -1;
+  fx_mu_params(p);
   p->every = 1;
   p->t1 = 0.0;
   return CH_OK;
 }
+
+// Reduction buffer of a CTA: two sums per warp, or the ten words of a sample's exact sums.
+size_t red_doubles(int threads) { return std::max<size_t>(10, (size_t)2 * (threads / 32)); }
 
 // C tile (nr+4 rows, dense pitch when rows move in 16-byte pieces) + mu tile (nr+2 rows,
 // pitch nx+1) + the FP64 reduction buffer; R' and the row sweep reuse the C tile's memory.
@@ -456,7 +500,7 @@ size_t rows_smem_bytes(int nr, int nx, size_t elt, int threads) {
   const size_t c_region = std::max((size_t)(nr + 4) * lc, (size_t)nr * (nx + 1));
   size_t b = (c_region + (size_t)(nr + 2) * (nx + 1)) * elt;
   b = (b + 15) & ~(size_t)15;
-  return b + (size_t)2 * (threads / 32) * sizeof(double);
+  return b + red_doubles(threads) * sizeof(double);
 }
 
 // Segment form: C tile buffer(s) (nr+4 rows, dense pitch; two when the kernel is
@@ -470,7 +514,7 @@ size_t seg_mtile(int nr, int nx, int S, size_t elt) {
 size_t seg_smem_bytes(size_t ccap, size_t mcap, int nbuf, size_t elt, int threads) {
   size_t b = ((size_t)nbuf * ccap + mcap + 28) * elt;
   b = (b + 15) & ~(size_t)15;
-  return b + (size_t)2 * (threads / 32) * sizeof(double);
+  return b + red_doubles(threads) * sizeof(double);
 }
 size_t rows_seg_smem_bytes(int nr, int nx, int S, size_t elt, int threads, int nbuf) {
   return seg_smem_bytes(seg_ctile(nr, nx), seg_mtile(nr, nx, S, elt), nbuf, elt, threads);
@@ -480,7 +524,7 @@ size_t rows_seg_smem_bytes(int nr, int nx, int S, size_t elt, int threads, int n
 size_t blk_smem_bytes(int nr, int nc, size_t elt, int threads) {
   size_t b = ((size_t)(nr + 4) * (nc + 4) + (size_t)(nr + 2) * (nc + 2)) * elt;
   b = (b + 15) & ~(size_t)15;
-  return b + (size_t)2 * (threads / 32) * sizeof(double);
+  return b + red_doubles(threads) * sizeof(double);
 }
 
 size_t sweep_smem_bytes(int nr, int nx, size_t elt) { return (size_t)nr * (nx + 1) * elt; }
@@ -628,12 +672,10 @@ int build_tiles(ch_ensemble* h, const ch_tuning& t) {
       p.kx32 = 0;
       p.rows_p = p.cols_p = 1;
       const int cr = fx_class(p.nx), br = std::min(p.ny, fx_band(p.nx)), cw = p.fx_cw;
-      fx_tables(p.p1x, p.p2x, fx_seg_rows(p.nx), p.nx, &h->hseg[k]);
-      fx_tables(p.p1y, p.p2y, fx_seg_cols(p.ny), p.ny, &h->hsegy[k]);
+      fx_member_tables(p, &h->hseg[k], &h->hsegy[k]);
+      fx_shape(p, &sh);
       int b = 0;
       for (int j0 = 0; j0 < p.ny; j0 += br, ++b) fxr[cr].push_back(Tile{k, j0, std::min(br, p.ny - j0), b, 0, 0});
-      sh.fx_smem[cr] = std::max(sh.fx_smem[cr], chk::fx_rows_smem(br, p.nx, fx_seg_rows(p.nx)));
-      sh.fx_cols_smem = std::max(sh.fx_cols_smem, chk::fx_cols_smem(p.fx_sy));
       p.nbands = b;
       p.partial_base = part;
       part += b;
@@ -1240,48 +1282,80 @@ int ch_series(ch_handle h, int member, double* out, int64_t cap, int64_t* n) {
 }  // extern "C"
 
 namespace chh {
-// Member k's field as FP64 values (FP32: hi, plus lo for compensated members).
-int read_member_field(ch_ensemble* h, int k, double* out) {
-  const MemberParams& p = h->hp[k];
-  const int64_t np = (int64_t)p.nx * p.ny;
-  if (h->precision == CH_FP64)
-    return copy_out(h, out, static_cast<double*>(h->C) + p.offset, sizeof(double) * np, "read field");
-  std::vector<float> tmp(np), lo;
-  if (int rc = copy_out(h, tmp.data(), static_cast<float*>(h->C) + p.offset, sizeof(float) * np, "read field")) return rc;
-  if (p.comp) {
-    lo.resize(np);
-    if (int rc = copy_out(h, lo.data(), static_cast<float*>(h->C) + p.lo_offset, sizeof(float) * np, "read field"))
-      return rc;
+// The fields of members k0 .. k1 - 1, one after another, between host memory (FP64 values) and the
+// device.  Members that follow each other in C move in one piece: FP64 as they are, FP32 through
+// the staging buffer, converted on the device (compensated members: hi + lo).  Synchronises.
+template <bool OUT>
+int move_fields(ch_ensemble* h, int k0, int k1, void* host, const char* what) {
+  double* at = static_cast<double*>(host);
+  if (h->precision == CH_FP32 && !h->stage) {
+    const int64_t n = std::min<int64_t>(ch_ensemble::kStage, std::max<int64_t>(h->w_points, h->total_points));
+    if (cudaMalloc(&h->stage, sizeof(double) * n) == cudaSuccess) {
+      h->stage_points = n;
+    } else {  // converted on the host below
+      cudaGetLastError();
+      h->stage = nullptr;
+    }
   }
-  for (int64_t i = 0; i < np; ++i) out[i] = p.comp ? (double)tmp[i] + (double)lo[i] : (double)tmp[i];
+  std::vector<float> hh, hl;
+  auto lo_delta = [&](int k) { return h->hp[k].comp ? h->hp[k].lo_offset - h->hp[k].offset : -1; };
+  for (int k = k0; k < k1;) {
+    // the run of members contiguous in C (and in their lo blocks)
+    const int64_t first = h->hp[k].offset, delta = lo_delta(k);
+    int64_t n = 0;
+    int q = k;
+    while (q < k1 && h->hp[q].offset == first + n && lo_delta(q) == delta)
+      n += (int64_t)h->hp[q].nx * h->hp[q].ny, ++q;
+    if (h->precision == CH_FP64) {
+      double* C = static_cast<double*>(h->C) + first;
+      CH_CUDA(cudaMemcpyAsync(OUT ? at : C, OUT ? C : at, sizeof(double) * n,
+                              OUT ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice, h->stream),
+              what);
+    } else if (!h->stage) {
+      float* hi = static_cast<float*>(h->C) + first;
+      float* lo = delta >= 0 ? hi + delta : nullptr;
+      hh.resize(n);
+      hl.resize(lo ? n : 0);
+      if (OUT) {
+        if (int rc = copy_out(h, hh.data(), hi, sizeof(float) * n, what)) return rc;
+        if (lo)
+          if (int rc = copy_out(h, hl.data(), lo, sizeof(float) * n, what)) return rc;
+        for (int64_t i = 0; i < n; ++i) at[i] = lo ? (double)hh[i] + (double)hl[i] : (double)hh[i];
+      } else {
+        for (int64_t i = 0; i < n; ++i) {
+          hh[i] = (float)at[i];
+          if (lo) hl[i] = (float)(at[i] - (double)hh[i]);
+        }
+        CH_CUDA(cudaMemcpyAsync(hi, hh.data(), sizeof(float) * n, cudaMemcpyHostToDevice, h->stream), what);
+        if (lo) CH_CUDA(cudaMemcpyAsync(lo, hl.data(), sizeof(float) * n, cudaMemcpyHostToDevice, h->stream), what);
+        CH_CUDA(cudaStreamSynchronize(h->stream), what);
+      }
+    } else {
+      float* hi = static_cast<float*>(h->C) + first;
+      for (int64_t d = 0; d < n; d += h->stage_points) {
+        const int64_t c = std::min(h->stage_points, n - d);
+        float* lo = delta >= 0 ? hi + delta + d : nullptr;
+        if (OUT) CH_CUDA(chk::launch_widen(hi + d, lo, h->stage, c, h->stream), what);
+        CH_CUDA(cudaMemcpyAsync(OUT ? at + d : h->stage, OUT ? h->stage : at + d, sizeof(double) * c,
+                                OUT ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice, h->stream),
+                what);
+        if (!OUT) CH_CUDA(chk::launch_narrow(h->stage, hi + d, lo, c, h->stream), what);
+      }
+    }
+    at += n;
+    k = q;
+  }
+  CH_CUDA(cudaStreamSynchronize(h->stream), what);
   return CH_OK;
 }
+
+// Member k's field as FP64 values (FP32: hi, plus lo for compensated members).
+int read_member_field(ch_ensemble* h, int k, double* out) { return move_fields<true>(h, k, k + 1, out, "read field"); }
 
 // Member k's field from FP64 values (FP32: rounded to hi, the remainder to lo for
 // compensated members).  Synchronises.
 int write_member_field(ch_ensemble* h, int k, const double* in) {
-  const MemberParams& p = h->hp[k];
-  const int64_t np = (int64_t)p.nx * p.ny;
-  if (h->precision == CH_FP64) {
-    CH_CUDA(cudaMemcpyAsync(static_cast<double*>(h->C) + p.offset, in, sizeof(double) * np, cudaMemcpyHostToDevice,
-                            h->stream),
-            "write field");
-  } else {
-    std::vector<float> hi(np), lo(p.comp ? np : 0);
-    for (int64_t i = 0; i < np; ++i) {
-      hi[i] = (float)in[i];
-      if (p.comp) lo[i] = (float)(in[i] - (double)hi[i]);
-    }
-    CH_CUDA(cudaMemcpyAsync(static_cast<float*>(h->C) + p.offset, hi.data(), sizeof(float) * np,
-                            cudaMemcpyHostToDevice, h->stream),
-            "write field");
-    if (p.comp)
-      CH_CUDA(cudaMemcpyAsync(static_cast<float*>(h->C) + p.lo_offset, lo.data(), sizeof(float) * np,
-                              cudaMemcpyHostToDevice, h->stream),
-              "write field");
-  }
-  CH_CUDA(cudaStreamSynchronize(h->stream), "write field");
-  return CH_OK;
+  return move_fields<false>(h, k, k + 1, const_cast<double*>(in), "write field");
 }
 }  // namespace chh
 
@@ -1306,41 +1380,13 @@ int ch_set_field(ch_handle h, int member, const double* in) {
 int ch_set_fields(ch_handle h, const double* in) {
   if (int rc = check_handle(h)) return rc;
   if (!in) return fail(CH_EINVAL, "in is NULL");
-  int64_t src = 0;
-  for (int k = 0; k < h->m; ++k) {
-    const MemberParams& p = h->hp[k];
-    const int64_t np = (int64_t)p.nx * p.ny;
-    if (h->precision == CH_FP64) {
-      CH_CUDA(cudaMemcpyAsync(static_cast<double*>(h->C) + p.offset, in + src, sizeof(double) * np,
-                              cudaMemcpyHostToDevice, h->stream),
-              "write fields");
-    } else if (int rc = write_member_field(h, k, in + src)) {
-      return rc;
-    }
-    src += np;
-  }
-  CH_CUDA(cudaStreamSynchronize(h->stream), "write fields");
-  return CH_OK;
+  return move_fields<false>(h, 0, h->m, const_cast<double*>(in), "write fields");
 }
 
 int ch_get_fields(ch_handle h, double* out) {
   if (int rc = check_handle(h)) return rc;
   if (!out) return fail(CH_EINVAL, "out is NULL");
-  int64_t dst = 0;
-  for (int k = 0; k < h->m; ++k) {
-    const MemberParams& p = h->hp[k];
-    const int64_t np = (int64_t)p.nx * p.ny;
-    if (h->precision == CH_FP64) {
-      CH_CUDA(cudaMemcpyAsync(out + dst, static_cast<double*>(h->C) + p.offset, sizeof(double) * np,
-                              cudaMemcpyDeviceToHost, h->stream),
-              "read fields");
-    } else if (int rc = read_member_field(h, k, out + dst)) {
-      return rc;
-    }
-    dst += np;
-  }
-  CH_CUDA(cudaStreamSynchronize(h->stream), "read fields");
-  return CH_OK;
+  return move_fields<true>(h, 0, h->m, out, "read fields");
 }
 
 int ch_launch_phase(ch_handle h, int phase) {

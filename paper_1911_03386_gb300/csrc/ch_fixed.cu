@@ -32,9 +32,9 @@
 //
 // Lines of n points are split into G = ceil(n / S) segments of S points (the last one may be
 // shorter), one lane (rows) or warp (columns) per segment.  Each recurrence is a pass from a
-// zero state over every segment, a Kogge-Stone scan of the end states in FP64 (its 24
-// operations per segment and pass overlap with the integer work) and a pass from the exact
-// periodic start state.
+// zero state over every segment, a Kogge-Stone scan of the end states (in the same arithmetic: in
+// FP64 it took the FP64 pipe a fifth of the kernels' time) and a pass from the exact periodic
+// start state.
 #include <cstdint>
 #include <type_traits>
 
@@ -46,48 +46,6 @@
 namespace chk {
 namespace {
 
-using i64 = long long;
-constexpr unsigned kAll = 0xffffffffu;
-
-// -------------------------------------------------------------------------------------
-// 64-bit fixed point
-// -------------------------------------------------------------------------------------
-// a b + c, 32 x 32 -> 64 bits, signed.
-__device__ __forceinline__ i64 madw(int a, int b, i64 c) {
-  i64 d;
-  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
-  return d;
-}
-
-// v = h 2^32 + l with l signed (so that every partial product is a signed one).
-__device__ __forceinline__ FxLimb limbs(i64 v) {
-  FxLimb q;
-  q.l = (int)v;
-  q.h = (int)(v >> 32) + (int)((unsigned)q.l >> 31);
-  return q;
-}
-
-// a b / 2^64 for |a| <= 2^62, |b| < 2^63, to about one unit: the product of the low limbs (at most
-// 1/4 unit) is left out, the middle products are rounded.
-__device__ __forceinline__ i64 mul_top(FxLimb a, FxLimb b) {
-  const i64 mid = madw(a.l, b.h, madw(a.h, b.l, 1ll << 31));
-  return madw(a.h, b.h, mid >> 32);
-}
-
-// v / 2^r (1 <= r <= 62), rounded to nearest, halves away from zero (a rounding that is not odd
-// in v would bias every point of a field the same way, and the mean is the mode that the solves
-// damp least).
-__device__ __forceinline__ i64 shift_down(i64 v, int r) { return (v + ((1ll << r) >> 1) + (v >> 63)) >> r; }
-
-// v 2^s for |s| <= 62: f(operation) with the operation for the sign of s (s the same in a warp).
-template <class F>
-__device__ __forceinline__ void with_shift(int s, const F& f) {
-  if (s >= 0)
-    f([s](i64 v) { return v << s; });
-  else
-    f([s](i64 v) { return shift_down(v, -s); });
-}
-
 // (double)v, truncated to 53 bits (it is the update of C, far below C itself), on the integer
 // pipes: the conversion instruction takes the FP64 pipe 16 SM clocks per warp, which the update
 // and the scans need.
@@ -98,17 +56,6 @@ __device__ __forceinline__ double to_double(i64 v) {
   const unsigned long long q = (m << lz) >> 11;  // 53 bits, the leading one adds 1 to the exponent
   const int hi = (int)(q >> 32) + ((1085 - lz) << 20) + ((int)(s >> 32) & 0x80000000);
   return m == 0 ? 0.0 : __hiloint2double(hi, (int)q);
-}
-
-// x 2^(59 - E) for |x| < 2^E, E = emax - 1022, from the fields of the binary64 value: the
-// 53-bit significand moved up by 6 bits, then down by the distance of its exponent from emax.
-__device__ __forceinline__ i64 to_fixed(i64 bits, int emax) {
-  const int hi = (int)(bits >> 32);
-  const int e = (hi >> 20) & 0x7ff;
-  const i64 m = ((i64)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)bits) << 6;
-  const i64 v = m >> min(emax - e, 63);
-  const i64 s = hi >> 31;
-  return (v ^ s) - s;
 }
 
 // Asynchronous global -> shared copy of one value.
@@ -131,22 +78,14 @@ struct Fx {
   unsigned top = 0;  // OR of the magnitudes' high words
   __device__ __forceinline__ Fx(const FxCoef& c, double, double) : p1(c.p1), p2(c.p2) {}
   static __device__ __forceinline__ State zero() { return FxLimb{0, 0}; }
-  // y = r + p1 a + p2 b to about one unit, for |a|, |b|, |y| < 2^62: the middle products are at most
-  // 2^61 (l p1.h), 2^60 (l p2.h) and 2^61 (h p.l), so their sum stays below 2^63.  They start at 2^63
-  // + 2^28, so that the sum is unsigned and its shift rounds; the high products take the 2^63 back.
-  __device__ __forceinline__ i64 step(State a, State b, i64 r) const {
-    i64 lo = madw(b.l, p2.h, (i64)((1ull << 63) + (1ull << 28)));
-    lo = madw(b.h, p2.l, lo);
-    i64 hi = madw(b.h, p2.h, -(1ll << 31));
-    lo = madw(a.l, p1.h, lo);
-    lo = madw(a.h, p1.l, lo);
-    hi = madw(a.h, p1.h, hi);
-    return r + (hi << 3) + (i64)((unsigned long long)lo >> 29);
+  __device__ __forceinline__ i64 step(State a, State b, i64 r) const { return fixed_dot<3>(p1, p2, a, b, r); }
+  // row[0] x0 + row[1] x1 + r of the scans
+  static __device__ __forceinline__ i64 dot(const FxLimb* row, i64 x0, i64 x1, i64 r) {
+    return fixed_dot<6>(row[0], row[1], limbs(x0), limbs(x1), r);
   }
   static constexpr bool kFixed = true;
   static __device__ __forceinline__ State state(i64 y) { return limbs(y); }
-  static __device__ __forceinline__ double value(State s) { return (double)(((i64)s.h << 32) + s.l); }
-  static __device__ __forceinline__ State start(double x) { return limbs(__double2ll_rn(x)); }
+  static __device__ __forceinline__ i64 value(State s) { return ((i64)s.h << 32) + s.l; }
   __device__ __forceinline__ void track(i64 y) {
     const int h = (int)(y >> 32);
     top |= (unsigned)(h ^ (h >> 31));
@@ -165,8 +104,14 @@ struct Fp {
   }
   static constexpr bool kFixed = false;
   static __device__ __forceinline__ State state(i64 y) { return __longlong_as_double(y); }
-  static __device__ __forceinline__ double value(State s) { return s; }
-  static __device__ __forceinline__ State start(double x) { return x; }
+  static __device__ __forceinline__ i64 value(State s) { return double_bits(s); }
+  static __device__ __forceinline__ double entry(FxLimb m) {  // times 2^58
+    return ldexp((double)(((i64)m.h << 32) + m.l), -58);
+  }
+  static __device__ __forceinline__ i64 dot(const FxLimb* row, i64 x0, i64 x1, i64 r) {
+    return double_bits(fma(entry(row[0]), __longlong_as_double(x0),
+                           fma(entry(row[1]), __longlong_as_double(x1), __longlong_as_double(r))));
+  }
   __device__ __forceinline__ void track(i64) {}
 };
 
@@ -229,45 +174,48 @@ __device__ __forceinline__ void pass_full(A& ar, i64* p, int es, int len, typena
 // segment), tab.B[l] = M^(S l) P, tab.B[32 + pos] = M^(distance from the line's end) P with P
 // = (I - M^n)^-1, all in shared memory.  (a, b): end state in, start state out.
 struct ScanTab {
-  double A[5][4], P[4], B[64][4];
+  FxLimb A[5][4], P[4], B[64][4];  // entries / 64, times 2^64, row-major
 };
+// The table into shared memory (16-byte asynchronous copies: Ax, Px, Bx lie like A, P, B).
 __device__ __forceinline__ void load_tab(ScanTab& t, const SegTable& g) {
-  const double* src = &g.A[0][0];
-  for (int k = threadIdx.x; k < 20; k += blockDim.x) (&t.A[0][0])[k] = src[k];
-  for (int k = threadIdx.x; k < 256; k += blockDim.x) (&t.B[0][0])[k] = (&g.B[0][0])[k];
-  if (threadIdx.x < 4) t.P[threadIdx.x] = g.P[threadIdx.x];
+  static_assert(sizeof(ScanTab) % 16 == 0, "whole pieces");
+  for (int k = threadIdx.x; k < (int)(sizeof(ScanTab) / 16); k += blockDim.x)
+    copy16(reinterpret_cast<char*>(&t) + 16 * k, reinterpret_cast<const char*>(&g.Ax[0][0]) + 16 * k);
 }
 
-template <bool REV>
-__device__ __forceinline__ void scan_states(const ScanTab& tab, double& a, double& b, int l, int G, int gw) {
+// Programmatic dependent launch: a step kernel lets its successor start (its CTAs take the SMs'
+// free slots, read their constant tables and wait) and waits itself until its predecessor has
+// finished and its writes are visible.  64^2 alone: 20.2 us per step without it, 16.5 with it.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;\n" ::: "memory");
+}
+
+template <bool REV, class A>
+__device__ __forceinline__ void scan_states(const ScanTab& tab, i64& a, i64& b, int l, int G, int gw, int levels, bool full) {
   const int pos = REV ? G - 1 - l : l;
-  const double e0 = a, e1 = b;
-#pragma unroll
-  for (int d = 0; d < 5; ++d) {
-    const int delta = 1 << d;
-    if (delta < gw) {
-      const double ya = REV ? __shfl_down_sync(kAll, a, delta, gw) : __shfl_up_sync(kAll, a, delta, gw);
-      const double yb = REV ? __shfl_down_sync(kAll, b, delta, gw) : __shfl_up_sync(kAll, b, delta, gw);
-      if (pos >= delta) {
-        const double na = fma(tab.A[d][0], ya, fma(tab.A[d][1], yb, a));
-        b = fma(tab.A[d][2], ya, fma(tab.A[d][3], yb, b));
-        a = na;
-      }
+  const i64 e0 = a, e1 = b;
+#pragma unroll 1
+  for (int d = 0, delta = 1; d < levels; ++d, delta *= 2) {
+    const i64 ya = REV ? __shfl_down_sync(kAll, a, delta, gw) : __shfl_up_sync(kAll, a, delta, gw);
+    const i64 yb = REV ? __shfl_down_sync(kAll, b, delta, gw) : __shfl_up_sync(kAll, b, delta, gw);
+    if (pos >= delta) {
+      a = A::dot(tab.A[d], ya, yb, a);
+      b = A::dot(tab.A[d] + 2, ya, yb, b);
     }
   }
-  double xa = REV ? __shfl_down_sync(kAll, a, 1, gw) : __shfl_up_sync(kAll, a, 1, gw);
-  double xb = REV ? __shfl_down_sync(kAll, b, 1, gw) : __shfl_up_sync(kAll, b, 1, gw);
-  if (pos == 0) xa = xb = 0.0;
-  double ta = a, tb = b;
-  if (!REV) {  // the last segment's own length
-    ta = fma(tab.P[0], xa, fma(tab.P[1], xb, e0));
-    tb = fma(tab.P[2], xa, fma(tab.P[3], xb, e1));
+  i64 xa = REV ? __shfl_down_sync(kAll, a, 1, gw) : __shfl_up_sync(kAll, a, 1, gw);
+  i64 xb = REV ? __shfl_down_sync(kAll, b, 1, gw) : __shfl_up_sync(kAll, b, 1, gw);
+  if (pos == 0) xa = xb = 0;
+  i64 ta = a, tb = b;
+  if (!REV && !full) {  // the last segment's own length
+    ta = A::dot(tab.P, xa, xb, e0);
+    tb = A::dot(tab.P + 2, xa, xb, e1);
   }
   ta = __shfl_sync(kAll, ta, REV ? 0 : G - 1, gw);
   tb = __shfl_sync(kAll, tb, REV ? 0 : G - 1, gw);
-  const double* B = tab.B[REV ? 32 + max(pos, 0) : min(l, 31)];
-  a = fma(B[0], ta, fma(B[1], tb, xa));
-  b = fma(B[2], ta, fma(B[3], tb, xb));
+  const FxLimb* B = tab.B[REV ? 32 + max(pos, 0) : min(l, 31)];
+  a = A::dot(B, ta, tb, xa);
+  b = A::dot(B + 2, ta, tb, xb);
 }
 
 __device__ __forceinline__ int bit_length_hi(unsigned top) { return 64 - __clz((int)top); }  // >= 32
@@ -399,21 +347,22 @@ __device__ __forceinline__ unsigned cta_or(unsigned top, unsigned* slots) {
 // Both recurrences of a row: segment seg (len points) of lane l of gw, G of them in use; top: OR of
 // the band's |R'|.  The band shares its shifts, so a band of W has one exponent.
 template <int NW, class A>
-__device__ __forceinline__ void row_solve(i64* seg, int len, int l, int G, int gw, A ar, const ScanTab& tab, int gain,
-                                          unsigned top, unsigned* slots, int& e_lsb, int& e_top) {
+__device__ __forceinline__ void row_solve(i64* seg, int len, int l, int G, int gw, int levels, bool full, A ar,
+                                          const ScanTab& tab, int gain, unsigned top, unsigned* slots, int& e_lsb,
+                                          int& e_top) {
   const int sl = 62 - gain - bit_length_hi(cta_or<NW>(top, slots));
   typename A::State a, b;
   pass_end(ar, seg, 1, len, sl, a, b);
-  double ea = A::value(a), eb = A::value(b);
-  scan_states<false>(tab, ea, eb, l, G, gw);
-  pass_full(ar, seg, 1, len, A::start(ea), A::start(eb));
+  i64 ea = A::value(a), eb = A::value(b);
+  scan_states<false, A>(tab, ea, eb, l, G, gw, levels, full);
+  pass_full(ar, seg, 1, len, A::state(ea), A::state(eb));
   const int sl2 = 62 - gain - bit_length_hi(cta_or<NW>(ar.top, slots + NW));
   i64* end = seg + max(len - 1, 0);
   pass_end(ar, end, -1, len, sl2, a, b);
   ea = A::value(a);
   eb = A::value(b);
-  scan_states<true>(tab, ea, eb, l, G, gw);
-  pass_full(ar, end, -1, len, A::start(ea), A::start(eb));
+  scan_states<true, A>(tab, ea, eb, l, G, gw, levels, full);
+  pass_full(ar, end, -1, len, A::state(ea), A::state(eb));
   e_lsb = -sl - sl2;
   e_top = e_lsb + bit_length_hi(cta_or<NW>(ar.top, slots + 2 * NW));
 }
@@ -425,6 +374,8 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
   const Tile tl = v.row_tiles[tile_base + blockIdx.x];
   const MemberParams& P = v.mp[tl.member];
   MemberState* st = v.ms + tl.member;
+  load_tab(*reinterpret_cast<ScanTab*>(smem), v.seg[tl.member]);
+  after_previous();
   bool sample;
   if (!stencil_prologue(tl, st, P, sample)) return;
   constexpr int NW = TH / 32;
@@ -462,7 +413,6 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
       }
     }
   }
-  load_tab(tab, v.seg[tl.member]);
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   unsigned top = 0;
   for (int s = warp; s < b.ns; s += NW) {  // this thread's own copies
@@ -498,17 +448,18 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
                        RhsFx<false>{P.fx_rho, P.fx_er});
     });
   if (sample)
-    band_partials_mu64<double>(v, tl, nx, nr, P, v.partials + P.partial_base + tl.index, red);
+    band_partials_field<double>(v, tl, nx, nr, P, v.partials + P.partial_base + tl.index, red);
 
   // rows: gw lanes per row (row_solve starts with a barrier: R' is complete)
   const int l = lane & (gw - 1), row = threadIdx.x / gw, r = min(row, nr - 1);
   const int len = l < G && row < nr ? min(S, nx - l * S) : 0;
   i64* seg = b.tile + r * b.pitch + l * (S + 1);
+  const bool full = nx % S == 0;
   int e_lsb, e_top;
   if (bad)
-    row_solve<NW>(seg, len, l, G, gw, Fp(P.fx_cx, P.p1x, P.p2x), tab, 0, 0u, wtop + NW, e_lsb, e_top);
+    row_solve<NW>(seg, len, l, G, gw, P.fx_lvx, full, Fp(P.fx_cx, P.p1x, P.p2x), tab, 0, 0u, wtop + NW, e_lsb, e_top);
   else
-    row_solve<NW>(seg, len, l, G, gw, Fx(P.fx_cx, 0.0, 0.0), tab, P.fx_gainx, top, wtop + NW, e_lsb, e_top);
+    row_solve<NW>(seg, len, l, G, gw, P.fx_lvx, full, Fx(P.fx_cx, 0.0, 0.0), tab, P.fx_gainx, top, wtop + NW, e_lsb, e_top);
   if (row < nr && l == 0) {
     const int eb = emax - 1022 - P.fx_kmu;
     v.wexp[P.fx_wexp + j0 + row] = bad ? make_short2(0, kBadRow) : make_short2((short)(e_lsb + eb), (short)(e_top + eb));
@@ -528,7 +479,7 @@ __global__ void __launch_bounds__(256) fx_observe_kernel(DevView v, int tile_bas
   __shared__ double red[16];
   const Tile tl = v.row_tiles[tile_base + blockIdx.x];
   const MemberParams& P = v.mp[tl.member];
-  band_partials_mu64<double>(v, tl, P.nx, tl.count, P, v.partials + P.partial_base + tl.index, red);
+  band_partials_field<double>(v, tl, P.nx, tl.count, P, v.partials + P.partial_base + tl.index, red);
 }
 
 // -------------------------------------------------------------------------------------
@@ -541,24 +492,26 @@ constexpr int kColThreads = 256;
 constexpr int kXsMax = 32 * 9;  // state exchange: G x (cw + 1), G cw <= 256
 
 template <class A>
-__device__ __forceinline__ int col_solve(A& ar, i64* y, int len, const ScanTab& tab, double2* xs, unsigned* wtop, int G,
-                                         int gw, int cw, int gain, typename A::State& a, typename A::State& b) {
+__device__ __forceinline__ int col_solve(A& ar, i64* y, int len, const ScanTab& tab, longlong2* xs, unsigned* wtop, int G,
+                                         int gw, int levels, bool full, int cw, int gain, typename A::State& a, typename A::State& b) {
   const int seg = threadIdx.x / cw, c = threadIdx.x - seg * cw;
   const int l = threadIdx.x & (gw - 1), sc = threadIdx.x / gw;  // scan: segment l of column sc
   auto exchange = [&](bool rev) {  // end state of this thread's segment in, its start state out
-    if (seg < G) xs[seg * (cw + 1) + c] = make_double2(A::value(a), A::value(b));
+    if (seg < G) xs[seg * (cw + 1) + c] = make_longlong2(A::value(a), A::value(b));
     __syncthreads();
-    double2* p = xs + min(l, G - 1) * (cw + 1) + min(sc, cw - 1);
-    double2 e = *p;
+    longlong2* p = xs + min(l, G - 1) * (cw + 1) + min(sc, cw - 1);
+    longlong2 e = *p;
+    i64 ea = e.x, eb = e.y;
     if (rev)
-      scan_states<true>(tab, e.x, e.y, l, G, gw);
+      scan_states<true, A>(tab, ea, eb, l, G, gw, levels, full);
     else
-      scan_states<false>(tab, e.x, e.y, l, G, gw);
+      scan_states<false, A>(tab, ea, eb, l, G, gw, levels, full);
+    e = make_longlong2(ea, eb);
     if (l < G && sc < cw) *p = e;
     __syncthreads();
     e = xs[min(seg, G - 1) * (cw + 1) + c];
-    a = A::start(e.x);
-    b = A::start(e.y);
+    a = A::state(e.x);
+    b = A::state(e.y);
   };
   exchange(false);
   pass_full(ar, y, kColThreads, len, a, b);
@@ -647,11 +600,13 @@ __device__ __forceinline__ void col_first(const A& ar, i64* y, int len, int S, c
 
 __global__ void __launch_bounds__(kColThreads, 3) fx_cols_kernel(DevView v, int tile_base) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ __align__(16) double2 xs[kXsMax];
-  __shared__ ScanTab tab;
+  __shared__ __align__(16) longlong2 xs[kXsMax];
+  __shared__ __align__(16) ScanTab tab;
   __shared__ unsigned wtop[kColThreads / 32];
   const Tile tl = v.colseg_tiles[tile_base + blockIdx.x];
   MemberState* st = v.ms + tl.member;
+  load_tab(tab, v.segy[tl.member]);
+  after_previous();
   if (!st->active) return;
   const MemberParams& P = v.mp[tl.member];
   const int nx = P.nx, ny = P.ny, G = P.fx_gy, gw = P.fx_gwy, gain = P.fx_gainy, S = P.fx_sy, cw = P.fx_cw;
@@ -699,7 +654,6 @@ __global__ void __launch_bounds__(kColThreads, 3) fx_cols_kernel(DevView v, int 
       if (tl.count > 16) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p + 128));
     }
   }
-  load_tab(tab, v.segy[tl.member]);
   int emax = -32768;
   for (int j = lane; j < ny; j += 32) emax = max(emax, (int)we[j].y);
   emax = __reduce_max_sync(kAll, emax);
@@ -712,14 +666,14 @@ __global__ void __launch_bounds__(kColThreads, 3) fx_cols_kernel(DevView v, int 
     col_first(ar, y, len, S, ws, a, b, [](short2 e, auto f) {
       f([e](i64 w) { return e.y == kBadRow ? w : double_bits(ldexp((double)w, e.x)); });
     });
-    col_solve(ar, y, len, tab, xs, wtop, G, gw, cw, 0, a, b);
+    col_solve(ar, y, len, tab, xs, wtop, G, gw, P.fx_lvy, ny % S == 0, cw, 0, a, b);
     col_update(ar, ye, len, Ce, nx, P.kappa, cv, a, b, [](i64 t) { return __longlong_as_double(t); });
   } else {
     Fx ar(P.fx_cy, 0.0, 0.0);
     FxLimb a, b;
     const int up = 62 - gain - emax;
     col_first(ar, y, len, S, ws, a, b, [up](short2 e, auto f) { with_shift(max(-62, min(62, up + (int)e.x)), f); });
-    const int sl = col_solve(ar, y, len, tab, xs, wtop, G, gw, cw, gain, a, b);
+    const int sl = col_solve(ar, y, len, tab, xs, wtop, G, gw, P.fx_lvy, ny % S == 0, cw, gain, a, b);
     col_update(ar, ye, len, Ce, nx, P.kappa * ldexp(1.0, -up - sl), cv, a, b, [](i64 t) { return to_double(t); });
   }
   if (tl.index == 0 && threadIdx.x == 0) finalize_sample(v, tl.member, st, P);
@@ -732,6 +686,26 @@ cudaError_t rows_limit() {
 
 }  // namespace
 
+// A step kernel; as a dependent launch up to one CTA per SM (above, CTAs that start in the slots their
+// predecessor happens to leave free are spread unevenly: 64 x 128^2 51 us per step with it, 39
+// without, 8 x 512^2 76 and 68).
+constexpr int kDependentCtas = 152;
+
+template <class K>
+void launch_dependent(K kernel, int grid, int block, size_t smem, cudaStream_t st, const DevView& v, int base) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3((unsigned)block, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = grid <= kDependentCtas ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, v, base);
+}
+
 cudaError_t launch_fx_rows(const DevView& v, const LaunchShape& sh, cudaStream_t st) {
   int base = sh.n_row_tiles;
   const int* n = sh.fx_rt;
@@ -741,19 +715,28 @@ cudaError_t launch_fx_rows(const DevView& v, const LaunchShape& sh, cudaStream_t
   // (a burst of 24 requests of 64^2 to 256^2 takes 35.2 ms in separate launches, 24.2 ms in one).
   if ((n[0] > 0) + (n[1] > 0) + (n[2] > 0) > 1) {
     const int all = n[0] + n[1] + n[2];
-    fx_rows_kernel<256, 4><<<all, 256, max(sm[0], max(sm[1], sm[2])), st>>>(v, base);
+    launch_dependent(fx_rows_kernel<256, 4>, all, 256, max(sm[0], max(sm[1], sm[2])), st, v, base);
     base += all;
-    if (n[3] > 0) fx_rows_kernel<256, 2><<<n[3], 256, sm[3], st>>>(v, base);
-    return cudaGetLastError();
+    if (n[3] > 0) launch_dependent(fx_rows_kernel<256, 2>, n[3], 256, sm[3], st, v, base);
+    return cudaPeekAtLastError();
   }
-  if (n[0] > 0) fx_rows_kernel<64, 14><<<n[0], 64, sm[0], st>>>(v, base);
+  // few tiles: larger CTAs (a sample's sums then take 8 warps instead of 2 or 4)
+  if (n[0] + n[1] > 0 && n[0] + n[1] <= kDependentCtas) {
+    launch_dependent(fx_rows_kernel<256, 4>, n[0] + n[1], 256, max(sm[0], sm[1]), st, v, base);
+    base += n[0] + n[1];
+    if (n[2] > 0) launch_dependent(fx_rows_kernel<256, 4>, n[2], 256, sm[2], st, v, base);
+    base += n[2];
+    if (n[3] > 0) launch_dependent(fx_rows_kernel<256, 2>, n[3], 256, sm[3], st, v, base);
+    return cudaPeekAtLastError();
+  }
+  if (n[0] > 0) launch_dependent(fx_rows_kernel<64, 14>, n[0], 64, sm[0], st, v, base);
   base += n[0];
-  if (n[1] > 0) fx_rows_kernel<128, 7><<<n[1], 128, sm[1], st>>>(v, base);
+  if (n[1] > 0) launch_dependent(fx_rows_kernel<128, 7>, n[1], 128, sm[1], st, v, base);
   base += n[1];
-  if (n[2] > 0) fx_rows_kernel<256, 4><<<n[2], 256, sm[2], st>>>(v, base);
+  if (n[2] > 0) launch_dependent(fx_rows_kernel<256, 4>, n[2], 256, sm[2], st, v, base);
   base += n[2];
-  if (n[3] > 0) fx_rows_kernel<256, 2><<<n[3], 256, sm[3], st>>>(v, base);
-  return cudaGetLastError();
+  if (n[3] > 0) launch_dependent(fx_rows_kernel<256, 2>, n[3], 256, sm[3], st, v, base);
+  return cudaPeekAtLastError();
 }
 
 cudaError_t launch_fx_observe(const DevView& v, const LaunchShape& sh, cudaStream_t st) {
@@ -763,8 +746,8 @@ cudaError_t launch_fx_observe(const DevView& v, const LaunchShape& sh, cudaStrea
 
 cudaError_t launch_fx_cols(const DevView& v, const LaunchShape& sh, cudaStream_t st) {
   const int base = sh.cst_n[0] + sh.cst_n[1] + sh.cst_n[2] + sh.cst_n[3];
-  if (sh.fx_ct > 0) fx_cols_kernel<<<sh.fx_ct, kColThreads, sh.fx_cols_smem, st>>>(v, base);
-  return cudaGetLastError();
+  if (sh.fx_ct > 0) launch_dependent(fx_cols_kernel, sh.fx_ct, kColThreads, sh.fx_cols_smem, st, v, base);
+  return cudaPeekAtLastError();
 }
 
 size_t fx_rows_smem(int nr, int nx, int S) {

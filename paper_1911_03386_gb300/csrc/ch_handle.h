@@ -68,6 +68,11 @@ struct ch_ensemble {
   cudaEvent_t fork = nullptr;
   int aux_used = 0;
 
+  // CH_FP32: staging of FP64 values for field transfers (allocated on first use, kept)
+  static constexpr int64_t kStage = (int64_t)1 << 22;
+  double* stage = nullptr;
+  int64_t stage_points = 0;
+
   bool has(int k) const { return present.empty() || present[k]; }
 
   chk::DevView view() const {
@@ -107,6 +112,13 @@ bool finite_pos(double x);
 int validate_desc(const ch_member_desc& d, int k);
 // FP64 constants of one member from its description (offset and tiling fields not set).
 int fill_params(const ch_member_desc& d, int precision, MemberParams* p);
+// Fixed-point constants of a member after fill_params (false where the form does not apply), its
+// scan tables, row class, rows per band and shared memory; none of them uses the heap.
+bool fx_params(MemberParams* p);
+void fx_member_tables(const MemberParams& p, chk::SegTable* x, chk::SegTable* y);
+int fx_class(int nx);
+int fx_band(int nx);
+void fx_shape(const MemberParams& p, chk::LaunchShape* sh);
 ch_tuning default_tuning();
 // Tiles and launch shapes for the present members under tuning t.
 int build_tiles(ch_ensemble* h, const ch_tuning& t);

@@ -46,6 +46,7 @@ struct MemberParams {
   int64_t partial_base;  // first partial slot
   int64_t series_cap;    // samples kept per member (ring)
   double L, hx, hy, gamma, dt;
+  double ihx2, ihy2;     // 1 / hx^2, 1 / hy^2
   // chemical potential  mu = C (C^2 - a) - bx (Ce + Cw) - by (Cn + Cs)
   double a, bx, by;
   // scaled explicit right-hand side  R' = (mu_e + mu_w) + rho (mu_n + mu_s) + w0 mu,
@@ -69,8 +70,10 @@ struct MemberParams {
   // fixed-point form (CH_FP64, default tuning, 16 <= nx, ny <= 1024): 1 + row class, or 0
   int fx;
   int fx_gx, fx_gwx, fx_gy, fx_gwy;  // segments per row / column, and the next power of two
+  int fx_lvx, fx_lvy;                // scan levels (above, the powers of M vanish in 62 bits)
   int fx_sx, fx_sy, fx_cw;           // points per segment (powers of two), columns per panel
   int fx_gainx, fx_gainy;            // log2 bound of the recurrences' gain
+  int fx_mu;                         // kmu, su, bx, by are set (any precision: the observables' sums)
   int fx_kmu, fx_su;                 // mu is held times 2^(kmu - E); su = 55 - kmu
   int fx_er, fx_square;              // rho product: dy << er; square: hx = hy
   FxCoef fx_cx, fx_cy;
@@ -96,6 +99,10 @@ struct SegTable {
   // backward recurrences from zero states; g = G0 of the forward homogeneous responses,
   // k = the backward homogeneous responses).
   float Hf[32][4];
+  // Fixed-point form (ch_fixed.cu; its own meaning of the entries, see fx_tables), entries / 64
+  // times 2^64.
+  alignas(16) FxLimb Ax[5][4];
+  FxLimb Px[4], Bx[64][4];
 };
 
 struct MemberState {
@@ -214,6 +221,10 @@ cudaError_t launch_init_fields(const DevView& v, int precision, int64_t max_poin
 // Initial fields of the members listed in `list` (device array of count member indices).
 cudaError_t launch_init_members(const DevView& v, int precision, const int* list, int count, int64_t max_points,
                                 cudaStream_t st);
+// CH_FP32 fields to / from FP64 values: out[i] = hi[i] (+ lo[i]), and hi[i] = in[i] rounded, lo[i] =
+// the rounded remainder (lo may be null).
+cudaError_t launch_widen(const float* hi, const float* lo, double* out, int64_t n, cudaStream_t st);
+cudaError_t launch_narrow(const double* in, float* hi, float* lo, int64_t n, cudaStream_t st);
 // One step = phases 0 (stencil or fused rows), 1 (row sweep, split form only), 2 (columns).
 cudaError_t launch_step(const DevView& v, int precision, const LaunchShape& sh, cudaStream_t st);
 cudaError_t launch_phase(const DevView& v, int precision, int phase, const LaunchShape& sh, cudaStream_t st);
@@ -227,7 +238,8 @@ int resident_classes(const LaunchShape& sh);
 // Dynamic shared memory of the cluster-resident kernel for rows of nx floats, nr per CTA.
 size_t resident_smem_bytes(int nx, int nr, int comp);
 cudaError_t set_kernel_smem_limits(int precision);
-// Fixed-point form (ch_fixed.cu): the row and column phases and the observables' partials.
+// Fixed-point form (ch_fixed.cu): the row and column phases (launch errors are read without
+// clearing them) and the observables' partials.
 cudaError_t launch_fx_rows(const DevView& v, const LaunchShape& sh, cudaStream_t st);
 cudaError_t launch_fx_cols(const DevView& v, const LaunchShape& sh, cudaStream_t st);
 cudaError_t launch_fx_observe(const DevView& v, const LaunchShape& sh, cudaStream_t st);

@@ -50,6 +50,7 @@
 // solution.  Two passes per recurrence whatever K, no shared-memory sweep traffic, no
 // barrier inside the sweep.
 #include <cstdint>
+
 #include <cuda_runtime.h>
 
 #include "ch_device.cuh"
@@ -89,6 +90,23 @@ __global__ void init_fields_kernel(DevView v, const int* list, int count) {
       if (sizeof(T) == 4 && P.comp)  // lo part: the exact remainder of the FP64 value
         static_cast<T*>(v.C)[P.lo_offset + p] = (T)__dsub_rn(c, (double)(T)c);
     }
+  }
+}
+
+// CH_FP32 fields to and from FP64 values, for transfers: the link moves the values as the caller
+// holds them (190 GB/s), and converting them on the device takes 0.05 ms per 16.8 M points where
+// one host thread took 12 ms (17 ms for hi + lo pairs).
+__global__ void widen_kernel(const float* __restrict__ hi, const float* __restrict__ lo, double* __restrict__ out,
+                             int64_t n) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    out[i] = lo ? (double)hi[i] + (double)lo[i] : (double)hi[i];
+}
+__global__ void narrow_kernel(const double* __restrict__ in, float* __restrict__ hi, float* __restrict__ lo, int64_t n) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const double x = in[i];
+    const float h = (float)x;
+    hi[i] = h;
+    if (lo) lo[i] = (float)(x - (double)h);
   }
 }
 
@@ -376,7 +394,7 @@ __device__ __forceinline__ void band_partials(const DevView& v, const Tile& tl, 
                                               double* red, int seg = 0) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   if (sizeof(T) == sizeof(float)) {
-    band_partials_mu64<T>(v, tl, nx, nr, P, slot, red);
+    band_partials_field<T>(v, tl, nx, nr, P, slot, red);
     return;
   }
   double sF = 0.0, sD = 0.0;
@@ -983,7 +1001,7 @@ __device__ __forceinline__ void seg_tile_setup(const DevView& v, const Tile& tl,
 // (28 T), then the FP64 reduction buffer.  PERSIST: a CTA walks the tiles blockIdx.x,
 // + gridDim.x, ... and copies the next tile's C band while it computes the current one.
 template <typename T, int S, bool PERSIST>
-__global__ void __launch_bounds__(256) rows_seg_kernel(DevView v, int base, int ntiles, int ccap, int mcap) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? (S == 16 ? 4 : 3) : 1) rows_seg_kernel(DevView v, int base, int ntiles, int ccap, int mcap) {
   extern __shared__ __align__(16) unsigned char smem[];
   T* Cbuf = reinterpret_cast<T*>(smem);
   T* Ms = Cbuf + (size_t)(PERSIST ? 2 : 1) * ccap;
@@ -1700,6 +1718,26 @@ __device__ __forceinline__ void res_partials(const float* Ct, const float* Lt, c
   block_sum2(sF, sD, red);
 }
 
+// The same in fixed point (FP64 where the values' range does not fit).
+template <int NX, int NR, bool COMP>
+__device__ __forceinline__ void res_sample(const float* Ct, const float* Lt, const MemberParams& P, double* red,
+                                           double& sF, double& sD) {
+  const bool ok = fixed_partials(
+      P, NX, NR, reinterpret_cast<unsigned long long*>(red),
+      [=](int r, int i) {
+        const int k = (r + 2) * NX + i;
+        return make_float2(Ct[k], COMP ? Lt[k] : 0.0f);
+      },
+      [=](float2 x, int emax) -> i64 { return COMP ? to_fixed(x.x, emax) + to_fixed(x.y, emax) : to_fixed(x.x, emax); },
+      [=](int r, int i) -> int {
+        const int e = (__float_as_int(Ct[(r + 2) * NX + i]) >> 23) & 0xff;
+        return e == 255 ? 2047 : e == 0 ? 0 : e + 896;
+      },
+      sF, sD);
+  if (!ok)
+    res_partials<NX, NR, COMP>(Ct, Lt, P, red, sF, sD);
+}
+
 // Shared memory of the resident kernel (bytes): C tile (and lo tile), mu/W tile, the
 // column end states (two step parities), the scan tables, the FP64 reduction buffer, the
 // per-rank partial slots (two step parities) and the member's state (rank 0).
@@ -1756,7 +1794,7 @@ __global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v
   if (OBS) {
     __syncthreads();
     double sF, sD;
-    res_partials<NX, NR, COMP>(Ct, Lt, P, red, sF, sD);
+    res_sample<NX, NR, COMP>(Ct, Lt, P, red, sF, sD);
     if (tid == 0) v.partials[P.partial_base + rank] = make_double2(sF, sD);
     return;
   }
@@ -1801,7 +1839,7 @@ __global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v
     const bool sample = ((n0 + s) % P.every) == 0;
     if (sample) {
       double sF, sD;
-      res_partials<NX, NR, COMP>(Ct, Lt, P, red, sF, sD);
+      res_sample<NX, NR, COMP>(Ct, Lt, P, red, sF, sD);
       if (tid == 0) st_peer2d(peer_addr(part + 8 * (s & 1) + rank, 0), make_double2(sF, sD));
     }
     // mu of own rows -1 .. 32 (tile row r + 1 of C) into mu/W tile row r
@@ -2301,7 +2339,10 @@ template <typename T>
 cudaError_t phase_impl(const DevView& v, int phase, const LaunchShape& sh, cudaStream_t st) {
   if (sizeof(T) == sizeof(double) && sh.fx_tiles > 0) {  // fixed-point members: rows and columns
     const cudaError_t e = phase == 0 ? launch_fx_rows(v, sh, st) : phase == 2 ? launch_fx_cols(v, sh, st) : cudaSuccess;
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return e;
+    }
   }
   if (sh.n_row_tiles == 0) return cudaSuccess;  // no member in the other forms
   switch (phase) {
@@ -2523,6 +2564,18 @@ cudaError_t launch_init_members(const DevView& v, int precision, const int* list
     init_fields_kernel<double><<<grid, 256, 0, st>>>(v, list, count);
   else
     init_fields_kernel<float><<<grid, 256, 0, st>>>(v, list, count);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_widen(const float* hi, const float* lo, double* out, int64_t n, cudaStream_t st) {
+  const int64_t blocks = (n + 255) / 256;
+  widen_kernel<<<(unsigned)(blocks < 2432 ? blocks : 2432), 256, 0, st>>>(hi, lo, out, n);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_narrow(const double* in, float* hi, float* lo, int64_t n, cudaStream_t st) {
+  const int64_t blocks = (n + 255) / 256;
+  narrow_kernel<<<(unsigned)(blocks < 2432 ? blocks : 2432), 256, 0, st>>>(in, hi, lo, n);
   return cudaGetLastError();
 }
 

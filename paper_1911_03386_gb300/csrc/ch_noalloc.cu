@@ -11,15 +11,26 @@
 // the row-solve result W, nx*ny doubles -- lives in the file-scope array below, which
 // exists on every GPU that loads the library from load until process exit.
 //
-// The kernels are the same two phases as a handle's step (13-point stencil + row sweep,
-// then column sweep + update; see ch_kernels.cu) without observables or step counters,
+// Grids that the fixed-point form takes (ch_fixed.cu: 16 to 1024 points per axis) run its two
+// kernels, whose tables a set-up kernel writes to a second static device array from its launch
+// parameters (so a captured call replays with them): 512^2 steps in 0.30 ms in the kernels below,
+// one thread per line on 32 SMs, and in 0.035 ms there.  The rule keeps to recurrences of a gain
+// up to 2^6 (gamma dt / h^4 up to about 1000): above, FP64's own rounding of a step exceeds 1e-13,
+// the agreement with a handle's FP64 kernels that this entry point has kept.
+//
+// Other grids run the kernels below: the same two phases as a handle's step (13-point stencil +
+// row sweep, then column sweep + update; see ch_kernels.cu) without observables or step counters,
 // with the member constants passed by value instead of from device tables.
+#include <algorithm>
+#include <climits>
 #include <cstdint>
 #include <cstdio>
 
 #include <cuda_runtime.h>
 
 #include "ch.h"
+#include "ch_handle.h"
+#include "ch_internal.h"
 
 namespace chk {
 void record_error(const char* msg);  // ch_api.cu
@@ -36,6 +47,77 @@ static __device__ __align__(256) double g_noalloc_scratch[kNoAllocMaxPoints];
 
 constexpr size_t kSmemMax = 227 * 1024;
 constexpr int kThreads = 256;
+
+// Device tables of the fixed-point kernels for the one field of a call.
+struct FixedTables {
+  chk::MemberParams mp;
+  chk::MemberState ms;
+  chk::SegTable seg, segy;
+  chk::Tile rows[128], cols[128];
+  double2 partials[128];
+  short2 wexp[1024];
+};
+static __device__ FixedTables g_noalloc_fixed;
+
+struct FixedSetup {  // by value in the set-up kernel's parameters
+  chk::MemberParams mp;
+  chk::SegTable seg, segy;
+};
+
+__global__ void noalloc_fixed_setup(FixedSetup s, FixedTables* t, int band) {
+  const int k = threadIdx.x;
+  if (k == 0) {
+    t->mp = s.mp;
+    t->seg = s.seg;
+    t->segy = s.segy;
+    chk::MemberState st = {};
+    st.step = 1;  // never a multiple of mp.every: no samples
+    st.remaining = chk::kUnbounded;
+    t->ms = st;
+  }
+  const int nx = s.mp.nx, ny = s.mp.ny, cw = s.mp.fx_cw;
+  if (k * band < ny) t->rows[k] = chk::Tile{0, k * band, min(band, ny - k * band), k, 0, 0};
+  if (k * cw < nx) t->cols[k] = chk::Tile{0, k * cw, min(cw, nx - k * cw), k, 0, 0};
+}
+
+// nsteps steps of the fixed-point kernels; false where the form does not apply.
+bool step_fixed(double* C, double* W, const ch_member_desc& d, int64_t nsteps, cudaStream_t st, int* rc) {
+  FixedSetup s;
+  if (chh::fill_params(d, CH_FP64, &s.mp) != CH_OK || !chh::fx_params(&s.mp)) return false;
+  if (s.mp.fx_gainx > 6 || s.mp.fx_gainy > 6) return false;
+  *rc = CH_ECUDA;
+  FixedTables* t = nullptr;
+  if (cudaGetSymbolAddress(reinterpret_cast<void**>(&t), g_noalloc_fixed) != cudaSuccess ||
+      chk::set_fx_smem_limits() != cudaSuccess)
+    return true;
+  s.mp.every = INT_MAX;
+  s.mp.fx = 1;
+  s.mp.fx_wexp = 0;
+  chh::fx_member_tables(s.mp, &s.seg, &s.segy);
+  const int band = std::min(d.ny, chh::fx_band(d.nx));
+  chk::LaunchShape sh{};
+  chh::fx_shape(s.mp, &sh);
+  s.mp.nbands = sh.fx_rt[chh::fx_class(d.nx)] = sh.fx_tiles = (d.ny + band - 1) / band;
+  sh.fx_ct = (d.nx + s.mp.fx_cw - 1) / s.mp.fx_cw;
+  chk::DevView v{};
+  v.C = C;
+  v.W = W;
+  v.mp = &t->mp;
+  v.ms = &t->ms;
+  v.row_tiles = t->rows;
+  v.colseg_tiles = t->cols;
+  v.partials = t->partials;
+  v.seg = &t->seg;
+  v.segy = &t->segy;
+  v.wexp = t->wexp;
+  v.m = 1;
+  if (nsteps > 0) noalloc_fixed_setup<<<1, 128, 0, st>>>(s, t, band);
+  if (cudaPeekAtLastError() != cudaSuccess) return true;
+  for (int64_t k = 0; k < nsteps; ++k)
+    if (chk::launch_fx_rows(v, sh, st) != cudaSuccess || chk::launch_fx_cols(v, sh, st) != cudaSuccess) return true;
+  *rc = CH_OK;
+  return true;
+}
 
 struct StepConsts {
   int nx, ny;
@@ -186,6 +268,19 @@ extern "C" int ch_step_field_noalloc(double* C, int nx, int ny, double L, double
     return na_fail(CH_EINVAL, "ch_step_field_noalloc: nx*ny exceeds the 1048576-point (1024x1024) scratch limit");
   if (!(L > 0.0) || !(gamma > 0.0) || !(dt > 0.0) || !(L < 1e300) || !(gamma < 1e300) || !(dt < 1e300))
     return na_fail(CH_EINVAL, "L, gamma and dt must be finite and > 0");
+  double* W = nullptr;
+  if (scratch_address(&W) != cudaSuccess) return na_fail(CH_ECUDA, "scratch set-up failed");
+  {
+    ch_member_desc d{};
+    d.nx = nx;
+    d.ny = ny;
+    d.L = L;
+    d.gamma = gamma;
+    d.dt = dt;
+    int rc = CH_OK;
+    if (step_fixed(C, W, d, nsteps, static_cast<cudaStream_t>(stream), &rc))
+      return rc == CH_OK ? CH_OK : na_fail(rc, "ch_step_field_noalloc: launch failed");
+  }
   StepConsts P;
   P.nx = nx;
   P.ny = ny;
@@ -211,8 +306,6 @@ extern "C" int ch_step_field_noalloc(double* C, int nx, int ny, double L, double
   if (rows_smem > kSmemMax || cols_smem > kSmemMax) return na_fail(CH_EINVAL, "grid line too long");
   P.br = br;
   P.bc = bc;
-  double* W = nullptr;
-  if (scratch_address(&W) != cudaSuccess) return na_fail(CH_ECUDA, "scratch set-up failed");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int row_blocks = (ny + br - 1) / br, col_blocks = (nx + bc - 1) / bc;
   // Launch errors are read with cudaPeekAtLastError, which leaves the error state as it

@@ -518,6 +518,7 @@ void ch_server_destroy(ch_server s) {
   cudaFree(h->dres);
   cudaFree(h->dpart);
   cudaFree(h->dobs);
+  cudaFree(h->stage);
   cudaFree(s->dlist);
   chh::free_aux(h);
   cudaStreamDestroy(h->own);
