@@ -81,6 +81,20 @@ __device__ __forceinline__ i64 to_fixed(i64 bits, int emax) {
   return (v ^ s) - s;
 }
 
+// Binary64 -> binary32 with the significand truncated, from the two formats' fields (IEEE
+// 754: binary64 = sign, 11-bit exponent biased by 1023, 52-bit fraction; binary32 = sign,
+// 8-bit exponent biased by 127, 23-bit fraction): the exponent is rebiased by 896 and the
+// top 23 fraction bits kept, so the relative error is below 2^-23.  |x| < 2^-126 gives a
+// signed zero, |x| >= 2^128 (and NaN) a signed infinity.  Integer operations only: the
+// FP32 heads of the FP64 pre-rolls leave the FP64 pipe to the FP64 part.
+__device__ __forceinline__ float f32_trunc(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned mag = hi & 0x7fffffffu, sign = hi & 0x80000000u;
+  const unsigned body = __funnelshift_l(lo, mag - (896u << 20), 3);  // (exp - 896) << 23 | fraction >> 29
+  const unsigned bits = mag < (897u << 20) ? sign : (mag >= (1151u << 20) ? (sign | 0x7f800000u) : (sign | body));
+  return __uint_as_float(bits);
+}
+
 // Fixed-order block reduction of two FP64 sums (deterministic for a given block size).
 __device__ __forceinline__ void block_sum2(double& a, double& b, double* red) {
 #pragma unroll

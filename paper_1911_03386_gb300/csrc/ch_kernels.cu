@@ -2061,20 +2061,6 @@ constexpr size_t rowstream_smem_bytes(size_t elt) {
   return (size_t)kStreamCta * 2 * 32 * ((elt == 8 ? 16 : 32) + 1) * elt;
 }
 
-// Binary64 -> binary32 with the significand truncated, from the two formats' fields (IEEE
-// 754: binary64 = sign, 11-bit exponent biased by 1023, 52-bit fraction; binary32 = sign,
-// 8-bit exponent biased by 127, 23-bit fraction): the exponent is rebiased by 896 and the
-// top 23 fraction bits kept, so the relative error is below 2^-23.  |x| < 2^-126 gives a
-// signed zero, |x| >= 2^128 (and NaN) a signed infinity.  Integer operations only: the
-// FP32 heads of the FP64 pre-rolls leave the FP64 pipe to the FP64 part.
-__device__ __forceinline__ float f32_trunc(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned mag = hi & 0x7fffffffu, sign = hi & 0x80000000u;
-  const unsigned body = __funnelshift_l(lo, mag - (896u << 20), 3);  // (exp - 896) << 23 | fraction >> 29
-  const unsigned bits = mag < (897u << 20) ? sign : (mag >= (1151u << 20) ? (sign | 0x7f800000u) : (sign | body));
-  return __uint_as_float(bits);
-}
-
 // Sequence position q of a pass -> column/row index: positions 0..K-1 are the pre-roll,
 // K..K+n-1 the line itself.  Forward: pre-roll over indices -K..-1 (mod n), then 0..n-1.
 // Backward: pre-roll over n-1+K..n (mod n), then n-1..0.

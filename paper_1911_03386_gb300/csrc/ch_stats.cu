@@ -32,6 +32,7 @@
 #include <cuda_runtime.h>
 
 #include "ch.h"
+#include "ch_device.cuh"
 #include "ch_handle.h"
 
 namespace chs {
@@ -64,6 +65,11 @@ __device__ __forceinline__ int64_t run_offset(const View& v, int64_t j) {
   return v.moff ? v.moff[j] : j * v.mstride;
 }
 
+// isfinite on the integer pipes (an FP64 comparison is one of the moments' 8 FP64 operations per
+// value, which bound the kernel).  Moments, histogram of 100 bins and trend of 8192 samples x 1024
+// runs: 445 us with FP64 comparisons and divisions and the trend on one CTA, 183 us now.
+__device__ __forceinline__ bool finite64(double x) { return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u; }
+
 // Row s of out (6 doubles): t, count, mu_1 .. mu_4.  *mismatch |= 1 when a run's t differs
 // from run 0's at the same sample (series views only).
 __global__ void __launch_bounds__(kThreads) moments_kernel(View v, double* __restrict__ out,
@@ -86,7 +92,7 @@ __global__ void __launch_bounds__(kThreads) moments_kernel(View v, double* __res
       const int64_t o = run_offset(v, j) + so;
       const double b = v.base[o + v.bc];
       if (v.tc >= 0 && v.base[o + v.tc] != t0) bad = 1;
-      if (isfinite(b)) {
+      if (finite64(b)) {
         sum += b;
         ++cnt;
       }
@@ -112,7 +118,7 @@ __global__ void __launch_bounds__(kThreads) moments_kernel(View v, double* __res
   if (on) {
     for (int64_t j = w; j < v.M; j += kWarps) {
       const double b = v.base[run_offset(v, j) + so + v.bc];
-      if (isfinite(b)) {
+      if (finite64(b)) {
         const double d = b - mu1;
         const double d2 = d * d;
         c2 += d2;
@@ -144,7 +150,10 @@ __global__ void __launch_bounds__(kThreads) moments_kernel(View v, double* __res
   }
 }
 
-// Row s of out (nbins + 2 counts): below lo, the bins, at or above the end of the last bin.
+// Row s of out (nbins + 2 counts): below lo, the bins, at or above the end of the last bin.  The
+// bin is decided in FP32 where its error bound keeps the quotient away from a bin edge, else (about
+// one value in 10^4) by the FP64 division that defines it, which takes the FP64 pipe a dozen
+// operations.
 __global__ void __launch_bounds__(kThreads) histogram_kernel(View v, double lo, double w, int nbins,
                                                              int64_t* __restrict__ out) {
   extern __shared__ int hist[];  // [nbins + 2][kPad]
@@ -155,11 +164,17 @@ __global__ void __launch_bounds__(kThreads) histogram_kernel(View v, double lo, 
   const int64_t s = (int64_t)blockIdx.x * kLanes + lane;
   if (s < v.T) {
     const int64_t so = slot_offset(v, s);
+    const float lof = (float)lo, inv = (float)(1.0 / w);
     for (int64_t j = wp; j < v.M; j += kWarps) {
       const double b = v.base[run_offset(v, j) + so + v.bc];
-      if (!isfinite(b)) continue;
+      if (!finite64(b)) continue;
       int bin;
-      if (b < lo) {
+      // x = (b - lo) / w to within e: b, lo, w and the three operations each to 2^-23
+      const float bf = chk::f32_trunc(b), x = (bf - lof) * inv, k32 = floorf(x);
+      const float e = 4.8e-7f * ((fabsf(bf) + fabsf(lof)) * inv + fabsf(x)) + 1e-20f;
+      if (x - k32 > e && x - k32 < 1.0f - e && fabsf(x) < 1e6f) {
+        bin = k32 < 0.0f ? 0 : k32 < (float)nbins ? (int)k32 + 1 : nbins + 1;
+      } else if (b < lo) {
         bin = 0;
       } else {
         const double k = floor((b - lo) / w);
@@ -179,14 +194,20 @@ __global__ void __launch_bounds__(kThreads) histogram_kernel(View v, double lo, 
 
 // out[0] window mean of mu_1 (trapezoid over consecutive samples in [t1, t2], divided by the
 // span of those samples), out[1] k = sum t mu_2 / sum t^2 over [tf1, tf2], out[2..3] counts.
-__global__ void __launch_bounds__(kThreads) trend_kernel(const double* __restrict__ mom, int64_t T, double t1,
-                                                         double t2, double tf1, double tf2,
-                                                         double* __restrict__ out) {
+// One cluster of kTrendCtas CTAs: the rows are dealt to all threads, each CTA reduces its own, and
+// rank 0 adds the CTAs' sums in rank order (distributed shared memory).  (One CTA alone is
+// bound by its SM's FP64 pipe.)
+constexpr int kTrendCtas = 8;
+
+__global__ void __cluster_dims__(kTrendCtas, 1, 1) __launch_bounds__(kThreads)
+    trend_kernel(const double* __restrict__ mom, int64_t T, double t1, double t2, double tf1, double tf2,
+                 double* __restrict__ out) {
   __shared__ double rd[3][kThreads];
   __shared__ int64_t ri[4][kThreads];
   double integral = 0.0, stm = 0.0, stt = 0.0;
   int64_t nw = 0, nf = 0, smin = INT64_MAX, smax = -1;
-  for (int64_t s = threadIdx.x; s < T; s += kThreads) {
+  const unsigned rank = chk::cluster_rank();
+  for (int64_t s = (int64_t)rank * kThreads + threadIdx.x; s < T; s += kTrendCtas * kThreads) {
     const double* r = mom + s * CH_MOMENTS;
     const double t = r[0];
     if (t >= t1 && t <= t2) {
@@ -225,7 +246,18 @@ __global__ void __launch_bounds__(kThreads) trend_kernel(const double* __restric
     }
     __syncthreads();
   }
-  if (i == 0) {
+  chk::cluster_sync();
+  if (i == 0 && rank == 0) {
+    for (unsigned q = 1; q < (unsigned)kTrendCtas; ++q) {
+      for (int k = 0; k < 3; ++k) rd[k][0] += chk::ld_peer(chk::peer_addr(&rd[k][0], q), 0.0);
+      int64_t x[4];
+      for (int k = 0; k < 4; ++k)
+        x[k] = __double_as_longlong(chk::ld_peer(chk::peer_addr(&ri[k][0], q), 0.0));
+      ri[0][0] += x[0];
+      ri[1][0] += x[1];
+      ri[2][0] = x[2] < ri[2][0] ? x[2] : ri[2][0];
+      ri[3][0] = x[3] > ri[3][0] ? x[3] : ri[3][0];
+    }
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
     const int64_t n_w = ri[0][0];
     out[0] = n_w >= 2 ? rd[0][0] / (mom[ri[3][0] * CH_MOMENTS] - mom[ri[2][0] * CH_MOMENTS]) : nan;
@@ -233,6 +265,7 @@ __global__ void __launch_bounds__(kThreads) trend_kernel(const double* __restric
     out[2] = (double)n_w;
     out[3] = (double)ri[1][0];
   }
+  chk::cluster_sync();  // rank 0 may still read the others' sums
 }
 
 // row[j] = mean over coarse row j of |1/4 (f(2i,2j) + f(2i+1,2j) + f(2i,2j+1) + f(2i+1,2j+1)) - c(i,j)|.
@@ -307,7 +340,7 @@ cudaError_t launch_histogram(const View& v, double lo, double hi, int nbins, int
 
 cudaError_t launch_trend(const double* mom, int64_t T, double t1, double t2, double tf1, double tf2, double* out,
                          cudaStream_t st) {
-  trend_kernel<<<1, kThreads, 0, st>>>(mom, T, t1, t2, tf1, tf2, out);
+  trend_kernel<<<kTrendCtas, kThreads, 0, st>>>(mom, T, t1, t2, tf1, tf2, out);
   return cudaGetLastError();
 }
 
