@@ -708,6 +708,7 @@ int build_tiles(ch_ensemble* h, const ch_tuning& t) {
       seg_tables(p.p1x, p.p2x, rc, p.seg_g, &h->hseg[k]);
       sh.seg_ccap[ri] = std::max(sh.seg_ccap[ri], (int)seg_ctile(br, p.nx));
       sh.seg_mcap[ri] = std::max(sh.seg_mcap[ri], (int)seg_mtile(br, p.nx, rc, h->elt));
+      sh.walk_smem[ri] = std::max(sh.walk_smem[ri], chk::walk_smem_bytes(br, p.nx, rc));
     }
     // FP32 heads of the FP64 streaming row sweeps' pre-rolls.  (The column stream with heads
     // measured slower: 0.299 against 0.259 ms at 256 x 256^2, so its pre-rolls stay FP64.)

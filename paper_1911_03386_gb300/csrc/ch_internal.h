@@ -185,6 +185,7 @@ struct LaunchShape {
   int seg_grid[2];       // CTAs of the persistent segment row kernel
   int seg_ccap[2], seg_mcap[2];  // elements of one C tile buffer / of the mu tile (max over the class)
   size_t seg_smem[2];    // dynamic shared memory of the segment-form row kernel
+  size_t walk_smem[2];   // the same of its one-tile form (FP32)
   // Column tiles of the segment form: cst_n[0] with S = 16, cst_n[1] with S = 32 (one CTA
   // per tile), then cst_n[2], cst_n[3] with S = 16, 32 over CTA pairs (tall columns).
   int cst_n[4];
@@ -235,6 +236,8 @@ cudaError_t launch_resident(const DevView& v, int precision, const LaunchShape& 
                             const cudaStream_t* streams, int nstreams);
 // Number of resident classes present in a launch shape.
 int resident_classes(const LaunchShape& sh);
+// Dynamic shared memory of the one-tile segment-form row kernel (FP32).
+size_t walk_smem_bytes(int nr, int nx, int S);
 // Dynamic shared memory of the cluster-resident kernel for rows of nx floats, nr per CTA.
 size_t resident_smem_bytes(int nx, int nr, int comp);
 cudaError_t set_kernel_smem_limits(int precision);

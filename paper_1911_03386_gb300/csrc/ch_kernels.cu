@@ -647,6 +647,74 @@ __device__ __forceinline__ void seg_sweep(T (&y)[R][S], T p1, T p2, int l, int G
   }
 }
 
+// The rows of a band from its mu tile (mu row r, r = 0 .. nr + 1, in tile row row_of(r), pitch lmp):
+// R' in registers, both recurrences, W stored.
+template <typename T, int S, class RowOf>
+__device__ __forceinline__ void seg_rows(const DevView& v, const Tile& tl, const MemberParams& P, const T* Ms, int lmp,
+                                         const T* Ks, RowOf row_of) {
+  const int nx = P.nx, j0 = tl.start, nr = tl.count;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  // rows: G lanes per row, groups of one warp take rows round-robin
+  const SegTable& tab = v.seg[tl.member];
+  const int G = P.seg_g;
+  const int lg = __ffs(G) - 1;
+  const int gpw = 32 / G, ngroups = nwarps * gpw;
+  const int l = lane & (G - 1), grp = warp * gpw + (lane >> lg);
+  T Bf[4], Bb[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    Bf[k] = pick<T>(tab.B[l][k], tab.Bf[l][k]);
+    Bb[k] = pick<T>(tab.B[G - 1 - l][k], tab.Bf[G - 1 - l][k]);
+  }
+  const T p1 = pick<T>(P.p1x, P.fp1x), p2 = pick<T>(P.p2x, P.fp2x), rho = pick<T>(P.rho, P.frho),
+          w0 = pick<T>(P.w0, P.fw0);
+  T* __restrict__ W = static_cast<T*>(v.W) + P.offset;
+  // FP32 with 16-point segments: two rows per group, their chains interleaved
+  constexpr int R = 1;  // rows per group (2 measured slower: fewer CTAs per SM)
+  const int rounds = (nr + R * ngroups - 1) / (R * ngroups);
+  for (int k = 0; k < rounds; ++k) {
+    T m[R][S];
+#pragma unroll
+    for (int t = 0; t < R; ++t) {
+      const int r = (k * ngroups + grp) * R + t;
+      const int rc = r < nr ? r : nr - 1, lo = l * (S + seg_pad<T>());
+      const T* mrow = Ms + (size_t)row_of(rc + 1) * lmp + lo;
+      const T* urow = Ms + (size_t)row_of(rc) * lmp + lo;
+      const T* drow = Ms + (size_t)row_of(rc + 2) * lmp + lo;
+#pragma unroll
+      for (int c = 0; c < S / 4; ++c) ld4(mrow + 4 * c, &m[t][4 * c]);
+      const T left = __shfl_sync(kFull, m[t][S - 1], (l + G - 1) & (G - 1), G);
+      const T right = __shfl_sync(kFull, m[t][0], (l + 1) & (G - 1), G);
+      T prev = left;
+#pragma unroll
+      for (int c = 0; c < S / 4; ++c) {
+        T up[4], dn[4];
+        ld4(urow + 4 * c, up);
+        ld4(drow + 4 * c, dn);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int u = 4 * c + q;
+          const T cur = m[t][u];
+          const T e = u + 1 < S ? m[t][u + 1] : right;
+          m[t][u] = fma(w0, cur, fma(rho, dn[q] + up[q], e + prev));
+          prev = cur;
+        }
+      }
+    }
+    seg_sweep<T, S, R, false>(m, p1, p2, l, G, lg, Ks, Bf);
+    seg_sweep<T, S, R, true>(m, p1, p2, l, G, lg, Ks, Bb);
+#pragma unroll
+    for (int t = 0; t < R; ++t) {
+      const int r = (k * ngroups + grp) * R + t;
+      if (r < nr) {
+        T* dst = W + (int64_t)(j0 + r) * nx + l * S;
+#pragma unroll
+        for (int c = 0; c < S / 4; ++c) st4(dst + 4 * c, &m[t][4 * c]);
+      }
+    }
+  }
+}
+
 // Segment-form row work of one band (tile tl of member P) whose C rows j0-2 .. j0+nr+1
 // are in Cs (dense pitch nx): mu tile Ms (nr+2 rows, pitch nx + 16 bytes per segment), the
 // sample partials, then R' in registers, the forward and backward recurrences and W
@@ -656,7 +724,7 @@ __device__ __forceinline__ void seg_sweep(T (&y)[R][S], T p1, T p2, int l, int G
 template <typename T, int S>
 __device__ __forceinline__ void seg_tile(const DevView& v, const Tile& tl, const MemberParams& P, const T* Cs, T* Ms,
                                          const T* Ks, double* red, bool sample) {
-  const int nx = P.nx, j0 = tl.start, nr = tl.count;
+  const int nx = P.nx, nr = tl.count;
   const int lmp = nx + seg_pad<T>() * (nx / S);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
 
@@ -703,62 +771,7 @@ __device__ __forceinline__ void seg_tile(const DevView& v, const Tile& tl, const
     __syncthreads();
   }
 
-  // rows: G lanes per row, groups of one warp take rows round-robin
-  const SegTable& tab = v.seg[tl.member];
-  const int G = P.seg_g;
-  const int lg = __ffs(G) - 1;
-  const int gpw = 32 / G, ngroups = nwarps * gpw;
-  const int l = lane & (G - 1), grp = warp * gpw + (lane >> lg);
-  T Bf[4], Bb[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    Bf[k] = pick<T>(tab.B[l][k], tab.Bf[l][k]);
-    Bb[k] = pick<T>(tab.B[G - 1 - l][k], tab.Bf[G - 1 - l][k]);
-  }
-  const T p1 = pick<T>(P.p1x, P.fp1x), p2 = pick<T>(P.p2x, P.fp2x), rho = pick<T>(P.rho, P.frho),
-          w0 = pick<T>(P.w0, P.fw0);
-  T* __restrict__ W = static_cast<T*>(v.W) + P.offset;
-  // FP32 with 16-point segments: two rows per group, their chains interleaved
-  constexpr int R = 1;  // rows per group (2 measured slower: fewer CTAs per SM)
-  const int rounds = (nr + R * ngroups - 1) / (R * ngroups);
-  for (int k = 0; k < rounds; ++k) {
-    T m[R][S];
-#pragma unroll
-    for (int t = 0; t < R; ++t) {
-      const int r = (k * ngroups + grp) * R + t;
-      const T* mrow = Ms + (size_t)((r < nr ? r : nr - 1) + 1) * lmp + l * (S + seg_pad<T>());
-#pragma unroll
-      for (int c = 0; c < S / 4; ++c) ld4(mrow + 4 * c, &m[t][4 * c]);
-      const T left = __shfl_sync(kFull, m[t][S - 1], (l + G - 1) & (G - 1), G);
-      const T right = __shfl_sync(kFull, m[t][0], (l + 1) & (G - 1), G);
-      T prev = left;
-#pragma unroll
-      for (int c = 0; c < S / 4; ++c) {
-        T up[4], dn[4];
-        ld4(mrow - lmp + 4 * c, up);
-        ld4(mrow + lmp + 4 * c, dn);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int u = 4 * c + q;
-          const T cur = m[t][u];
-          const T e = u + 1 < S ? m[t][u + 1] : right;
-          m[t][u] = fma(w0, cur, fma(rho, dn[q] + up[q], e + prev));
-          prev = cur;
-        }
-      }
-    }
-    seg_sweep<T, S, R, false>(m, p1, p2, l, G, lg, Ks, Bf);
-    seg_sweep<T, S, R, true>(m, p1, p2, l, G, lg, Ks, Bb);
-#pragma unroll
-    for (int t = 0; t < R; ++t) {
-      const int r = (k * ngroups + grp) * R + t;
-      if (r < nr) {
-        T* dst = W + (int64_t)(j0 + r) * nx + l * S;
-#pragma unroll
-        for (int c = 0; c < S / 4; ++c) st4(dst + 4 * c, &m[t][4 * c]);
-      }
-    }
-  }
+  seg_rows<T, S>(v, tl, P, Ms, lmp, Ks, [](int r) { return r; });
 }
 
 // -------------------------------------------------------------------------------------
@@ -1035,6 +1048,125 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? (S == 16 ? 4 : 3) : 1) r
     t = nt;
     cur ^= 1;
   }
+}
+
+// -------------------------------------------------------------------------------------
+// Fused row kernel, segment form in one tile (FP32): mu is formed in place, so the band takes half
+// the shared memory of a C and a mu tile and an SM holds four CTAs instead of two (rows_seg_kernel,
+// latency-bound at 16 warps per SM: 64 x 512^2 compensated 76 us per launch, here 60; 16 x 1024^2
+// 72 us, 60).  A warp takes strips of 32 CPL columns, CPL per lane, with three C rows in registers:
+// the upper half of the mu rows going down (mu row r over C row r), the lower half going up (mu row
+// r over C row r + 2), so that the C rows both halves read stay until both have read them.  Strip
+// edges go through Es.  The same operations in the same order as seg_tile.
+// Shared memory: tile (nr + 4) x (nx + 4 per segment), Es ns x 2 x (nr + 4), the 24 scan constants
+// and the sample flag, the reduction buffer.
+// -------------------------------------------------------------------------------------
+template <int S, int CPL>
+__global__ void __launch_bounds__(256, S == 16 ? 4 : 3) rows_walk_kernel(DevView v, int base) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const Tile tl = v.row_tiles[base + blockIdx.x];
+  MemberState* st = v.ms + tl.member;
+  if (st->remaining <= 0) {
+    if (tl.index == 0 && threadIdx.x == 0) st->active = 0;
+    return;
+  }
+  const MemberParams& P = v.mp[tl.member];
+  const int nx = P.nx, ny = P.ny, j0 = tl.start, nr = tl.count;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int pitch = nx + 4 * (nx / S), ns = (nx + 32 * CPL - 1) / (32 * CPL);
+  float* Cs = reinterpret_cast<float*>(smem);
+  float* Es = Cs + (size_t)(nr + 4) * pitch;
+  float* Ks = Es + ((2 * ns * (nr + 4) + 3) & ~3);
+  int* s_sample = reinterpret_cast<int*>(Ks + 24);
+  double* red = red_buffer(smem, (size_t)(reinterpret_cast<unsigned char*>(Ks + 28) - smem));
+  {
+    const float* field = static_cast<const float*>(v.C) + P.offset;
+    const int nq = nx >> 2;
+    for (int r = warp; r < nr + 4; r += nwarps) {
+      int j = j0 - 2 + r;
+      j = j < 0 ? j + ny : (j >= ny ? j - ny : j);
+      const float* src = field + (int64_t)j * nx;
+      float* d = Cs + (size_t)r * pitch;
+      for (int q = lane; q < nq; q += 32) cp_async16(d + seg_addr<float, S>(4 * q), src + 4 * q);
+    }
+  }
+  seg_tile_setup<float>(v, tl, P, Ks, s_sample);
+  cp_async_wait_all();
+  __syncthreads();
+  for (int k = threadIdx.x; k < 2 * ns * (nr + 4); k += blockDim.x) {
+    const int e = k / (nr + 4), t = k - e * (nr + 4), s = e >> 1;
+    const int i = (e & 1) ? min(32 * CPL * (s + 1), nx) - 1 : 32 * CPL * s;
+    Es[k] = Cs[(size_t)t * pitch + seg_addr<float, S>(i)];
+  }
+  __syncthreads();
+  const int h = (nr + 2) / 2;  // mu rows 0 .. h - 1 going down, h .. nr + 1 going up
+  {
+    const float a = P.fa, bx = P.fbx, by = P.fby;
+    for (int item = warp; item < 2 * ns; item += nwarps) {
+      const int s = item >> 1;
+      const bool up = item & 1;
+      const int lanes = min(32, (nx - 32 * CPL * s) / CPL);
+      const int i = 32 * CPL * s + CPL * min(lane, lanes - 1);
+      float* col = Cs + seg_addr<float, S>(i);
+      const float* ew = Es + (2 * (s == 0 ? ns - 1 : s - 1) + 1) * (nr + 4) + 1;
+      const float* ee = Es + (2 * (s + 1 == ns ? 0 : s + 1)) * (nr + 4) + 1;
+      const int r_first = up ? nr + 1 : 0, step = up ? -1 : 1, count = up ? nr + 2 - h : h;
+      // p: the row already passed on the walk's side, c: the centre row, x: the next one
+      float p[CPL], c[CPL], x[CPL];
+      auto ld = [&](int r, float* q) {
+        if constexpr (CPL == 4)
+          ld4(col + (size_t)r * pitch, q);
+        else {
+          const float2 t = *reinterpret_cast<const float2*>(col + (size_t)r * pitch);
+          q[0] = t.x;
+          q[1] = t.y;
+        }
+      };
+      ld(up ? nr + 3 : 0, p);
+      ld(up ? nr + 2 : 1, c);
+      int r = r_first;
+#pragma unroll 2
+      for (int k = 0; k < count; ++k, r += step) {
+        ld(up ? r : r + 2, x);
+        float w = __shfl_up_sync(kFull, c[CPL - 1], 1), e = __shfl_down_sync(kFull, c[0], 1);
+        if (lane == 0) w = ew[r];
+        if (lane == lanes - 1) e = ee[r];
+        float m[CPL];
+#pragma unroll
+        for (int q = 0; q < CPL; ++q) {
+          const float ce = q + 1 < CPL ? c[q + 1 < CPL ? q + 1 : q] : e;
+          const float cw = q > 0 ? c[q > 0 ? q - 1 : 0] : w;
+          const float u = c[q] * fmaf(c[q], c[q], -a);
+          m[q] = fmaf(-by, x[q] + p[q], fmaf(-bx, ce + cw, u));
+        }
+        float* out = col + (size_t)(up ? r + 2 : r) * pitch;
+        if (lane < lanes) {
+          if constexpr (CPL == 4)
+            st4(out, m);
+          else
+            *reinterpret_cast<float2*>(out) = make_float2(m[0], m[1]);
+        }
+#pragma unroll
+        for (int q = 0; q < CPL; ++q) {
+          p[q] = c[q];
+          c[q] = x[q];
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (*s_sample) {
+    band_partials_field<float>(v, tl, nx, nr, P, v.partials + P.partial_base + tl.index, red);
+    __syncthreads();
+  }
+  seg_rows<float, S>(v, tl, P, Cs, pitch, Ks, [h](int r) { return r < h ? r : r + 2; });
+}
+
+// Shared memory of rows_walk_kernel for a band of nr rows.
+size_t rows_walk_smem(int nr, int nx, int S) {
+  const int cpl = S == 16 ? 2 : 4, ns = (nx + 32 * cpl - 1) / (32 * cpl);
+  const size_t f = (size_t)(nr + 4) * (nx + 4 * (nx / S)) + ((2 * ns * (nr + 4) + 3) & ~3) + 28;
+  return ((f * sizeof(float) + 15) & ~(size_t)15) + 16 * sizeof(double);
 }
 
 // -------------------------------------------------------------------------------------
@@ -2273,6 +2405,15 @@ size_t rowT_smem_bytes(int nw) {
   return b + (size_t)2 * nw * sizeof(double);
 }
 
+// The segment-form row kernel of one class, one CTA per band: FP32 in one tile, FP64 in two.
+template <typename T, int S>
+void rows_plain(const DevView& v, const LaunchShape& sh, int c, int base, int n, int threads, cudaStream_t st) {
+  if constexpr (sizeof(T) == sizeof(float))
+    rows_walk_kernel<S, S == 16 ? 2 : 4><<<n, threads, sh.walk_smem[c], st>>>(v, base);
+  else
+    rows_seg_kernel<T, S, false><<<n, threads, sh.seg_smem[c], st>>>(v, base, n, sh.seg_ccap[c], sh.seg_mcap[c]);
+}
+
 template <typename T>
 void seg_launch(const DevView& v, const LaunchShape& sh, cudaStream_t st) {
   const int threads = min(sh.rows_threads, 256);
@@ -2291,12 +2432,12 @@ void seg_launch(const DevView& v, const LaunchShape& sh, cudaStream_t st) {
         if (sh.seg_persist)
           rows_seg_kernel<T, 16, true><<<grid, threads, sm, st>>>(v, base, n, cc, mc);
         else
-          rows_seg_kernel<T, 16, false><<<grid, threads, sm, st>>>(v, base, n, cc, mc);
+          rows_plain<T, 16>(v, sh, c, base, n, threads, st);
       } else {
         if (sh.seg_persist)
           rows_seg_kernel<T, 32, true><<<grid, threads, sm, st>>>(v, base, n, cc, mc);
         else
-          rows_seg_kernel<T, 32, false><<<grid, threads, sm, st>>>(v, base, n, cc, mc);
+          rows_plain<T, 32>(v, sh, c, base, n, threads, st);
       }
     }
     base += n;
@@ -2472,12 +2613,19 @@ cudaError_t smem_limits_impl() {
     return e;
   if ((e = cudaFuncSetAttribute(rowsT_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) != cudaSuccess)
     return e;
-  if ((e = cudaFuncSetAttribute(rows_seg_kernel<T, 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) !=
-      cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(rows_seg_kernel<T, 32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) !=
-      cudaSuccess)
-    return e;
+  if constexpr (sizeof(T) == sizeof(float)) {
+    if ((e = cudaFuncSetAttribute(rows_walk_kernel<16, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) !=
+            cudaSuccess ||
+        (e = cudaFuncSetAttribute(rows_walk_kernel<32, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) !=
+            cudaSuccess)
+      return e;
+  } else {
+    if ((e = cudaFuncSetAttribute(rows_seg_kernel<T, 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) !=
+            cudaSuccess ||
+        (e = cudaFuncSetAttribute(rows_seg_kernel<T, 32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) !=
+            cudaSuccess)
+      return e;
+  }
   if ((e = cudaFuncSetAttribute(rows_seg_kernel<T, 16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) !=
       cudaSuccess)
     return e;
@@ -2505,6 +2653,8 @@ cudaError_t set_kernel_smem_limits(int precision) {
     return e;
   return res_smem_limit<256, 64, true>();
 }
+
+size_t walk_smem_bytes(int nr, int nx, int S) { return rows_walk_smem(nr, nx, S); }
 
 size_t resident_smem_bytes(int nx, int nr, int comp) { return res_smem_bytes(nx, nr, comp != 0); }
 
