@@ -95,6 +95,9 @@ __device__ __forceinline__ float f32_trunc(double x) {
   return __uint_as_float(bits);
 }
 
+// A line on its way to L2.
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p)); }
+
 // Fixed-order block reduction of two FP64 sums (deterministic for a given block size).
 __device__ __forceinline__ void block_sum2(double& a, double& b, double* red) {
 #pragma unroll

@@ -46,18 +46,6 @@
 namespace chk {
 namespace {
 
-// (double)v, truncated to 53 bits (it is the update of C, far below C itself), on the integer
-// pipes: the conversion instruction takes the FP64 pipe 16 SM clocks per warp, which the update
-// and the scans need.
-__device__ __forceinline__ double to_double(i64 v) {
-  const i64 s = v >> 63;
-  const unsigned long long m = (unsigned long long)((v ^ s) - s);
-  const int lz = __clzll((i64)m);
-  const unsigned long long q = (m << lz) >> 11;  // 53 bits, the leading one adds 1 to the exponent
-  const int hi = (int)(q >> 32) + ((1085 - lz) << 20) + ((int)(s >> 32) & 0x80000000);
-  return m == 0 ? 0.0 : __hiloint2double(hi, (int)q);
-}
-
 // Asynchronous global -> shared copy of one value.
 __device__ __forceinline__ void copy8(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
@@ -558,22 +546,21 @@ __device__ __forceinline__ void col_update(const A& ar, const i64* y, int len, d
   }
 }
 
-// The scaled forward pass from a zero state over W as its copies arrive, in 4 groups of S / 4 rows
-// per segment.  Rows come in bands of one exponent that start at multiples of 8 (ws: the segment's
+// The scaled forward pass from a zero state over W as its copies arrive, in 4 groups of 8 rows per
+// segment.  Rows come in bands of one exponent that start at multiples of 8 (ws: the segment's
 // row exponents).
 template <class A, class Scaled>
 __device__ __forceinline__ void col_first(const A& ar, i64* y, int len, int S, const short2* ws,
                                           typename A::State& a, typename A::State& b, const Scaled& scaled) {
   a = A::zero();
   b = A::zero();
-  const int per = max(S >> 2, 8);
 #pragma unroll 1
   for (int k = 0; k < S; k += 8) {
     if (k == 0)
       asm volatile("cp.async.wait_group 3;\n" ::: "memory");
-    else if (k == per)
+    else if (k == 8)
       asm volatile("cp.async.wait_group 2;\n" ::: "memory");
-    else if (k == 2 * per)
+    else if (k == 16)
       asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     else
       asm volatile("cp.async.wait_group 0;\n" ::: "memory");
@@ -622,40 +609,46 @@ __global__ void __launch_bounds__(kColThreads, 3) fx_cols_kernel(DevView v, int 
   // All of the panel's W in flight in up to 4 groups of rows of every segment (value u of segment g
   // at u 256 + g cw, so a row piece of the panel is contiguous on both sides), in 16-byte pieces
   // where the rows allow it; C on its way to L2 for the update.
+  // the row exponents' maxima, 8 loads ahead of the copies (ny <= 256; the rest below)
+  short2 we8[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) we8[k] = we[min(lane + 32 * k, ny - 1)];
   {
     i64* Y = reinterpret_cast<i64*>(smem);
-    const i64* Wm = static_cast<const i64*>(v.W) + P.offset + tl.start;
     const bool wide = !((nx | tl.count) & 1);
-    const int E = wide ? 2 : 1, cols = wide ? tl.count >> 1 : tl.count, per = max(S >> 2, 8);
-    const int half = wide ? cw >> 1 : cw, rows_at_once = kColThreads / half;
+    const int half = wide ? cw >> 1 : cw, cols = wide ? tl.count >> 1 : tl.count;
     const int tc = threadIdx.x % half, tr = threadIdx.x / half;
-    for (int g = 0; g < 4; ++g) {
-      // rows u0 .. u0 + per - 1 of every segment, numbered q = segment per + (u - u0)
-      const int u0 = g * per;
-      if (u0 < S && tc < cols)
-        for (int q = tr; q < G * per; q += rows_at_once) {
-          const int sq = q / per, u = u0 + q - sq * per, j = sq * S + u;
-          if (j < ny) {
-            const i64* src = Wm + (int64_t)j * nx + E * tc;
-            i64* dst = Y + u * kColThreads + sq * cw + E * tc;
-            if (wide)
-              copy16(dst, src);
-            else
-              copy8(dst, src);
-          }
+    // a thread copies column piece tc of rows u0 + (tr & 7) of segments tr / 8, + step, ...
+    const int step = kColThreads / half / 8, u = tr & 7, s0 = tr >> 3, E = wide ? 2 : 1;
+    const i64* Wm = static_cast<const i64*>(v.W) + P.offset + tl.start + E * tc;
+    const int64_t dsrc = (int64_t)step * S * nx;
+    for (int u0 = 0; u0 < 32; u0 += 8) {
+      if (u0 < S && tc < cols) {
+        const i64* src = Wm + (int64_t)(s0 * S + u0 + u) * nx;
+        i64* dst = Y + (u0 + u) * kColThreads + s0 * cw + E * tc;
+        for (int q = s0, j = s0 * S + u0 + u; q < G && j < ny; q += step, j += step * S) {
+          if (wide)
+            copy16(dst, src);
+          else
+            copy8(dst, src);
+          src += dsrc;
+          dst += step * cw;
         }
+      }
       asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
     const char* Cm = static_cast<const char*>(v.C) + 8 * (P.offset + tl.start);
     for (int j = threadIdx.x; j < ny; j += kColThreads) {
       const char* p = Cm + (int64_t)j * nx * 8;
-      asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p));
-      asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p + 8 * (tl.count - 1)));
-      if (tl.count > 16) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p + 128));
+      prefetch_l2(p);
+      prefetch_l2(p + 8 * (tl.count - 1));
+      if (tl.count > 16) prefetch_l2(p + 128);
     }
   }
   int emax = -32768;
-  for (int j = lane; j < ny; j += 32) emax = max(emax, (int)we[j].y);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) emax = max(emax, (int)we8[k].y);
+  for (int j = lane + 256; j < ny; j += 32) emax = max(emax, (int)we[j].y);
   emax = __reduce_max_sync(kAll, emax);
   const bool bad = emax == kBadRow;
   i64* const ye = y + max(len - 1, 0) * kColThreads;
@@ -674,7 +667,7 @@ __global__ void __launch_bounds__(kColThreads, 3) fx_cols_kernel(DevView v, int 
     const int up = 62 - gain - emax;
     col_first(ar, y, len, S, ws, a, b, [up](short2 e, auto f) { with_shift(max(-62, min(62, up + (int)e.x)), f); });
     const int sl = col_solve(ar, y, len, tab, xs, wtop, G, gw, P.fx_lvy, ny % S == 0, cw, gain, a, b);
-    col_update(ar, ye, len, Ce, nx, P.kappa * ldexp(1.0, -up - sl), cv, a, b, [](i64 t) { return to_double(t); });
+    col_update(ar, ye, len, Ce, nx, P.kappa * ldexp(1.0, -up - sl), cv, a, b, [](i64 t) { return (double)t; });
   }
   if (tl.index == 0 && threadIdx.x == 0) finalize_sample(v, tl.member, st, P);
 }
