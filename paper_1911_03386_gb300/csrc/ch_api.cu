@@ -848,6 +848,13 @@ int upload_tiles(ch_ensemble* h) {
     if (e == cudaSuccess) cap = need;
     return e;
   };
+  for (int c = 0; c < chk::kResClasses; ++c) {
+    if (h->shape.res_n[c] > 0 && h->res_cap[c] == 0 && chk::resident_capacity(c, &h->res_cap[c]) != cudaSuccess) {
+      cudaGetLastError();
+      h->res_cap[c] = 0;
+    }
+    h->shape.res_cap[c] = h->res_cap[c];
+  }
   cudaError_t e;
   if ((e = ensure((void**)&h->drt, h->cap_rt, h->rt.size(), sizeof(Tile))) != cudaSuccess ||
       (e = ensure((void**)&h->dst, h->cap_st, h->st.size(), sizeof(Tile))) != cudaSuccess ||
@@ -1038,14 +1045,15 @@ int fork_resident(ch_ensemble* h, int64_t n) {
   const int nc = chk::resident_classes(h->shape);
   if (nc == 0 || n <= 0) return CH_OK;
   if (nc == 1 && h->shape.n_row_tiles + h->shape.fx_tiles == 0) {  // nothing to overlap with
-    CH_CUDA(chk::launch_resident(h->view(), h->precision, h->shape, n, &h->stream, 1), "resident step launch");
+    CH_CUDA(chk::launch_resident(h->view(), h->precision, h->shape, n, &h->stream, 1, true),
+            "resident step launch");
     return CH_OK;
   }
   if (int rc = ensure_aux(h)) return rc;
   const int na = std::min(nc, (int)ch_ensemble::kAux);
   CH_CUDA(cudaEventRecord(h->fork, h->stream), "fork");
   for (int i = 0; i < na; ++i) CH_CUDA(cudaStreamWaitEvent(h->aux[i], h->fork, 0), "fork");
-  CH_CUDA(chk::launch_resident(h->view(), h->precision, h->shape, n, h->aux, na), "resident step launch");
+  CH_CUDA(chk::launch_resident(h->view(), h->precision, h->shape, n, h->aux, na, false), "resident step launch");
   for (int i = 0; i < na; ++i) CH_CUDA(cudaEventRecord(h->aux_done[i], h->aux[i]), "join");
   h->aux_used = na;
   return CH_OK;

@@ -28,6 +28,7 @@ struct ch_ensemble {
   std::vector<Tile> cst;            // CTAs of the segment column kernel
   std::vector<Tile> rt, st, ct;   // stencil/fused bands, row-sweep bands, column panels
   std::vector<Tile> rest;         // members of the cluster-resident form (FP32), by class
+  int res_cap[chk::kResClasses] = {};  // LaunchShape::res_cap, found when a class is first used
   chk::LaunchShape shape{};
   ch_tuning tuning{};             // as requested (0 / -1 = default)
   bool fx_fused = false;          // server: the fixed-point form beside the fused one

@@ -193,6 +193,7 @@ struct LaunchShape {
   size_t colseg_smem[4];
   // cluster-resident members (FP32): tiles per class (see res_class)
   int res_n[kResClasses];
+  int res_cap[kResClasses];  // clusters of the class the device holds at once (0: not known)
   // fixed-point members (FP64): row tiles by class after the n_row_tiles others, column tiles
   // after the other segment-form ones
   int fx_rt[kFxRowClasses], fx_ct;
@@ -231,9 +232,12 @@ cudaError_t launch_step(const DevView& v, int precision, const LaunchShape& sh, 
 cudaError_t launch_phase(const DevView& v, int precision, int phase, const LaunchShape& sh, cudaStream_t st);
 cudaError_t launch_observe(const DevView& v, int precision, const LaunchShape& sh, cudaStream_t st);
 // nsteps steps of every cluster-resident member (no-op when there are none), in launches
-// of at most kResChunk steps; each class present goes to streams[i % nstreams].
+// of at most kResChunk steps; each class present goes to streams[i % nstreams].  alone: nothing
+// else runs beside them (members then take turns in what would be a nearly empty last wave).
 cudaError_t launch_resident(const DevView& v, int precision, const LaunchShape& sh, int64_t nsteps,
-                            const cudaStream_t* streams, int nstreams);
+                            const cudaStream_t* streams, int nstreams, bool alone);
+// Clusters of resident class ci that the device holds at once.
+cudaError_t resident_capacity(int ci, int* cap);
 // Number of resident classes present in a launch shape.
 int resident_classes(const LaunchShape& sh);
 // Dynamic shared memory of the one-tile segment-form row kernel (FP32).

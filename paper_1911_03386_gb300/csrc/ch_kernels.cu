@@ -1892,8 +1892,14 @@ __host__ __device__ constexpr size_t res_smem_bytes(int nx, int nr, bool comp) {
          16 * sizeof(double2) + (sizeof(MemberState) + 15) / 16 * 16;
 }
 
+// The steps of a launch.  Clusters take positions pos, pos + 1, ..: position p is the (p / width)-th
+// of `parts` equal parts of nsteps steps of the member of tile base + p % width.
+struct ResRun {
+  int base, width, pos, parts, nsteps;
+};
+
 template <int NX, int NR, bool COMP, bool OBS>
-__global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v, int tile_base, int64_t nsteps) {
+__global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v, ResRun run) {
   constexpr int TH = 8 * NR;      // threads per CTA
   constexpr int S = NX / 16;      // row points per lane
   constexpr int SC = NX / 8;      // column points per thread
@@ -1912,7 +1918,9 @@ __global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v
   MemberState* lst = reinterpret_cast<MemberState*>(part + 16);
 
   const unsigned Q = cluster_size(), rank = cluster_rank();
-  const Tile tl = v.res_tiles[tile_base + blockIdx.x / Q];
+  const int pos = run.pos + (int)(blockIdx.x / Q), part_k = pos / run.width;  // (see ResRun)
+  const Tile tl = v.res_tiles[run.base + pos - part_k * run.width];
+  const int nsteps = run.nsteps * (part_k + 1) / run.parts - run.nsteps * part_k / run.parts;
   const int m = tl.member;
   const MemberParams& P = v.mp[m];
   MemberState* st = v.ms + m;
@@ -2540,9 +2548,10 @@ cudaError_t phase_impl(const DevView& v, int phase, const LaunchShape& sh, cudaS
   return cudaGetLastError();
 }
 
-// One launch of the resident kernel over the n tiles of one class (clusters of Q CTAs).
+// One launch of the resident kernel over n positions of `run` (clusters of Q CTAs); cap: only
+// how many such clusters the device holds at once.
 template <int NX, int NR, bool COMP, bool OBS>
-cudaError_t res_launch(const DevView& v, int base, int n, int Q, int64_t nsteps, cudaStream_t st) {
+cudaError_t res_launch(const DevView& v, const ResRun& run, int n, int Q, cudaStream_t st, int* cap) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(n * Q), 1, 1);
   cfg.blockDim = dim3(8 * NR, 1, 1);
@@ -2555,32 +2564,54 @@ cudaError_t res_launch(const DevView& v, int base, int n, int Q, int64_t nsteps,
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, res_kernel<NX, NR, COMP, OBS>, v, base, nsteps);
+  if (cap) return cudaOccupancyMaxActiveClusters(cap, res_kernel<NX, NR, COMP, OBS>, &cfg);
+  return cudaLaunchKernelEx(&cfg, res_kernel<NX, NR, COMP, OBS>, v, run);
 }
 
 template <bool OBS>
-cudaError_t res_all(const DevView& v, const LaunchShape& sh, int64_t nsteps, cudaStream_t st) {
-  int base = 0;
-  for (int ci = 0; ci < kResClasses; ++ci) {
-    const int n = sh.res_n[ci];
-    if (n <= 0) continue;
-    const int Q = ci % 8 + 1;
-    const bool comp = (ci / 8) & 1;
-    const int form = ci / 16;  // 0: 128 columns, 32 rows; 1: 256 columns, 32 rows; 2: 256, 64
-    cudaError_t e;
-    if (form == 2)
-      e = comp ? res_launch<256, 64, true, OBS>(v, base, n, Q, nsteps, st)
-               : res_launch<256, 64, false, OBS>(v, base, n, Q, nsteps, st);
-    else if (form == 1)
-      e = comp ? res_launch<256, 32, true, OBS>(v, base, n, Q, nsteps, st)
-               : res_launch<256, 32, false, OBS>(v, base, n, Q, nsteps, st);
-    else
-      e = comp ? res_launch<128, 32, true, OBS>(v, base, n, Q, nsteps, st)
-               : res_launch<128, 32, false, OBS>(v, base, n, Q, nsteps, st);
-    if (e != cudaSuccess) return e;
-    base += n;
+cudaError_t res_class_launch(const DevView& v, int ci, const ResRun& run, int n, cudaStream_t st, int* cap = nullptr) {
+  const int Q = ci % 8 + 1;
+  const bool comp = (ci / 8) & 1;
+  switch (ci / 16) {  // 0: 128 columns, 32 rows; 1: 256 columns, 32 rows; 2: 256, 64
+    case 2:
+      return comp ? res_launch<256, 64, true, OBS>(v, run, n, Q, st, cap)
+                  : res_launch<256, 64, false, OBS>(v, run, n, Q, st, cap);
+    case 1:
+      return comp ? res_launch<256, 32, true, OBS>(v, run, n, Q, st, cap)
+                  : res_launch<256, 32, false, OBS>(v, run, n, Q, st, cap);
+    default:
+      return comp ? res_launch<128, 32, true, OBS>(v, run, n, Q, st, cap)
+                  : res_launch<128, 32, false, OBS>(v, run, n, Q, st, cap);
   }
-  return cudaSuccess;
+}
+
+// Steps of the n members of one class.  The clusters the device holds at once (cap) take whole
+// members while more than 2 cap are left; where the rest, cap + b of them, would end in a wave of b,
+// they take turns instead: their steps in `parts` equal parts, cap members per launch in cyclic
+// order, so that every launch but the last is full.  A launch costs about one step's time (load and
+// store of the fields, drain), a wave of b 0.7 of a full one while every CTA has an SM to itself;
+// the cheapest number of parts is taken.  us per step without and with turns, 160 steps per call
+// (256^2: cap 36): 40 x 256^2 12.5 and 9.2, 54 x 256^2 14.9 and 11.7, 256 x 256^2 55.6 and 54.7,
+// 256 x 128^2 24.5 and 22.5.
+cudaError_t res_turns(const DevView& v, int ci, int n, int nsteps, int cap, cudaStream_t st) {
+  const int b = cap > 0 ? n % cap : 0, width = b > 0 && n > cap ? cap + b : 0;
+  int parts = 1;
+  if (width > 0) {
+    double best = (nsteps + 1) * (2 * b <= cap ? 1.7 : 2.0);
+    for (int r = 2; r <= 16 && r <= nsteps; ++r) {
+      const double t = ((width * r + cap - 1) / cap) * ((double)nsteps / r + 1.0);
+      if (t < best) {
+        best = t;
+        parts = r;
+      }
+    }
+  }
+  const int whole = parts > 1 ? n - width : n;
+  cudaError_t e = cudaSuccess;
+  if (whole > 0) e = res_class_launch<false>(v, ci, ResRun{0, whole, 0, 1, nsteps}, whole, st);
+  for (int pos = 0; parts > 1 && pos < width * parts && e == cudaSuccess; pos += cap)
+    e = res_class_launch<false>(v, ci, ResRun{whole, width, pos, parts, nsteps}, min(cap, width * parts - pos), st);
+  return e;
 }
 
 template <int NX, int NR, bool COMP>
@@ -2613,7 +2644,14 @@ cudaError_t observe_impl(const DevView& v, const LaunchShape& sh, cudaStream_t s
     stencil_block_kernel<T, true><<<sh.rt_blk, sh.rows_threads, sh.blk_smem, st>>>(v, whole);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  if (sizeof(T) == sizeof(float) && (e = res_all<true>(v, sh, 0, st)) != cudaSuccess) return e;
+  if (sizeof(T) == sizeof(float)) {
+    int base = 0;
+    for (int ci = 0; ci < kResClasses; ++ci) {
+      const int n = sh.res_n[ci];
+      if (n > 0 && (e = res_class_launch<true>(v, ci, ResRun{base, n, 0, 1, 0}, n, st)) != cudaSuccess) return e;
+      base += n;
+    }
+  }
   if (sizeof(T) == sizeof(double) && (e = launch_fx_observe(v, sh, st)) != cudaSuccess) return e;
   obs_finalize_kernel<<<(v.m + 127) / 128, 128, 0, st>>>(v);
   return cudaGetLastError();
@@ -2683,29 +2721,28 @@ size_t walk_smem_bytes(int nr, int nx, int S) { return rows_walk_smem(nr, nx, S)
 size_t resident_smem_bytes(int nx, int nr, int comp) { return res_smem_bytes(nx, nr, comp != 0); }
 
 cudaError_t launch_resident(const DevView& v, int precision, const LaunchShape& sh, int64_t nsteps,
-                            const cudaStream_t* streams, int nstreams) {
+                            const cudaStream_t* streams, int nstreams, bool alone) {
   if (precision == 0 || nsteps <= 0) return cudaSuccess;
   // the classes present, each on its own stream (round robin)
   int base = 0, j = 0;
   for (int ci = 0; ci < kResClasses; ++ci) {
     const int n = sh.res_n[ci];
     if (n <= 0) continue;
-    LaunchShape one{};
-    one.res_n[ci] = n;
-    const DevView vc = [&] {
-      DevView w = v;
-      w.res_tiles = v.res_tiles + base;
-      return w;
-    }();
+    DevView vc = v;
+    vc.res_tiles += base;
     const cudaStream_t st = streams[j++ % nstreams];
     for (int64_t done = 0; done < nsteps; done += kResChunk) {
       const int64_t k = nsteps - done < kResChunk ? nsteps - done : kResChunk;
-      cudaError_t e = res_all<false>(vc, one, k, st);
+      cudaError_t e = res_turns(vc, ci, n, (int)k, alone ? sh.res_cap[ci] : 0, st);
       if (e != cudaSuccess) return e;
     }
     base += n;
   }
   return cudaSuccess;
+}
+
+cudaError_t resident_capacity(int ci, int* cap) {
+  return res_class_launch<false>(DevView{}, ci, ResRun{}, 1, nullptr, cap);
 }
 
 int resident_classes(const LaunchShape& sh) {
