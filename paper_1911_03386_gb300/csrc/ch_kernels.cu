@@ -1804,6 +1804,92 @@ __device__ __forceinline__ float2 mat2v_add(const float* A, float2 v, float2 w) 
   return make_float2(fmaf(A[0], v.x, fmaf(A[1], v.y, w.x)), fmaf(A[2], v.x, fmaf(A[3], v.y, w.y)));
 }
 
+// Two FP32 values in one 64-bit register pair, and a fused multiply-add of both in one instruction
+// (each half rounded as fmaf).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 r) {
+  float2 x;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x.x), "=f"(x.y) : "l"(r));
+  return x;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// seg_sweep of two FP32 rows over 16 lanes, their values in pairs: the same operations in half the
+// instructions.
+template <int S, bool REV>
+__device__ __forceinline__ void seg_sweep2(f32x2 (&y)[S], f32x2 p1, f32x2 p2, int l, const float* Ks, const float (&B)[4]) {
+  f32x2 a = 0, b = 0;
+#pragma unroll
+  for (int k = 0; k < S; ++k) {
+    const f32x2 v = fma2(p1, a, fma2(p2, b, y[REV ? S - 1 - k : k]));
+    b = a;
+    a = v;
+  }
+  float2 fa = unpack2(a), fb = unpack2(b);
+  const int pos = REV ? 15 - l : l;
+#pragma unroll
+  for (int d = 0; d < 4; ++d) {
+    const int delta = 1 << d;
+    float A[4];
+    ld4(Ks + 4 * d, A);
+    float2 ya, yb;
+    ya.x = REV ? __shfl_down_sync(kFull, fa.x, delta, 16) : __shfl_up_sync(kFull, fa.x, delta, 16);
+    ya.y = REV ? __shfl_down_sync(kFull, fa.y, delta, 16) : __shfl_up_sync(kFull, fa.y, delta, 16);
+    yb.x = REV ? __shfl_down_sync(kFull, fb.x, delta, 16) : __shfl_up_sync(kFull, fb.x, delta, 16);
+    yb.y = REV ? __shfl_down_sync(kFull, fb.y, delta, 16) : __shfl_up_sync(kFull, fb.y, delta, 16);
+    if (pos >= delta) {
+      const float nx = fmaf(A[0], ya.x, fmaf(A[1], yb.x, fa.x)), ny = fmaf(A[0], ya.y, fmaf(A[1], yb.y, fa.y));
+      fb.x = fmaf(A[2], ya.x, fmaf(A[3], yb.x, fb.x));
+      fb.y = fmaf(A[2], ya.y, fmaf(A[3], yb.y, fb.y));
+      fa = make_float2(nx, ny);
+    }
+  }
+  constexpr int last = REV ? 0 : 15;
+  float Pm[4];
+  ld4(Ks + 20, Pm);
+  auto start = [&](float& sa, float& sb) {
+    const float Ea = __shfl_sync(kFull, sa, last, 16), Eb = __shfl_sync(kFull, sb, last, 16);
+    const float xa = fmaf(Pm[0], Ea, Pm[1] * Eb), xb = fmaf(Pm[2], Ea, Pm[3] * Eb);
+    float pa = REV ? __shfl_down_sync(kFull, sa, 1, 16) : __shfl_up_sync(kFull, sa, 1, 16);
+    float pb = REV ? __shfl_down_sync(kFull, sb, 1, 16) : __shfl_up_sync(kFull, sb, 1, 16);
+    if (pos == 0) pa = pb = 0.0f;
+    sa = fmaf(B[0], xa, fmaf(B[1], xb, pa));
+    sb = fmaf(B[2], xa, fmaf(B[3], xb, pb));
+  };
+  start(fa.x, fb.x);
+  start(fa.y, fb.y);
+  a = pack2(fa.x, fa.y);
+  b = pack2(fb.x, fb.y);
+#pragma unroll
+  for (int k = 0; k < S; ++k) {
+    const int u = REV ? S - 1 - k : k;
+    const f32x2 v = fma2(p1, a, fma2(p2, b, y[u]));
+    y[u] = v;
+    b = a;
+    a = v;
+  }
+}
+
 // FP64 partial sums of the F and dF/dt densities over the CTA's own rows (C tile rows
 // 2 .. 33; hi + lo for compensated members), mu recomputed in FP64 from the stored field.
 // Thread = column i of a block of 32 NX / 256 rows, walking down with three field rows in
@@ -1971,13 +2057,13 @@ __global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v
       else if (k < 160)
         x = (k - 96) >> 2 < ns ? ty.Bf[(k - 96) >> 2][k & 3] : 0.f;
       else
-        x = ty.Hf[(k - 160) >> 2][k & 3];
+        x = ty.Hf[2 * ((k - 160) >> 3) + (k & 1)][(k >> 1) & 3];  // two rows' values side by side
       Ks[k] = x;
     }
   }
   const float* KB = Ks + 32;   // row start-state matrices M^(S l), l = 0 .. 15
   const float* KC = Ks + 96;   // column powers M^(SC k), k = 0 .. ns - 1
-  const float* KH = Ks + 160;  // column segment responses (g1, g2, k1, k2) per row
+  const float* KH = Ks + 160;  // column segment responses g1, g2, k1, k2 of two rows each
   // row phase: 16 lanes per row, rows 2 grp and 2 grp + 1
   const int l = tid & 15, grp = tid >> 4;
   const float a = P.fa, bx = P.fbx, by = P.fby, rho = P.frho, w0 = P.fw0;
@@ -2000,29 +2086,24 @@ __global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v
       const int q = tid % NQ, gr = tid / NQ, r1 = MT * (gr + 1) / NG;  // warp-uniform (NQ >= 32)
       int r = MT * gr / NG;
       const float* c0 = Ct + (r + 1) * NX;
-      float cc[4], nn[4], so[4];
-      ld4(c0 - NX + 4 * q, nn);
-      ld4(c0 + 4 * q, cc);
+      const ulonglong2* col = reinterpret_cast<const ulonglong2*>(c0 + 4 * q);  // values in pairs
+      const f32x2 na2 = pack2(-a, -a), nbx2 = pack2(-bx, -bx), nby2 = pack2(-by, -by);
+      ulonglong2 nn = col[-NQ], cc = col[0];
 #pragma unroll 3
-      for (; r < r1; ++r, c0 += NX) {
-        ld4(c0 + NX + 4 * q, so);
-        float w = __shfl_up_sync(kFull, cc[3], 1), e = __shfl_down_sync(kFull, cc[0], 1);
+      for (; r < r1; ++r, c0 += NX, col += NQ) {
+        const ulonglong2 so = col[NQ];
+        const float2 c01 = unpack2(cc.x), c23 = unpack2(cc.y);
+        float w = __shfl_up_sync(kFull, c23.y, 1), e = __shfl_down_sync(kFull, c01.x, 1);
         if (lane == 0) w = c0[q == 0 ? NX - 1 : 4 * q - 1];
         if (lane == 31) e = c0[q == NQ - 1 ? 0 : 4 * q + 4];
-        float out[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float ce = k < 3 ? cc[k + 1] : e;
-          const float cw = k > 0 ? cc[k - 1] : w;
-          const float u = cc[k] * fmaf(cc[k], cc[k], -a);
-          out[k] = fmaf(-by, so[k] + nn[k], fmaf(-bx, ce + cw, u));
-        }
-        st4(Mw + res_swz<NX>(r, 4 * q), out);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          nn[k] = cc[k];
-          cc[k] = so[k];
-        }
+        const f32x2 ew01 = pack2(c01.y + w, c23.x + c01.x), ew23 = pack2(c23.y + c01.y, e + c23.x);
+        const f32x2 u01 = mul2(cc.x, fma2(cc.x, cc.x, na2)), u23 = mul2(cc.y, fma2(cc.y, cc.y, na2));
+        ulonglong2 out;
+        out.x = fma2(nby2, add2(so.x, nn.x), fma2(nbx2, ew01, u01));
+        out.y = fma2(nby2, add2(so.y, nn.y), fma2(nbx2, ew23, u23));
+        *reinterpret_cast<ulonglong2*>(Mw + res_swz<NX>(r, 4 * q)) = out;
+        nn = cc;
+        cc = so;
       }
     }
     __syncthreads();
@@ -2059,9 +2140,18 @@ __global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v
       {
         float B[4];
         ld4(KB + 4 * l, B);
-        seg_sweep<float, S, 2, false>(y, p1x, p2x, l, 16, 4, Ks, B);
+        f32x2 z[S];
+#pragma unroll
+        for (int u = 0; u < S; ++u) z[u] = pack2(y[0][u], y[1][u]);
+        seg_sweep2<S, false>(z, pack2(p1x, p1x), pack2(p2x, p2x), l, Ks, B);
         ld4(KB + 4 * (15 - l), B);
-        seg_sweep<float, S, 2, true>(y, p1x, p2x, l, 16, 4, Ks, B);
+        seg_sweep2<S, true>(z, pack2(p1x, p1x), pack2(p2x, p2x), l, Ks, B);
+#pragma unroll
+        for (int u = 0; u < S; ++u) {
+          const float2 x = unpack2(z[u]);
+          y[0][u] = x.x;
+          y[1][u] = x.y;
+        }
       }
       __syncthreads();  // every mu read of this step is done: W replaces mu
 #pragma unroll
@@ -2118,53 +2208,61 @@ __global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v
       }
       const float* A = Ks + 24;  // M^SC: one segment, either direction
       const float* PP = Ks + 28; // (I - M^ny)^-1
-      const float Eb[4] = {KH[0], KH[1], KH[4], KH[5]};  // (x_0, x_1) per unit start state s
-      // forward: the total from zero, the periodic start x0, then s_k = M^(SC k) x0 + Y_k-1;
-      // backward end states with their true start: e_k + Eb s_k (kept in E[k].z, .w)
+      const float Eb[4] = {KH[0], KH[2], KH[1], KH[3]};  // (x_0, x_1) per unit start state s
+      // forward: the prefix Y_k-1 from zero (kept in E[k].x, .y) and the total, the periodic start
+      // x0, then s_k = M^(SC k) x0 + Y_k-1; backward end states with their true start: e_k + Eb s_k
+      // (kept in E[k].z, .w)
       float2 Y = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int k = 0; k < KMAX; ++k)
-        if (k < ns) Y = mat2v_add(A, Y, make_float2(E[k].x, E[k].y));
-      const float2 x0 = mat2v(PP, Y);
-      float2 s_own = x0, s_next = x0;
-      Y = make_float2(0.f, 0.f);
 #pragma unroll
       for (int k = 0; k < KMAX; ++k) {
         if (k < ns) {
-          const float2 sk = mat2v_add(KC + 4 * k, x0, Y);
+          const float2 f = make_float2(E[k].x, E[k].y);
+          E[k].x = Y.x;
+          E[k].y = Y.y;
+          Y = mat2v_add(A, Y, f);
+        }
+      }
+      const float2 x0 = mat2v(PP, Y);
+      float2 s_own = x0, s_next = x0;
+#pragma unroll
+      for (int k = 0; k < KMAX; ++k) {
+        if (k < ns) {
+          const float2 sk = mat2v_add(KC + 4 * k, x0, make_float2(E[k].x, E[k].y));
           if (k == gs) s_own = sk;
           if (k == (gs + 1 == ns ? 0 : gs + 1)) s_next = sk;
           const float2 eb = mat2v_add(Eb, sk, make_float2(E[k].z, E[k].w));
           E[k].z = eb.x;
           E[k].w = eb.y;
-          Y = mat2v_add(A, Y, make_float2(E[k].x, E[k].y));
         }
       }
-      // backward, segments from the last: the total, the periodic start of the last
-      // segment, then t_k = M^(SC (ns-1-k)) t_last + Z_k+1
+      // backward, segments from the last: the total (with the two sums Z_k+1 that are needed), the
+      // periodic start of the last segment, then t_k = M^(SC (ns-1-k)) t_last + Z_k+1
       // (k runs down from KMAX - 1 so that E is indexed by constants and stays in registers)
-      float2 Z = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int k = KMAX - 1; k >= 0; --k)
-        if (k < ns) Z = mat2v_add(A, Z, make_float2(E[k].z, E[k].w));
-      const float2 tl0 = mat2v(PP, Z);
-      float2 t_own = tl0, t_prev = tl0;
-      Z = make_float2(0.f, 0.f);
+      const int gp = gs == 0 ? ns - 1 : gs - 1;
+      float2 Z = make_float2(0.f, 0.f), z_own = Z, z_prev = Z;
 #pragma unroll
       for (int k = KMAX - 1; k >= 0; --k) {
         if (k < ns) {
-          const float2 tk = mat2v_add(KC + 4 * (ns - 1 - k), tl0, Z);
-          if (k == gs) t_own = tk;
-          if (k == (gs == 0 ? ns - 1 : gs - 1)) t_prev = tk;
+          if (k == gs) z_own = Z;
+          if (k == gp) z_prev = Z;
           Z = mat2v_add(A, Z, make_float2(E[k].z, E[k].w));
         }
       }
+      const float2 tl0 = mat2v(PP, Z);
+      const float2 t_own = mat2v_add(KC + 4 * (ns - 1 - gs), tl0, z_own);
+      const float2 t_prev = mat2v_add(KC + 4 * (ns - 1 - gp), tl0, z_prev);
       // the solution of this segment: closed form inside, the combination at its ends
+      {
+        const f32x2 sx = pack2(s_own.x, s_own.x), sy = pack2(s_own.y, s_own.y), tx = pack2(t_own.x, t_own.x),
+                    ty = pack2(t_own.y, t_own.y);
 #pragma unroll
-      for (int u = 2; u < SC - 2; ++u) {
-        float H[4];
-        ld4(KH + 4 * u, H);
-        y[u] = fmaf(H[3], t_own.y, fmaf(H[2], t_own.x, fmaf(H[1], s_own.y, fmaf(H[0], s_own.x, y[u]))));
+        for (int u = 2; u < SC - 2; u += 2) {
+          const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(KH + 4 * u);
+          const ulonglong2 k = *reinterpret_cast<const ulonglong2*>(KH + 4 * u + 4);
+          const float2 x = unpack2(fma2(k.y, ty, fma2(k.x, tx, fma2(g.y, sy, fma2(g.x, sx, pack2(y[u], y[u + 1]))))));
+          y[u] = x.x;
+          y[u + 1] = x.y;
+        }
       }
       y[0] = t_prev.x;
       y[1] = t_prev.y;
