@@ -1984,13 +1984,13 @@ struct ResRun {
   int base, width, pos, parts, nsteps;
 };
 
-template <int NX, int NR, bool COMP, bool OBS>
+// KMAX: column segments at most (ny / (NX / 8)).
+template <int NX, int NR, bool COMP, bool OBS, int KMAX>
 __global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v, ResRun run) {
   constexpr int TH = 8 * NR;      // threads per CTA
   constexpr int S = NX / 16;      // row points per lane
   constexpr int SC = NX / 8;      // column points per thread
   constexpr int NSEG = NR / SC;   // column segments per CTA
-  constexpr int KMAX = 256 / SC;  // column segments at most (ny <= 256)
   constexpr int NQ = NX / 4;      // 16-byte quads per row
   constexpr int CT = NR + 4, MT = NR + 2;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -2648,7 +2648,7 @@ cudaError_t phase_impl(const DevView& v, int phase, const LaunchShape& sh, cudaS
 
 // One launch of the resident kernel over n positions of `run` (clusters of Q CTAs); cap: only
 // how many such clusters the device holds at once.
-template <int NX, int NR, bool COMP, bool OBS>
+template <int NX, int NR, bool COMP, bool OBS, int KMAX = 8>
 cudaError_t res_launch(const DevView& v, const ResRun& run, int n, int Q, cudaStream_t st, int* cap) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(n * Q), 1, 1);
@@ -2662,8 +2662,8 @@ cudaError_t res_launch(const DevView& v, const ResRun& run, int n, int Q, cudaSt
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cap) return cudaOccupancyMaxActiveClusters(cap, res_kernel<NX, NR, COMP, OBS>, &cfg);
-  return cudaLaunchKernelEx(&cfg, res_kernel<NX, NR, COMP, OBS>, v, run);
+  if (cap) return cudaOccupancyMaxActiveClusters(cap, res_kernel<NX, NR, COMP, OBS, KMAX>, &cfg);
+  return cudaLaunchKernelEx(&cfg, res_kernel<NX, NR, COMP, OBS, KMAX>, v, run);
 }
 
 template <bool OBS>
@@ -2678,8 +2678,11 @@ cudaError_t res_class_launch(const DevView& v, int ci, const ResRun& run, int n,
       return comp ? res_launch<256, 32, true, OBS>(v, run, n, Q, st, cap)
                   : res_launch<256, 32, false, OBS>(v, run, n, Q, st, cap);
     default:
-      return comp ? res_launch<128, 32, true, OBS>(v, run, n, Q, st, cap)
-                  : res_launch<128, 32, false, OBS>(v, run, n, Q, st, cap);
+      if (Q <= 4)
+        return comp ? res_launch<128, 32, true, OBS, 8>(v, run, n, Q, st, cap)
+                    : res_launch<128, 32, false, OBS, 8>(v, run, n, Q, st, cap);
+      return comp ? res_launch<128, 32, true, OBS, 16>(v, run, n, Q, st, cap)
+                  : res_launch<128, 32, false, OBS, 16>(v, run, n, Q, st, cap);
   }
 }
 
@@ -2712,12 +2715,12 @@ cudaError_t res_turns(const DevView& v, int ci, int n, int nsteps, int cap, cuda
   return e;
 }
 
-template <int NX, int NR, bool COMP>
+template <int NX, int NR, bool COMP, int KMAX = 8>
 cudaError_t res_smem_limit() {
   const int b = (int)res_smem_bytes(NX, NR, COMP);
-  cudaError_t e = cudaFuncSetAttribute(res_kernel<NX, NR, COMP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  cudaError_t e = cudaFuncSetAttribute(res_kernel<NX, NR, COMP, false, KMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(res_kernel<NX, NR, COMP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  return cudaFuncSetAttribute(res_kernel<NX, NR, COMP, true, KMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
 }
 
 template <typename T>
@@ -2808,7 +2811,8 @@ cudaError_t set_kernel_smem_limits(int precision) {
   cudaError_t e;
   if (precision == 0) return (e = smem_limits_impl<double>()) != cudaSuccess ? e : set_fx_smem_limits();
   if ((e = smem_limits_impl<float>()) != cudaSuccess || (e = res_smem_limit<128, 32, false>()) != cudaSuccess ||
-      (e = res_smem_limit<128, 32, true>()) != cudaSuccess || (e = res_smem_limit<256, 32, false>()) != cudaSuccess ||
+      (e = res_smem_limit<128, 32, true>()) != cudaSuccess || (e = res_smem_limit<128, 32, false, 16>()) != cudaSuccess ||
+      (e = res_smem_limit<128, 32, true, 16>()) != cudaSuccess || (e = res_smem_limit<256, 32, false>()) != cudaSuccess ||
       (e = res_smem_limit<256, 32, true>()) != cudaSuccess || (e = res_smem_limit<256, 64, false>()) != cudaSuccess)
     return e;
   return res_smem_limit<256, 64, true>();
