@@ -1984,8 +1984,8 @@ struct ResRun {
   int base, width, pos, parts, nsteps;
 };
 
-// KMAX: column segments at most (ny / (NX / 8)).
-template <int NX, int NR, bool COMP, bool OBS, int KMAX>
+// KMAX: column segments (ny / (NX / 8)) at most, or exactly (FULL).
+template <int NX, int NR, bool COMP, bool OBS, int KMAX, bool FULL>
 __global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v, ResRun run) {
   constexpr int TH = 8 * NR;      // threads per CTA
   constexpr int S = NX / 16;      // row points per lane
@@ -2038,7 +2038,7 @@ __global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v
   }
   // column phase: column c, rows g SC .. g SC + SC - 1 of this CTA = segment gs of ns
   const int c = tid % NX, g = tid / NX;
-  const int ns = (int)Q * NSEG, gs = (int)rank * NSEG + g;
+  const int ns = FULL ? KMAX : (int)Q * NSEG, gs = (int)rank * NSEG + g;
   {
     const SegTable& tx = v.seg[m];
     const SegTable& ty = v.segy[m];
@@ -2650,6 +2650,8 @@ cudaError_t phase_impl(const DevView& v, int phase, const LaunchShape& sh, cudaS
 // how many such clusters the device holds at once.
 template <int NX, int NR, bool COMP, bool OBS, int KMAX = 8>
 cudaError_t res_launch(const DevView& v, const ResRun& run, int n, int Q, cudaStream_t st, int* cap) {
+  const auto kernel = !OBS && Q * (NR / (NX / 8)) == KMAX ? res_kernel<NX, NR, COMP, OBS, KMAX, !OBS>
+                                                           : res_kernel<NX, NR, COMP, OBS, KMAX, false>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(n * Q), 1, 1);
   cfg.blockDim = dim3(8 * NR, 1, 1);
@@ -2662,8 +2664,8 @@ cudaError_t res_launch(const DevView& v, const ResRun& run, int n, int Q, cudaSt
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cap) return cudaOccupancyMaxActiveClusters(cap, res_kernel<NX, NR, COMP, OBS, KMAX>, &cfg);
-  return cudaLaunchKernelEx(&cfg, res_kernel<NX, NR, COMP, OBS, KMAX>, v, run);
+  if (cap) return cudaOccupancyMaxActiveClusters(cap, kernel, &cfg);
+  return cudaLaunchKernelEx(&cfg, kernel, v, run);
 }
 
 template <bool OBS>
@@ -2718,9 +2720,12 @@ cudaError_t res_turns(const DevView& v, int ci, int n, int nsteps, int cap, cuda
 template <int NX, int NR, bool COMP, int KMAX = 8>
 cudaError_t res_smem_limit() {
   const int b = (int)res_smem_bytes(NX, NR, COMP);
-  cudaError_t e = cudaFuncSetAttribute(res_kernel<NX, NR, COMP, false, KMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(res_kernel<NX, NR, COMP, true, KMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  const auto limit = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(res_kernel<NX, NR, COMP, false, KMAX, false>, limit, b)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(res_kernel<NX, NR, COMP, false, KMAX, true>, limit, b)) != cudaSuccess)
+    return e;
+  return cudaFuncSetAttribute(res_kernel<NX, NR, COMP, true, KMAX, false>, limit, b);
 }
 
 template <typename T>
