@@ -248,9 +248,9 @@ chk::FxLimb fx_limb(double v) {
 // whose last one may be shorter (len points): A[d] = M^(S 2^d), P = M^len, B[l] = M^(S l) (I -
 // M^n)^-1 for segment l, B[32 + pos] = M^(distance of segment pos from the line's end) (I -
 // M^n)^-1, pos counted from the end.  False if an entry is too large for the scans' products (a
-// line short against the decay of M); t may be null.
-bool fx_tables(double p1, double p2, int S, int n, chk::SegTable* t, int* levels = nullptr) {
-  if (t) std::memset(t, 0, sizeof *t);
+// line short against the decay of M).
+bool fx_tables(double p1, double p2, int S, int n, chk::SegTable* t, int* levels) {
+  std::memset(t, 0, sizeof *t);
   const int G = (n + S - 1) / S, len = n - (G - 1) * S;
   const double M[4] = {p1, p2, 1.0, 0.0};
   double MS[4] = {1.0, 0.0, 0.0, 1.0}, ML[4] = {1.0, 0.0, 0.0, 1.0}, Mn[4] = {1.0, 0.0, 0.0, 1.0};
@@ -265,33 +265,31 @@ bool fx_tables(double p1, double p2, int S, int n, chk::SegTable* t, int* levels
     for (int i = 0; i < 4; ++i) {
       if (!(std::fabs(m[i]) < 15.0))
         ok = false;
-      else if (t)
-        to[i] = fx_limb(std::ldexp(m[i], 58));
+      else
+        to[i] = fx_limb(m[i] * 0x1p58);
     }
   };
-  chk::SegTable none;
-  chk::SegTable& T = t ? *t : none;
   double Ad[4] = {MS[0], MS[1], MS[2], MS[3]};
   int lv = 0;
   for (int q = 0; q < 5 && (1 << q) < G; ++q) {
     for (double x : Ad)
       if (std::fabs(x) >= 0x1p-62) lv = q + 1;
-    put(T.Ax[q], Ad);
+    put(t->Ax[q], Ad);
     mat2_mul(Ad, Ad, Ad);
   }
-  put(T.Px, ML);
+  put(t->Px, ML);
   double F[4] = {P[0], P[1], P[2], P[3]}, R[4];
   for (int l = 0; l < G; ++l) {
-    put(T.Bx[l], F);
+    put(t->Bx[l], F);
     mat2_mul(MS, F, F);
   }
-  put(T.Bx[32], P);
+  put(t->Bx[32], P);
   mat2_mul(ML, P, R);
   for (int pos = 1; pos < G; ++pos) {
-    put(T.Bx[32 + pos], R);
+    put(t->Bx[32 + pos], R);
     mat2_mul(MS, R, R);
   }
-  if (levels) *levels = lv;
+  *levels = lv;
   return ok;
 }
 
@@ -333,11 +331,12 @@ void fx_mu_params(MemberParams* p) {
 
 // The member's constants of the fixed-point form; false where it does not apply: lines of 16 to
 // 1024 points whose recurrences gain at most 2^9 (s up to about 1e5: above, 64 bits minus the
-// gain's headroom would hold less than FP64).
-bool fx_params(MemberParams* p) {
+// gain's headroom would hold less than FP64).  x, y: its scan tables, filled in where it applies.
+bool fx_params(MemberParams* p, chk::SegTable* x, chk::SegTable* y) {
   if (p->nx < 16 || p->ny < 16 || p->nx > 1024 || p->ny > 1024) return false;
   p->fx_gainx = fx_gain(p->p1x, p->p2x);
-  p->fx_gainy = fx_gain(p->p1y, p->p2y);
+  const bool alike = p->nx == p->ny && p->p1x == p->p1y && p->p2x == p->p2y;  // both directions
+  p->fx_gainy = alike ? p->fx_gainx : fx_gain(p->p1y, p->p2y);
   if (p->fx_gainx > 9 || p->fx_gainy > 9) return false;
   if (!p->fx_mu) return false;
   int er = 0;
@@ -360,13 +359,11 @@ bool fx_params(MemberParams* p) {
   p->fx_sy = sy;
   p->fx_cw = fx_panel(p->ny);
   p->fx_gwy = pow2(p->fx_gy);
-  return fx_tables(p->p1x, p->p2x, sx, p->nx, nullptr, &p->fx_lvx) &&
-         fx_tables(p->p1y, p->p2y, sy, p->ny, nullptr, &p->fx_lvy);
-}
-
-void fx_member_tables(const MemberParams& p, chk::SegTable* x, chk::SegTable* y) {
-  fx_tables(p.p1x, p.p2x, p.fx_sx, p.nx, x);
-  fx_tables(p.p1y, p.p2y, p.fx_sy, p.ny, y);
+  if (!fx_tables(p->p1x, p->p2x, sx, p->nx, x, &p->fx_lvx)) return false;
+  if (!alike || sx != sy) return fx_tables(p->p1y, p->p2y, sy, p->ny, y, &p->fx_lvy);
+  *y = *x;
+  p->fx_lvy = p->fx_lvx;
+  return true;
 }
 
 // Shared memory of the member's tiles into the launch shape (the largest of its class).
@@ -620,7 +617,7 @@ int build_tiles(ch_ensemble* h, const ch_tuning& t) {
   for (int k = 0; k < h->m; ++k) {
     if (!h->has(k)) continue;
     MemberParams& p = h->hp[k];
-    p.fx = fx_on && fx_params(&p) ? 1 + fx_class(p.nx) : 0;
+    p.fx = fx_on && fx_params(&p, &h->hseg[k], &h->hsegy[k]) ? 1 + fx_class(p.nx) : 0;
     if (resident(p) || p.fx) continue;
     if (t.row_seg == 1 && !split && !rowT_fits(p))
       return fail(CH_EINVAL, "row_seg 1: some member's nx is not 32 times at most 16");
@@ -672,7 +669,6 @@ int build_tiles(ch_ensemble* h, const ch_tuning& t) {
       p.kx32 = 0;
       p.rows_p = p.cols_p = 1;
       const int cr = fx_class(p.nx), br = std::min(p.ny, fx_band(p.nx)), cw = p.fx_cw;
-      fx_member_tables(p, &h->hseg[k], &h->hsegy[k]);
       fx_shape(p, &sh);
       int b = 0;
       for (int j0 = 0; j0 < p.ny; j0 += br, ++b) fxr[cr].push_back(Tile{k, j0, std::min(br, p.ny - j0), b, 0, 0});

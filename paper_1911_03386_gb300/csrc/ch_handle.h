@@ -115,8 +115,7 @@ int validate_desc(const ch_member_desc& d, int k);
 int fill_params(const ch_member_desc& d, int precision, MemberParams* p);
 // Fixed-point constants of a member after fill_params (false where the form does not apply), its
 // scan tables, row class, rows per band and shared memory; none of them uses the heap.
-bool fx_params(MemberParams* p);
-void fx_member_tables(const MemberParams& p, chk::SegTable* x, chk::SegTable* y);
+bool fx_params(MemberParams* p, chk::SegTable* x, chk::SegTable* y);
 int fx_class(int nx);
 int fx_band(int nx);
 void fx_shape(const MemberParams& p, chk::LaunchShape* sh);

@@ -85,10 +85,21 @@ struct MemberParams {
 // for the companion matrix M = [[p1, p2], [1, 0]] of the recurrence, 2x2 row-major:
 // A[d] = M^(S 2^d) (scan steps), B[l] = M^(S l) (start state of lane l from the periodic
 // start state), P = (I - M^nx)^-1 (periodic start state from the scan total).
+// A member of the fixed-point form (ch_fixed.cu) has Ax, Px and Bx in their place, with meanings of
+// their own (see fx_tables), entries / 64 times 2^64.
 struct SegTable {
-  double A[5][4];
-  double B[64][4];       // up to 64 segments: columns over a CTA pair (rows use at most 32)
-  double P[4];
+  union {
+    alignas(16) double A[5][4];
+    FxLimb Ax[5][4];
+  };
+  union {
+    double P[4];
+    FxLimb Px[4];
+  };
+  union {
+    double B[64][4];     // up to 64 segments: columns over a CTA pair (rows use at most 32)
+    FxLimb Bx[64][4];
+  };
   float Af[5][4];        // the same rounded to FP32
   float Bf[64][4];
   float Pf[4];
@@ -99,10 +110,6 @@ struct SegTable {
   // backward recurrences from zero states; g = G0 of the forward homogeneous responses,
   // k = the backward homogeneous responses).
   float Hf[32][4];
-  // Fixed-point form (ch_fixed.cu; its own meaning of the entries, see fx_tables), entries / 64
-  // times 2^64.
-  alignas(16) FxLimb Ax[5][4];
-  FxLimb Px[4], Bx[64][4];
 };
 
 struct MemberState {

@@ -83,7 +83,7 @@ __global__ void noalloc_fixed_setup(FixedSetup s, FixedTables* t, int band) {
 // nsteps steps of the fixed-point kernels; false where the form does not apply.
 bool step_fixed(double* C, double* W, const ch_member_desc& d, int64_t nsteps, cudaStream_t st, int* rc) {
   FixedSetup s;
-  if (chh::fill_params(d, CH_FP64, &s.mp) != CH_OK || !chh::fx_params(&s.mp)) return false;
+  if (chh::fill_params(d, CH_FP64, &s.mp) != CH_OK || !chh::fx_params(&s.mp, &s.seg, &s.segy)) return false;
   if (s.mp.fx_gainx > 6 || s.mp.fx_gainy > 6) return false;
   *rc = CH_ECUDA;
   FixedTables* t = nullptr;
@@ -93,7 +93,6 @@ bool step_fixed(double* C, double* W, const ch_member_desc& d, int64_t nsteps, c
   s.mp.every = INT_MAX;
   s.mp.fx = 1;
   s.mp.fx_wexp = 0;
-  chh::fx_member_tables(s.mp, &s.seg, &s.segy);
   const int band = std::min(d.ny, chh::fx_band(d.nx));
   chk::LaunchShape sh{};
   chh::fx_shape(s.mp, &sh);
