@@ -5,7 +5,7 @@ Workload (default): an ensemble of 256 independent periodic runs on 256x256 grid
 gamma = 0.005, dt = 1e-3, 20 000 steps (t = 20), members 0-127 at C0 = 0 and 128-255 at
 C0 = 0.4, uniform noise +-0.1, F / dF/dt / beta sampled every 100 steps and beta averaged
 over t >= 4, FP64.  One benchmark "step" is one sampling interval: 100 time steps of
-every member (stencil + row sweep, column sweep + update) including the sample.  The
+every member (rows, columns + update) including the sample.  The
 default --steps 200 therefore times the whole 20 000-step horizon.
 
 Reported:
@@ -15,7 +15,8 @@ Reported:
                  are uploaded from page-locked host memory and every step ends with a
                  device-to-host read of F, dF/dt, beta (ch_observables).
   fp32           the FP32 form on the same workload (throughput, <beta> against FP64).
-  roofline       the dominant kernel against its bound (FP64 pipe for the FP64 path).
+  roofline       the dominant kernel against its bound (integer multiply pipe for the FP64
+                 path's fixed-point form).
   ensemble_stats moments, histograms and trend statistics of beta across runs: kernel
                  times on a paper-size synthetic ensemble and the workload's own values.
   droplets       Model 1: 100 droplet populations of 512 to t = 40 (adaptive Dormand-Prince
@@ -64,11 +65,16 @@ HBM_PEAK, HBM_PEAK_SOURCE = _hbm_peak()
 #   resident (cluster-resident FP32 form) the whole step on chip: mu (9) + R' (6) + row
 #            recurrences (8) + column recurrences (8) + update (2) flop; the field crosses HBM
 #            once per launch (read and written: 2 words per point per launch, not per step)
-KERNEL_WORK = {"stencil": (15.0, 2), "rowsweep": (8.0, 2), "rows": (23.0, 2), "cols": (10.0, 3), "resident": (33.0, 0)}
+#   fx_rows, fx_cols: rows and cols of the fixed-point FP64 step (csrc/ch_fixed.cu)
+KERNEL_WORK = {"fx_rows": (23.0, 2), "fx_cols": (10.0, 3), "stencil": (15.0, 2), "rowsweep": (8.0, 2), "rows": (23.0, 2), "cols": (10.0, 3), "resident": (33.0, 0)}
 # The same work in FP64 pipe operations (an ADD or MUL takes a pipe slot like an FMA):
 #   stencil  mu 6 (3 FMA, 1 MUL, 2 ADD) + R' 4 (2 FMA, 2 ADD); rowsweep 4 (2 FMA per
 #   recurrence); cols 5 (4 FMA + the update FMA)
 KERNEL_OPS = {"stencil": 10.0, "rowsweep": 4.0, "rows": 14.0, "cols": 5.0}
+# The fixed-point kernels' 32 x 32 -> 64 bit multiply-adds per point: a recurrence step 6 (two
+# directions of two passes each: 24), a product of the stencil 3 (mu: three products)
+KERNEL_WIDE = {"fx_rows": 33.0, "fx_cols": 24.0}
+WIDE_PER_CLOCK = 32 / 1.27  # per SM and clock (measured: 1.27 SM clocks per warp instruction)
 
 
 # ------------------------------------------------------------------------------------------
@@ -193,7 +199,7 @@ def finite_or_none(x):
     return x
 
 
-STEP_SOURCES = ("ch_api.cu", "ch_internal.h", "ch_kernels.cu")  # the step's kernels and launch shapes
+STEP_SOURCES = ("ch_api.cu", "ch_device.cuh", "ch_fixed.cu", "ch_internal.h", "ch_kernels.cu")  # the step's kernels and launch shapes
 
 
 def kernel_source_hash():
@@ -225,7 +231,9 @@ def kernel_name(phase, t, elt, nx=256):
     """Kernel that runs a phase under tuning t (member 0's kernel classes)."""
     ty = "double" if elt == 8 else "float"
     if phase == "resident":
-        return "res_kernel<%d, %d, false, false>" % (nx, t.get("resident_rows") or 32)
+        return "res_kernel<%d, %d>" % (nx, t.get("resident_rows") or 32)
+    if phase in ("fx_rows", "fx_cols"):
+        return phase + "_kernel"
     if phase == "stencil":
         return "stencil_kernel<%s>" % ty
     if phase == "rowsweep":
@@ -288,10 +296,13 @@ def run_gpu_leg(ch, torch, p, prec, K, W, rank, world, dist, profile_kernels=Tru
     out = {"ms": ms, "pts": npts * K * STEPS_PER_BENCH_STEP, "clocks": clk.summary(), "beta_avg": avg,
            }
     out["tuning"] = e.tuning()
-    out["launches"] = K * STEPS_PER_BENCH_STEP * (3 if out["tuning"]["split"] else 2)
+    # FP64 members of 16 to 1024 points a side step in fixed point under the default tuning
+    fixed = prec == ch.CH_FP64 and 16 <= min(p["nx"], p["ny"]) and max(p["nx"], p["ny"]) <= 1024
+    out["launches"] = K * STEPS_PER_BENCH_STEP * (3 if out["tuning"]["split"] and not fixed else 2)
     if profile_kernels and out["tuning"]["resident"] == 1:
         # The cluster-resident form runs a sampling interval (100 steps) as one launch of its
-        # kernel: events around each launch, over 4 intervals after the timed region.
+        # kernel (where members take turns in its last wave, several: not counted): events around
+        # each interval, over 4 intervals after the timed region.
         out["launches"] = K
         reps = 4
         evs = [torch.cuda.Event(enable_timing=True) for _ in range(reps + 1)]
@@ -307,7 +318,7 @@ def run_gpu_leg(ch, torch, p, prec, K, W, rank, world, dist, profile_kernels=Tru
         # Per-kernel durations: events around each phase launch on the engine's stream,
         # over 2 sampling intervals of the same state after the timed region.
         split = out["tuning"]["split"]
-        names = ["stencil", "rowsweep", "cols"] if split else ["rows", None, "cols"]
+        names = ["fx_rows", None, "fx_cols"] if fixed else ["stencil", "rowsweep", "cols"] if split else ["rows", None, "cols"]
         reps = 2 * STEPS_PER_BENCH_STEP
         evs = [torch.cuda.Event(enable_timing=True) for _ in range(4 * reps)]
         for r in range(reps):
@@ -578,12 +589,14 @@ def value_estimate(res):
 # precision (resident32: FP32 and 32 members):
 #   resident32  FP32, cluster-resident form, 32 members of the 256 x 256 ensemble (one wave
 #               of clusters): one res_kernel launch per 100 steps
-#   stream64    FP64 split form, the whole 256-member ensemble (256 MB, above the L2):
-#               stencil_kernel, rowstream_kernel, colstream_kernel per step
+#   fixed64     FP64 in fixed point (the default), the whole 256-member ensemble (256 MB, above
+#               the L2): fx_rows_kernel, fx_cols_kernel per step
+#   stream64    the same in the FP64 split form: stencil_kernel, rowstream_kernel,
+#               colstream_kernel per step
 #   segment32   FP32 with the resident form off, the whole ensemble (134 MB):
 #               rows_seg_kernel, colseg_kernel per step
 # name: (precision, ch_tuning.resident, members, workload)
-KERNEL_CASES = {"resident32": ("fp32", 0, 32, "ensemble"), "stream64": ("fp64", -1, 256, "ensemble"),
+KERNEL_CASES = {"resident32": ("fp32", 0, 32, "ensemble"), "fixed64": ("fp64", 0, 256, "ensemble"), "stream64": ("fp64", -1, 256, "ensemble"),
                 "segment32": ("fp32", -1, 256, "ensemble"), "long16": ("fp32", -1, 16, "long")}
 
 
@@ -599,7 +612,7 @@ def kernel_case(name):
     descs = [dict(nx=p["nx"], ny=p["ny"], L=p["L"], gamma=p["gamma"], dt=p["dt"], C0=p["C0"][stride * k],
                   seed=wl.BASE_SEED, counter_base=k * p["nx"] * p["ny"]) for k in range(members)]
     with ch.Ensemble.batch(descs, ch.CH_FP32 if prec == "fp32" else ch.CH_FP64) as e:
-        e.set_tuning(resident=res)
+        e.set_tuning(resident=res, **({"split": 1} if name == "stream64" else {}))
         stream = torch.cuda.Stream()
         e.set_stream(stream.cuda_stream)
         # sampling every 100 steps; the 1024^2 workload averages over the last 80 % of its horizon
@@ -867,7 +880,21 @@ def main():
         per_launch = {k: {"ms": v, "achieved_tflops": KERNEL_WORK[k][0] * npts / (v * 1e-3) / 1e12,
                           "achieved_gbs": KERNEL_WORK[k][1] * elt * npts / (v * 1e-3) / 1e9} for k, v in ks.items()}
         step_ms = sum(ks.values())
-        if bound == "alu":
+        if dom in KERNEL_WIDE:
+            # the integer multiply pipe: the wide multiply-adds that the arithmetic takes against
+            # the measured rate of the instruction
+            sms = peaks["sms"] if peaks is not None else 152
+            mhz = (res.get("clocks") or {}).get("sm_mhz") or 2070.0
+            ach, pk = KERNEL_WIDE[dom] * npts / (ks[dom] * 1e-3), sms * WIDE_PER_CLOCK * mhz * 1e6
+            rl = {"bound": "alu", "kernel": tname, "achieved": ach / 1e12, "peak": pk / 1e12,
+                  "unit": "T wide multiply-adds/s (32 x 32 -> 64 bit)", "frac": ach / pk,
+                  "peak_source": "derived: %d SMs x 25.2 per clock (measured rate of the instruction) x %.0f MHz "
+                                 "(median SM clock of the timed region)" % (sms, mhz),
+                  "wide_ops_per_point": KERNEL_WIDE[dom],
+                  "achieved_flop_tflops": flops * npts / (ks[dom] * 1e-3) / 1e12}
+            if peaks is not None:
+                rl["probe_fp64_fma_tflops"] = peaks["fp64"]["tflops"]
+        elif bound == "alu":
             # the FP64 pipe issues an ADD or MUL in a slot an FMA would take: achieved is
             # counted in FMA-equivalent flops (2 per pipe operation) against the measured FMA
             # rate, i.e. the fraction of pipe slots the kernel's minimal operations fill; the
@@ -906,7 +933,7 @@ def main():
 
     def resident_roofline(res, tname, step_ms, elt):
         # The cluster-resident kernel keeps the field on chip: its bound is the SM (FP32
-        # issue and shared-memory latency), so it is stated against the measured FP32 FMA
+        # issue and the latencies of shared memory), so it is stated against the measured FP32 FMA
         # rate with its minimal 33 flop per point and step.  Beside it: the HBM rate a
         # streaming step would need for the same throughput at the 16 B per point minimum
         # of any factorised ADI step, and the traffic it actually needs (one read and one

@@ -361,18 +361,18 @@ int ch_seg_tables(double s, int seg, int groups, double* out);
  * allocation's synchronisation and latency after start-up, and processes whose device
  * memory budget is fixed at start.  The call allocates no device memory (on success it
  * touches no host heap either): its one intermediate, the row-solve result W, lives in a
- * static device array of 1,048,576 doubles (8 MiB) that every GPU loading libch holds
- * until the process exits.  So nx*ny must be <= 1,048,576 (e.g. 1024 x 1024); larger
+ * static device array of 1,048,576 doubles (8 MiB), and its tables in another of under
+ * 64 KiB, that every GPU loading libch holds until the process exits.  So nx*ny must be <= 1,048,576 (e.g. 1024 x 1024); larger
  * grids are rejected with CH_EINVAL and a message in ch_last_error().
  *
  * Every call looks up the array's device address in the current context
  * (cudaGetSymbolAddress, which allocates nothing) and sets the kernels' shared-memory
  * limits, so a device reset or a switch to another context between calls is safe.  The
  * first call on a device also loads the library's kernels there: make it before any
- * stream capture on that device.  All calls on a device share the array, which keeps
- * the last call's contents; every step overwrites all of W before reading it, so
- * nothing needs clearing.  Calls whose work overlaps on the GPU (other streams, other
- * host threads) race on the array: serialise them.
+ * stream capture on that device.  All calls on a device share the arrays, which keep
+ * the last call's contents; every call writes its tables and every step all of W before
+ * reading them, so nothing needs clearing.  Calls whose work overlaps on the GPU (other streams, other
+ * host threads) race on the arrays: serialise them.
  * Errors: CH_EINVAL (NULL C, nx or ny < 5, nx*ny above the limit, L/gamma/dt not finite
  * and > 0, nsteps < 0), CH_ECUDA (set-up or launch failed).  Launch errors are read
  * without clearing the CUDA error state, so an error the caller left pending also gives

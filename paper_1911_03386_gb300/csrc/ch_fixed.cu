@@ -11,9 +11,9 @@
 //                    integers, one exponent per row)
 //   fx_cols_kernel   a panel of up to 32 columns: both column recurrences of W, C += kappa Z
 //
-// Measured (us per step of a whole ensemble, the FP64 kernels before): 256 x 256^2 rows 207 +
-// columns 164 = 0.362 ms (stencil 0.334 + rows 0.196 + columns 0.241 = 0.762 ms); 16 x 1024^2
-// 0.432 ms (1.43 ms); 64^2 alone 20 us (70 us).  At 256^2 a point takes about 290 instructions of
+// Measured (us per step of a whole ensemble, the FP64 kernels before): 256 x 256^2 rows 219 +
+// columns 136 = 0.347 ms (stencil 0.334 + rows 0.196 + columns 0.241 = 0.762 ms); 16 x 1024^2
+// 0.406 ms (1.43 ms); 64^2 alone 14.6 us (70 us).  At 256^2 a point takes about 290 instructions of
 // the row kernel and 170 of the column kernel; both are bound by issue slots and the integer
 // multiply pipe (56 % and 44 % of the issue slots used), not by HBM (40 bytes per point, 0.1 ms).
 //

@@ -1751,9 +1751,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(sizeof(T) == 4 ? 102
 //           t_k over s_{k+1}).  Every CTA computes the same s_k, t_k with the same
 //           operations, so it updates its halo rows -- its neighbours' boundary rows --
 //           itself, bit for bit as the neighbours update them: no halo exchange.
-// Bound by the latencies and wavefronts of shared memory: the walks and the adjacent rows, which
-// change only what is read how often, took 256 x 256^2 from 59.2 to 55.8 us per step and 32 x 256^2
-// from 8.2 to 7.7.
+// Bound by latencies: shared memory, the cluster barrier, the serial chains.  us per step of
+// 256 x 256^2 / 32 x 256^2 / 256 x 128^2: 59.2 / 8.2 / 24.7; with the walks and the adjacent rows
+// 55.8 / 7.7 / 24.5; turns in the last wave (res_turns) 54.6 / 7.7 / 22.5; two FP32 values per
+// instruction 53.5 / 7.6 / 22.5; the combination in two serial walks instead of four 51.1 / 7.2 /
+// 22.3; built for the column segments there are (KMAX, FULL) 48.2 / 6.8 / 16.8.
 // The end states are double-buffered by step parity (a CTA may start the next step while
 // others still read this step's).  Sample steps add the FP64 partial sums of the F and
 // dF/dt densities (mu recomputed in FP64 from the stored field, as in the other FP32
