@@ -173,7 +173,9 @@ __device__ __forceinline__ void load_tab(ScanTab& t, const SegTable& g) {
 
 // Programmatic dependent launch: a step kernel lets its successor start (its CTAs take the SMs'
 // free slots, read their constant tables and wait) and waits itself until its predecessor has
-// finished and its writes are visible.  64^2 alone: 20.2 us per step without it, 16.5 with it.
+// finished and its writes are visible.  What is read before the wait -- the tiles and the scan
+// tables -- must therefore not come from the predecessor (tables_ready, launch_fx_rows).  64^2 alone:
+// 20.2 us per step without it, 16.5 with it.
 __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;\n" ::: "memory");
 }
@@ -685,7 +687,7 @@ cudaError_t rows_limit() {
 constexpr int kDependentCtas = 152;
 
 template <class K>
-void launch_dependent(K kernel, int grid, int block, size_t smem, cudaStream_t st, const DevView& v, int base) {
+void launch_dependent(K kernel, int grid, int block, size_t smem, cudaStream_t st, const DevView& v, int base, bool ready) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
   cfg.blockDim = dim3((unsigned)block, 1, 1);
@@ -695,11 +697,11 @@ void launch_dependent(K kernel, int grid, int block, size_t smem, cudaStream_t s
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = grid <= kDependentCtas ? 1 : 0;
+  cfg.numAttrs = ready && grid <= kDependentCtas ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, v, base);
 }
 
-cudaError_t launch_fx_rows(const DevView& v, const LaunchShape& sh, cudaStream_t st) {
+cudaError_t launch_fx_rows(const DevView& v, const LaunchShape& sh, cudaStream_t st, bool tables_ready) {
   int base = sh.n_row_tiles;
   const int* n = sh.fx_rt;
   const size_t* sm = sh.fx_smem;
@@ -708,27 +710,27 @@ cudaError_t launch_fx_rows(const DevView& v, const LaunchShape& sh, cudaStream_t
   // (a burst of 24 requests of 64^2 to 256^2 takes 35.2 ms in separate launches, 24.2 ms in one).
   if ((n[0] > 0) + (n[1] > 0) + (n[2] > 0) > 1) {
     const int all = n[0] + n[1] + n[2];
-    launch_dependent(fx_rows_kernel<256, 4>, all, 256, max(sm[0], max(sm[1], sm[2])), st, v, base);
+    launch_dependent(fx_rows_kernel<256, 4>, all, 256, max(sm[0], max(sm[1], sm[2])), st, v, base, tables_ready);
     base += all;
-    if (n[3] > 0) launch_dependent(fx_rows_kernel<256, 2>, n[3], 256, sm[3], st, v, base);
+    if (n[3] > 0) launch_dependent(fx_rows_kernel<256, 2>, n[3], 256, sm[3], st, v, base, tables_ready);
     return cudaPeekAtLastError();
   }
   // few tiles: larger CTAs (a sample's sums then take 8 warps instead of 2 or 4)
   if (n[0] + n[1] > 0 && n[0] + n[1] <= kDependentCtas) {
-    launch_dependent(fx_rows_kernel<256, 4>, n[0] + n[1], 256, max(sm[0], sm[1]), st, v, base);
+    launch_dependent(fx_rows_kernel<256, 4>, n[0] + n[1], 256, max(sm[0], sm[1]), st, v, base, tables_ready);
     base += n[0] + n[1];
-    if (n[2] > 0) launch_dependent(fx_rows_kernel<256, 4>, n[2], 256, sm[2], st, v, base);
+    if (n[2] > 0) launch_dependent(fx_rows_kernel<256, 4>, n[2], 256, sm[2], st, v, base, tables_ready);
     base += n[2];
-    if (n[3] > 0) launch_dependent(fx_rows_kernel<256, 2>, n[3], 256, sm[3], st, v, base);
+    if (n[3] > 0) launch_dependent(fx_rows_kernel<256, 2>, n[3], 256, sm[3], st, v, base, tables_ready);
     return cudaPeekAtLastError();
   }
-  if (n[0] > 0) launch_dependent(fx_rows_kernel<64, 14>, n[0], 64, sm[0], st, v, base);
+  if (n[0] > 0) launch_dependent(fx_rows_kernel<64, 14>, n[0], 64, sm[0], st, v, base, tables_ready);
   base += n[0];
-  if (n[1] > 0) launch_dependent(fx_rows_kernel<128, 7>, n[1], 128, sm[1], st, v, base);
+  if (n[1] > 0) launch_dependent(fx_rows_kernel<128, 7>, n[1], 128, sm[1], st, v, base, tables_ready);
   base += n[1];
-  if (n[2] > 0) launch_dependent(fx_rows_kernel<256, 4>, n[2], 256, sm[2], st, v, base);
+  if (n[2] > 0) launch_dependent(fx_rows_kernel<256, 4>, n[2], 256, sm[2], st, v, base, tables_ready);
   base += n[2];
-  if (n[3] > 0) launch_dependent(fx_rows_kernel<256, 2>, n[3], 256, sm[3], st, v, base);
+  if (n[3] > 0) launch_dependent(fx_rows_kernel<256, 2>, n[3], 256, sm[3], st, v, base, tables_ready);
   return cudaPeekAtLastError();
 }
 
@@ -737,9 +739,9 @@ cudaError_t launch_fx_observe(const DevView& v, const LaunchShape& sh, cudaStrea
   return cudaGetLastError();
 }
 
-cudaError_t launch_fx_cols(const DevView& v, const LaunchShape& sh, cudaStream_t st) {
+cudaError_t launch_fx_cols(const DevView& v, const LaunchShape& sh, cudaStream_t st, bool tables_ready) {
   const int base = sh.cst_n[0] + sh.cst_n[1] + sh.cst_n[2] + sh.cst_n[3];
-  if (sh.fx_ct > 0) launch_dependent(fx_cols_kernel, sh.fx_ct, kColThreads, sh.fx_cols_smem, st, v, base);
+  if (sh.fx_ct > 0) launch_dependent(fx_cols_kernel, sh.fx_ct, kColThreads, sh.fx_cols_smem, st, v, base, tables_ready);
   return cudaPeekAtLastError();
 }
 

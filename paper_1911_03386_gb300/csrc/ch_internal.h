@@ -253,9 +253,11 @@ size_t walk_smem_bytes(int nr, int nx, int S);
 size_t resident_smem_bytes(int nx, int nr, int comp);
 cudaError_t set_kernel_smem_limits(int precision);
 // Fixed-point form (ch_fixed.cu): the row and column phases (launch errors are read without
-// clearing them) and the observables' partials.
-cudaError_t launch_fx_rows(const DevView& v, const LaunchShape& sh, cudaStream_t st);
-cudaError_t launch_fx_cols(const DevView& v, const LaunchShape& sh, cudaStream_t st);
+// clearing them) and the observables' partials.  tables_ready: the member's tiles and scan tables
+// were written by work that the stream has already waited for in full (host copies); false makes the
+// launches wait for all earlier work of the stream before any of their CTAs starts.
+cudaError_t launch_fx_rows(const DevView& v, const LaunchShape& sh, cudaStream_t st, bool tables_ready = true);
+cudaError_t launch_fx_cols(const DevView& v, const LaunchShape& sh, cudaStream_t st, bool tables_ready = true);
 cudaError_t launch_fx_observe(const DevView& v, const LaunchShape& sh, cudaStream_t st);
 cudaError_t set_fx_smem_limits();
 size_t fx_rows_smem(int nr, int nx, int S);

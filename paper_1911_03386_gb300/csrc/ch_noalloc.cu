@@ -112,8 +112,11 @@ bool step_fixed(double* C, double* W, const ch_member_desc& d, int64_t nsteps, c
   v.m = 1;
   if (nsteps > 0) noalloc_fixed_setup<<<1, 128, 0, st>>>(s, t, band);
   if (cudaPeekAtLastError() != cudaSuccess) return true;
+  // The step kernels read their tiles and tables before they wait for their predecessor, so the
+  // first step, which follows the kernel that writes those tables, is launched in plain stream order.
   for (int64_t k = 0; k < nsteps; ++k)
-    if (chk::launch_fx_rows(v, sh, st) != cudaSuccess || chk::launch_fx_cols(v, sh, st) != cudaSuccess) return true;
+    if (chk::launch_fx_rows(v, sh, st, k > 0) != cudaSuccess || chk::launch_fx_cols(v, sh, st, k > 0) != cudaSuccess)
+      return true;
   *rc = CH_OK;
   return true;
 }
