@@ -318,9 +318,15 @@ int fx_panel(int ny) { return ny <= 256 ? 32 : ny <= 512 ? 16 : 8; }
 // Constants of mu in fixed point (any member whose stencil coefficients fit).
 void fx_mu_params(MemberParams* p) {
   p->fx_square = p->hx == p->hy;
-  // |C| < 2^E: |mu| / 2^E <= 3 + 4 (bx + by) for E <= 1 and |R'| <= 4 (1 + rho) |mu|, which has
-  // to fit 62 bits (60 where R' takes a product with rho)
-  const double bound = 4.0 * (1.0 + p->rho) * (3.0 + 4.0 * (p->bx + p->by));
+  p->fx_tall = p->hy < p->hx;
+  p->fx_ratio = p->fx_tall ? (p->hy * p->hy) / (p->hx * p->hx) : p->rho;
+  p->fx_w0 = -2.0 * (1.0 + p->fx_ratio);
+  p->fx_kappa = p->fx_tall ? p->dt / (p->hy * p->hy * p->cx * p->cy) : p->kappa;
+  // |C| < 2^E: |mu| / 2^E <= 3 + 4 (bx + by) for E <= 1 and |R'| <= 4 (1 + ratio) |mu|, which has
+  // to fit 62 bits (60 where R' takes a product).  The ratio is at most 1 whatever the grid: with
+  // rho = (hx / hy)^2 in its place a tall grid's headroom came out of mu (17 x 600: 39 bits of mu and
+  // 94 times the FP64 kernels' error on a separated field).
+  const double bound = 4.0 * (1.0 + p->fx_ratio) * (3.0 + 4.0 * (p->bx + p->by));
   p->fx_mu = std::isfinite(bound) && bound < 1e9;
   if (!p->fx_mu) return;
   p->fx_kmu = std::min(55, (p->fx_square ? 62 : 60) - (int)std::ceil(std::log2(bound)));
@@ -340,10 +346,9 @@ bool fx_params(MemberParams* p, chk::SegTable* x, chk::SegTable* y) {
   if (p->fx_gainx > 9 || p->fx_gainy > 9) return false;
   if (!p->fx_mu) return false;
   int er = 0;
-  if (std::frexp(p->rho, &er) > 1.0 - 1e-9) ++er;  // rho < 2^er, not by rounding alone
+  if (std::frexp(p->fx_ratio, &er) > 1.0 - 1e-9) ++er;  // ratio < 2^er, not by rounding alone
   p->fx_er = std::max(0, er + 1);
-  if (p->fx_er > 40) return false;
-  p->fx_rho = fx_limb(std::ldexp(p->rho, 64 - p->fx_er));
+  p->fx_rl = fx_limb(std::ldexp(p->fx_ratio, 64 - p->fx_er));
   p->fx_cx = chk::FxCoef{fx_limb(std::ldexp(p->p1x, 61)), fx_limb(std::ldexp(p->p2x, 61))};
   p->fx_cy = chk::FxCoef{fx_limb(std::ldexp(p->p1y, 61)), fx_limb(std::ldexp(p->p2y, 61))};
   auto pow2 = [](int g) {
@@ -1496,7 +1501,8 @@ int ch_debug_row_solve(ch_handle h, int member, double* out) {
   CH_CUDA(chk::launch_phase(h->view(), h->precision, 1, h->shape, h->stream), "row phase");
   const MemberParams& p = h->hp[member];
   const int64_t np = (int64_t)p.nx * p.ny;
-  const double scale = p.dt / (p.hx * p.hx * p.cx);
+  const double h2 = p.fx && p.fx_tall ? p.hy * p.hy : p.hx * p.hx;
+  const double scale = p.dt / (h2 * p.cx);
   if (h->precision == CH_FP64) {
     if (int rc = copy_out(h, out, static_cast<double*>(h->W) + p.offset, sizeof(double) * np, "read W")) return rc;
     if (p.fx) {  // 64-bit integers with an exponent per row (rows held in FP64: as they are)

@@ -236,22 +236,29 @@ struct MuFp {
     return double_bits(fma(-by, s + n, fma(-bx, e + w, c * fma(c, c, -a))));
   }
 };
-// R' at m with neighbours e, w, n, s (SQ: hx = hy, exact).
-template <bool SQ>
+// R' at m with neighbours e, w, n, s, in units of the closer spacing (FORM 0: hx = hy, exact; 1: hx <
+// hy, dx + ratio dy; 2: hx > hy, ratio dx + dy).  The product's rounding is the one rounding in R'
+// that no difference damps afterwards, so forms 1 and 2 first move the differences up by the `up`
+// bits that the band's largest |mu| leaves free (mu of a smooth field is far below the bound that
+// sets its unit).
+template <int FORM>
 struct RhsFx {
-  FxLimb rho;
-  int er;
+  FxLimb ratio;
+  int er, up = 0;
   __device__ __forceinline__ i64 operator()(i64 m, i64 e, i64 w, i64 n, i64 s) const {
     const i64 dx = e + w - 2 * m, dy = n + s - 2 * m;
-    return SQ ? dx + dy : dx + mul_top(limbs(dy << er), rho);
+    if (FORM == 0) return dx + dy;
+    const i64 d = FORM == 1 ? dx : dy, q = FORM == 1 ? dy : dx;
+    return (d << up) + mul_top(limbs(q << (er + up)), ratio);
   }
 };
 struct RhsFp {
-  double rho, w0;
+  bool tall;
+  double ratio, w0;
   __device__ __forceinline__ i64 operator()(i64 m_, i64 e_, i64 w_, i64 n_, i64 s_) const {
     const double m = __longlong_as_double(m_), e = __longlong_as_double(e_), w = __longlong_as_double(w_),
                  n = __longlong_as_double(n_), s = __longlong_as_double(s_);
-    return double_bits(fma(w0, m, fma(rho, s + n, e + w)));
+    return double_bits(fma(w0, m, tall ? fma(ratio, e + w, s + n) : fma(ratio, s + n, e + w)));
   }
 };
 
@@ -304,26 +311,6 @@ __device__ __forceinline__ void walk_strips(const Band& b, int rows, const i64* 
   }
 }
 
-// mu, then R' (with the OR of its magnitudes in top), over the tile.
-template <bool FIXED, class Mu, class Rhs>
-__device__ __forceinline__ void band_rhs(const Band& b, i64* Es, i64* Em, unsigned& top, int emax, const Mu& mu,
-                                         const Rhs& rhs) {
-  walk_strips(
-      b, b.nr + 2, Es, [emax](i64 c) { return FIXED ? to_fixed(c, emax) : c; }, mu,
-      [&](i64 m, int s, int r, int lane, int last) {
-        if (lane == 0) Em[edge_index(b.nr + 2, s, 0) + r] = m;
-        if (lane == last) Em[edge_index(b.nr + 2, s, 1) + r] = m;
-      });
-  __syncthreads();
-  top = 0;
-  walk_strips(
-      b, b.nr, Em, [](i64 m) { return m; }, rhs,
-      [&](i64 m, int, int, int lane, int last) {
-        const int h = (int)(m >> 32);
-        if (FIXED && lane <= last) top |= (unsigned)(h ^ (h >> 31));
-      });
-}
-
 // OR of `top` over the CTA (slots: one per warp, not in use; ends with every thread past it).
 template <int NW>
 __device__ __forceinline__ unsigned cta_or(unsigned top, unsigned* slots) {
@@ -332,6 +319,37 @@ __device__ __forceinline__ unsigned cta_or(unsigned top, unsigned* slots) {
   if (lane == 0) slots[threadIdx.x >> 5] = top;
   __syncthreads();
   return __reduce_or_sync(kAll, lane < NW ? slots[lane] : 0u);
+}
+
+// mu, then R' (with the OR of its magnitudes in top), over the tile.  FORM: of RhsFx, or -1 in FP64;
+// slots: one word per warp, not in use.
+template <int NW, int FORM, class Mu, class Rhs>
+__device__ __forceinline__ void band_rhs(const Band& b, i64* Es, i64* Em, unsigned& top, int emax, const Mu& mu, Rhs& rhs,
+                                         unsigned* slots) {
+  constexpr bool FIXED = FORM >= 0;
+  const auto magnitude = [](i64 m) {
+    const int h = (int)(m >> 32);
+    return (unsigned)(h ^ (h >> 31));
+  };
+  top = 0;
+  walk_strips(
+      b, b.nr + 2, Es, [emax](i64 c) { return FIXED ? to_fixed(c, emax) : c; }, mu,
+      [&](i64 m, int s, int r, int lane, int last) {
+        if (lane == 0) Em[edge_index(b.nr + 2, s, 0) + r] = m;
+        if (lane == last) Em[edge_index(b.nr + 2, s, 1) + r] = m;
+        if (FORM > 0 && lane <= last) top |= magnitude(m);
+      });
+  // a difference is at most 4 |mu|: below 2^62 moved up by er + up, R' (twice that) below 2^62 by up
+  if constexpr (FORM > 0)
+    rhs.up = max(0, 60 - max(rhs.er, 1) - bit_length_hi(cta_or<NW>(top, slots)));
+  else
+    __syncthreads();
+  top = 0;
+  walk_strips(
+      b, b.nr, Em, [](i64 m) { return m; }, rhs,
+      [&](i64 m, int, int, int lane, int last) {
+        if (FIXED && lane <= last) top |= magnitude(m);
+      });
 }
 
 // Both recurrences of a row: segment seg (len points) of lane l of gw, G of them in use; top: OR of
@@ -360,7 +378,7 @@ __device__ __forceinline__ void row_solve(i64* seg, int len, int l, int G, int g
 template <int TH, int MINB>
 __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_base) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ unsigned wtop[4 * (TH / 32)];
+  __shared__ unsigned wtop[5 * (TH / 32)];
   const Tile tl = v.row_tiles[tile_base + blockIdx.x];
   const MemberParams& P = v.mp[tl.member];
   MemberState* st = v.ms + tl.member;
@@ -425,17 +443,26 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
     Es[k] = bad ? c : to_fixed(c, emax);
   }
   __syncthreads();
-  if (bad)
-    band_rhs<false>(b, Es, Em, top, emax, MuFp{P.a, P.bx, P.by}, RhsFp{P.rho, P.w0});
-  else
+  int up = 0;  // R' is held times 2^(kmu + up - E)
+  if (bad) {
+    RhsFp rhs{P.fx_tall != 0, P.fx_ratio, P.fx_w0};
+    band_rhs<NW, -1>(b, Es, Em, top, emax, MuFp{P.a, P.bx, P.by}, rhs, wtop + 4 * NW);
+  } else
     with_shift(2 * (emax - 1022) + 6 - P.fx_su, [&](auto sh) {
       const i64 one = 1ll << (60 - P.fx_su);
+      auto fixed = [&](auto mu, auto rhs, auto form) {
+        band_rhs<NW, decltype(form)::value>(b, Es, Em, top, emax, mu, rhs, wtop + 4 * NW);
+        up = rhs.up;
+      };
       if (P.fx_square)
-        band_rhs<true>(b, Es, Em, top, emax, MuFx<true, decltype(sh)>{P.fx_bx, P.fx_by, one, sh},
-                       RhsFx<true>{P.fx_rho, P.fx_er});
+        fixed(MuFx<true, decltype(sh)>{P.fx_bx, P.fx_by, one, sh}, RhsFx<0>{P.fx_rl, P.fx_er},
+              std::integral_constant<int, 0>());
+      else if (!P.fx_tall)
+        fixed(MuFx<false, decltype(sh)>{P.fx_bx, P.fx_by, one, sh}, RhsFx<1>{P.fx_rl, P.fx_er},
+              std::integral_constant<int, 1>());
       else
-        band_rhs<true>(b, Es, Em, top, emax, MuFx<false, decltype(sh)>{P.fx_bx, P.fx_by, one, sh},
-                       RhsFx<false>{P.fx_rho, P.fx_er});
+        fixed(MuFx<false, decltype(sh)>{P.fx_bx, P.fx_by, one, sh}, RhsFx<2>{P.fx_rl, P.fx_er},
+              std::integral_constant<int, 2>());
     });
   if (sample)
     band_partials_field<double>(v, tl, nx, nr, P, v.partials + P.partial_base + tl.index, red);
@@ -451,7 +478,7 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
   else
     row_solve<NW>(seg, len, l, G, gw, P.fx_lvx, full, Fx(P.fx_cx, 0.0, 0.0), tab, P.fx_gainx, top, wtop + NW, e_lsb, e_top);
   if (row < nr && l == 0) {
-    const int eb = emax - 1022 - P.fx_kmu;
+    const int eb = emax - 1022 - P.fx_kmu - up;
     v.wexp[P.fx_wexp + j0 + row] = bad ? make_short2(0, kBadRow) : make_short2((short)(e_lsb + eb), (short)(e_top + eb));
   }
   // W to HBM as whole rows (row_solve ends with a barrier)
@@ -662,14 +689,14 @@ __global__ void __launch_bounds__(kColThreads, 3) fx_cols_kernel(DevView v, int 
       f([e](i64 w) { return e.y == kBadRow ? w : double_bits(ldexp((double)w, e.x)); });
     });
     col_solve(ar, y, len, tab, xs, wtop, G, gw, P.fx_lvy, ny % S == 0, cw, 0, a, b);
-    col_update(ar, ye, len, Ce, nx, P.kappa, cv, a, b, [](i64 t) { return __longlong_as_double(t); });
+    col_update(ar, ye, len, Ce, nx, P.fx_kappa, cv, a, b, [](i64 t) { return __longlong_as_double(t); });
   } else {
     Fx ar(P.fx_cy, 0.0, 0.0);
     FxLimb a, b;
     const int up = 62 - gain - emax;
     col_first(ar, y, len, S, ws, a, b, [up](short2 e, auto f) { with_shift(max(-62, min(62, up + (int)e.x)), f); });
     const int sl = col_solve(ar, y, len, tab, xs, wtop, G, gw, P.fx_lvy, ny % S == 0, cw, gain, a, b);
-    col_update(ar, ye, len, Ce, nx, P.kappa * ldexp(1.0, -up - sl), cv, a, b, [](i64 t) { return (double)t; });
+    col_update(ar, ye, len, Ce, nx, P.fx_kappa * ldexp(1.0, -up - sl), cv, a, b, [](i64 t) { return (double)t; });
   }
   if (tl.index == 0 && threadIdx.x == 0) finalize_sample(v, tl.member, st, P);
 }

@@ -75,9 +75,12 @@ struct MemberParams {
   int fx_gainx, fx_gainy;            // log2 bound of the recurrences' gain
   int fx_mu;                         // kmu, su, bx, by are set (any precision: the observables' sums)
   int fx_kmu, fx_su;                 // mu is held times 2^(kmu - E); su = 55 - kmu
-  int fx_er, fx_square;              // rho product: dy << er; square: hx = hy
+  // R' of the fixed-point form, from the second differences dx, dy of mu: dx + ratio dy, or where
+  // hy < hx ratio dx + dy (1 / rho times the other form's; kappa times rho), so ratio <= 1
+  int fx_er, fx_square, fx_tall;     // ratio product: d << er; square: hx = hy; tall: hy < hx
+  double fx_ratio, fx_w0, fx_kappa;  // w0 = -2 (1 + ratio)
   FxCoef fx_cx, fx_cy;
-  FxLimb fx_bx, fx_by, fx_rho;       // bx, by times 2^(kmu + 5); rho times 2^(64 - er)
+  FxLimb fx_bx, fx_by, fx_rl;        // bx, by times 2^(kmu + 5); ratio times 2^(64 - er)
   int64_t fx_wexp;                   // first row exponent in DevView::wexp
 };
 

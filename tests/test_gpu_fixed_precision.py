@@ -1,0 +1,120 @@
+"""Precision of the fixed-point form of the CH_FP64 step (csrc/ch_fixed.cu): its error and that of
+the FP64 kernels (tuning split = 1), both against the same steps in extended precision (numpy
+longdouble, at least 64 significant bits), on grids of every aspect ratio.
+
+Tolerances: the form has to be no less precise than the FP64 kernels.  Both errors are sums of many
+roundings of about the same size, so the root mean squares over a field agree to a few per cent and
+the largest ones to a factor of two: 1.25 and 2 times the FP64 kernels' error.
+"""
+import math
+
+import numpy as np
+import pytest
+
+import paper_1911_03386_gb300 as ch
+
+pytestmark = pytest.mark.gpu
+
+TWO_PI = 2 * math.pi
+LD = np.longdouble
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+
+    __graft_entry__.build()
+
+
+def laplacian(f, hx, hy):
+    return ((np.roll(f, -1, 1) - 2 * f + np.roll(f, 1, 1)) / hx ** 2
+            + (np.roll(f, -1, 0) - 2 * f + np.roll(f, 1, 0)) / hy ** 2)
+
+
+def solve_rows(R, s):
+    """(I + s D^4)^-1 along axis 1, periodic: D^4 = (z - 2 + 1/z)^2 factored into a forward and a
+    backward recurrence with the characteristic root a inside the unit circle, a + 1/a = 2 + i/sqrt(s)."""
+    s = LD(s)
+    w = np.clongdouble(2) + np.clongdouble(1j) / np.sqrt(s)
+    d = np.sqrt(w * w - 4)
+    a = 2 / (w + d if abs(w + d) >= abs(w - d) else w - d)
+    p1, p2, c = 2 * a.real, -(a.real ** 2 + a.imag ** 2), s / (a.real ** 2 + a.imag ** 2)
+    n, pre = R.shape[1], int(50 / -math.log(math.sqrt(float(-p2)))) + 50  # the wrap has decayed below 1e-21
+
+    def forward(r):
+        r = np.ascontiguousarray(r.T)
+        x = y = np.zeros(r.shape[1], LD)
+        out = np.empty_like(r)
+        for q in range(-pre, n):
+            x, y = r[q % n] + p1 * x + p2 * y, x
+            if q >= 0:
+                out[q] = x
+        return out.T
+
+    return forward(forward(R)[:, ::-1])[:, ::-1] / c
+
+
+def steps_extended(f, L, gamma, dt, n):
+    ny, nx = f.shape
+    C, hx, hy, g, dt = f.astype(LD), LD(L) / nx, LD(L) / ny, LD(gamma), LD(dt)
+    for _ in range(n):
+        R = dt * laplacian(C * C * C - C - g * laplacian(C, hx, hy), hx, hy)
+        W = solve_rows(R, g * dt / hx ** 4)
+        C = C + solve_rows(W.T, g * dt / hy ** 4).T
+    return C
+
+
+def noise(ny, nx):
+    return 0.1 * (2 * np.random.default_rng(nx * 5003 + ny).random((ny, nx)) - 1)
+
+
+def separated(ny, nx):
+    x, y = np.arange(nx) * TWO_PI / nx, np.arange(ny) * TWO_PI / ny
+    f = np.cos(2 * x)[None, :] * np.cos(3 * y + 0.4)[:, None] + 0.7 * np.sin(x[None, :] - 4 * y[:, None])
+    return np.tanh(2.5 * f)
+
+
+def errors(f, L, gamma, dt, nsteps):
+    ny, nx = f.shape
+    ref = steps_extended(f, L, gamma, dt, nsteps)
+    out = []
+    for t in ({}, dict(split=1)):
+        with ch.Ensemble.create(nx, ny, L, gamma, dt, [0.0], 1, ch.CH_FP64) as e:
+            if t:
+                e.set_tuning(**t)
+            e.set_field(0, f)
+            e.step(nsteps)
+            d = np.abs(e.field(0) - ref)
+            out.append((float(np.sqrt(np.mean(d * d))), float(np.max(d))))
+    return out
+
+
+# gamma dt / h^4 of the closer spacing: 220, 420, 3200 | 0.86 at a spacing of 2 pi / 128 | wide, 420
+GRIDS = [(33, 512, TWO_PI), (17, 600, TWO_PI), (17, 1000, TWO_PI), (140, 513, 513 * TWO_PI / 128),
+         (200, 1024, 1024 * TWO_PI / 128), (97, 100, TWO_PI), (600, 17, TWO_PI)]
+
+
+@pytest.mark.parametrize("start", [noise, separated])
+@pytest.mark.parametrize("nx,ny,L", GRIDS)
+def test_no_less_precise_than_fp64_at_any_aspect_ratio(nx, ny, L, start):
+    fixed, fp64 = errors(start(ny, nx), L, 0.01, 5e-4, 2)
+    assert fixed[0] <= 1.25 * fp64[0]
+    assert fixed[1] <= 2.0 * fp64[1]
+
+
+@pytest.mark.parametrize("nx,ny", [(33, 512), (17, 600)])
+def test_allocation_free_step_of_tall_grids(nx, ny):
+    # its stated agreement with the FP64 kernels: 1e-13
+    torch = pytest.importorskip("torch")
+    f = noise(ny, nx)
+    with ch.Ensemble.create(nx, ny, TWO_PI, 0.01, 5e-4, [0.0], 1, ch.CH_FP64) as e:
+        e.set_tuning(split=1)
+        e.set_field(0, f)
+        e.step(2)
+        want = e.field(0)
+    C = torch.tensor(f, dtype=torch.float64, device="cuda").contiguous()
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    ch.ch_step_field_noalloc(C.data_ptr(), nx, ny, TWO_PI, 0.01, 5e-4, 2, st.cuda_stream)
+    st.synchronize()
+    assert np.max(np.abs(C.cpu().numpy() - want)) <= 1e-13
