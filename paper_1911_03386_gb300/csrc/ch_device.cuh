@@ -126,12 +126,13 @@ __device__ __forceinline__ void block_sum2(double& a, double& b, double* red) {
 // tile rows 2..nr+1) with mu recomputed in FP64 from the stored field once per point.  A
 // warp walks a strip of rows down a chunk of 31 columns, carrying three C rows and two mu
 // rows in registers; lane 31 holds the column after the chunk, so east neighbours come
-// from the next lane.  Fixed work split and order: deterministic.
+// from the next lane.  The work is split over the first nwarps warps and added in their order, so the
+// sums depend on nwarps but on no other property of the CTA.
 template <typename T>
 __device__ void band_partials_mu64(const DevView& v, const Tile& tl, int nx, int nr, const MemberParams& P,
-                                   double2* slot, double* red) {
+                                   double2* slot, double* red, int nwarps) {
   const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double a = P.a, bx = P.bx, by = P.by;
   // the stored field in FP64 (hi + lo for compensated members), read from global memory:
   // band row q of the tile is field row j0 - 2 + q (periodic)
@@ -151,7 +152,7 @@ __device__ void band_partials_mu64(const DevView& v, const Tile& tl, int nx, int
   // unscaled sums: (C^2 - 1)^2, (D+x C)^2, (D+y C)^2, (D+x mu)^2, (D+y mu)^2 (the grid
   // spacings and prefactors are applied once per thread at the end)
   double sw = 0.0, sdx = 0.0, sdy = 0.0, smx = 0.0, smy = 0.0;
-  for (int item = warp; item < nchunk * nstrip; item += nwarps) {
+  for (int item = warp < nwarps ? warp : nchunk * nstrip; item < nchunk * nstrip; item += nwarps) {
     const int k = item % nchunk, r0 = (item / nchunk) * hs, r1 = min(nr, r0 + hs);
     if (r0 >= r1) continue;
     const int i = (31 * k + lane) % nx;
@@ -346,10 +347,11 @@ __device__ __noinline__ bool fixed_partials(const MemberParams& P, int nx, int n
 }
 
 // The band's partial sums (tile tl) from the stored field in global memory, FP64 values or FP32 ones
-// (hi + lo for compensated members): in fixed point, or in FP64 where the range does not fit.
+// (hi + lo for compensated members): in fixed point, or in FP64 where the range does not fit (split over
+// nwarps warps, all of the CTA's if 0).
 template <typename T>
 __device__ void band_partials_field(const DevView& v, const Tile& tl, int nx, int nr, const MemberParams& P,
-                                    double2* slot, double* red) {
+                                    double2* slot, double* red, int nwarps = 0) {
   const T* H = static_cast<const T*>(v.C) + P.offset;
   const T* Lo = P.comp ? static_cast<const T*>(v.C) + P.lo_offset : nullptr;
   const int ny = P.ny, j0 = tl.start;
@@ -382,7 +384,7 @@ __device__ void band_partials_field(const DevView& v, const Tile& tl, int nx, in
       },
       sF, sD);
   if (!ok) {
-    band_partials_mu64<T>(v, tl, nx, nr, P, slot, red);
+    band_partials_mu64<T>(v, tl, nx, nr, P, slot, red, nwarps ? nwarps : (int)(blockDim.x >> 5));
     return;
   }
   if (threadIdx.x == 0) *slot = make_double2(sF, sD);

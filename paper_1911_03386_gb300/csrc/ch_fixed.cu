@@ -375,6 +375,10 @@ __device__ __forceinline__ void row_solve(i64* seg, int len, int l, int G, int g
   e_top = e_lsb + bit_length_hi(cta_or<NW>(ar.top, slots + 2 * NW));
 }
 
+// Warps that share a sample's FP64 sums (a band out of the scaled range): those of the row class's own
+// CTA, so that a member's samples do not depend on the CTA size that its company leads to.
+__device__ __forceinline__ int sample_warps(const MemberParams& P) { return P.fx == 1 ? 2 : P.fx == 2 ? 4 : 8; }
+
 template <int TH, int MINB>
 __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_base) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -465,7 +469,7 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
               std::integral_constant<int, 2>());
     });
   if (sample)
-    band_partials_field<double>(v, tl, nx, nr, P, v.partials + P.partial_base + tl.index, red);
+    band_partials_field<double>(v, tl, nx, nr, P, v.partials + P.partial_base + tl.index, red, sample_warps(P));
 
   // rows: gw lanes per row (row_solve starts with a barrier: R' is complete)
   const int l = lane & (gw - 1), row = threadIdx.x / gw, r = min(row, nr - 1);
@@ -496,7 +500,7 @@ __global__ void __launch_bounds__(256) fx_observe_kernel(DevView v, int tile_bas
   __shared__ double red[16];
   const Tile tl = v.row_tiles[tile_base + blockIdx.x];
   const MemberParams& P = v.mp[tl.member];
-  band_partials_field<double>(v, tl, P.nx, tl.count, P, v.partials + P.partial_base + tl.index, red);
+  band_partials_field<double>(v, tl, P.nx, tl.count, P, v.partials + P.partial_base + tl.index, red, sample_warps(P));
 }
 
 // -------------------------------------------------------------------------------------
@@ -732,7 +736,7 @@ cudaError_t launch_fx_rows(const DevView& v, const LaunchShape& sh, cudaStream_t
   int base = sh.n_row_tiles;
   const int* n = sh.fx_rt;
   const size_t* sm = sh.fx_smem;
-  // Classes only set the CTA size (a row's arithmetic does not depend on it): where several of the
+  // Classes only set the CTA size (a run's results do not depend on it): where several of the
   // short ones are present they share a launch, since a mix of small runs is bound by its launches
   // (a burst of 24 requests of 64^2 to 256^2 takes 35.2 ms in separate launches, 24.2 ms in one).
   if ((n[0] > 0) + (n[1] > 0) + (n[2] > 0) > 1) {
