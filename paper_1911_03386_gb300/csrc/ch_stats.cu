@@ -165,13 +165,15 @@ __global__ void __launch_bounds__(kThreads) histogram_kernel(View v, double lo, 
   if (s < v.T) {
     const int64_t so = slot_offset(v, s);
     const float lof = (float)lo, inv = (float)(1.0 / w);
+    // f32_trunc takes |b| < 2^-126 to zero, an error of up to 2^-126 / w in x
+    const float e0 = fmaf(1.2e-38f, inv, 1e-20f);
     for (int64_t j = wp; j < v.M; j += kWarps) {
       const double b = v.base[run_offset(v, j) + so + v.bc];
       if (!finite64(b)) continue;
       int bin;
-      // x = (b - lo) / w to within e: b, lo, w and the three operations each to 2^-23
+      // x = (b - lo) / w to within e: b, lo, w and the three operations each to 2^-23, and e0
       const float bf = chk::f32_trunc(b), x = (bf - lof) * inv, k32 = floorf(x);
-      const float e = 4.8e-7f * ((fabsf(bf) + fabsf(lof)) * inv + fabsf(x)) + 1e-20f;
+      const float e = 4.8e-7f * ((fabsf(bf) + fabsf(lof)) * inv + fabsf(x)) + e0;
       if (x - k32 > e && x - k32 < 1.0f - e && fabsf(x) < 1e6f) {
         bin = k32 < 0.0f ? 0 : k32 < (float)nbins ? (int)k32 + 1 : nbins + 1;
       } else if (b < lo) {
