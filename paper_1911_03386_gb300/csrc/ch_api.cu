@@ -492,7 +492,8 @@ int fill_params(const ch_member_desc& d, int precision, MemberParams* p) {
   return CH_OK;
 }
 
-using chk::red_doubles;
+// Reduction buffer of a CTA: two sums per warp, or the ten words of a sample's exact sums.
+size_t red_doubles(int threads) { return std::max<size_t>(10, (size_t)2 * (threads / 32)); }
 
 // C tile (nr+4 rows, dense pitch when rows move in 16-byte pieces) + mu tile (nr+2 rows,
 // pitch nx+1) + the FP64 reduction buffer; R' and the row sweep reuse the C tile's memory.

@@ -246,7 +246,7 @@ __device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + 
 // warp and scheduler: a sample cost as much as 7 FP64 or 30 FP32 steps.  In integers (the arithmetic
 // of the step's mu, sums of squares of 128 bits per strip and lane added exactly, so the result does
 // not depend on the CTA's size) it costs about one.  A warp takes 29 columns (lanes 0, 30 and 31 are their neighbours) of a
-// strip of 4 or 8 rows.  sums: red_doubles() words of shared memory; ends with every thread past a barrier;
+// strip of 4 or 8 rows.  sums: 80 bytes of shared memory; ends with every thread past a barrier;
 // false (nothing summed) where the values' range does not fit, the same in every thread.
 template <class Load, class Conv, class Mag>
 __device__ __noinline__ bool fixed_partials(const MemberParams& P, int nx, int nr, unsigned long long* sums, Load load,
@@ -268,7 +268,7 @@ __device__ __noinline__ bool fixed_partials(const MemberParams& P, int nx, int n
   const int emax = __reduce_max_sync(kAll, lane < nw ? (int)slots[lane] : 0);
   __syncthreads();
   if (!P.fx_mu || emax > 1023 || emax < 823) return false;
-  if (threadIdx.x < kExactSumWords) sums[threadIdx.x] = 0;
+  if (threadIdx.x < 10) sums[threadIdx.x] = 0;
   __syncthreads();
   const int E = emax - 1022, sh = 2 * E + 4;
   const i64 one = 1ll << 58;

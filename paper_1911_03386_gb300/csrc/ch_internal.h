@@ -211,13 +211,6 @@ struct LaunchShape {
   int fx_tiles;          // row tiles of all classes
 };
 
-// Reduction buffer of a CTA that takes a sample, in doubles: two sums per warp, or the words of a
-// sample's exact sums.
-constexpr int kExactSumWords = 10;
-constexpr size_t red_doubles(int threads) {
-  return threads / 16 > kExactSumWords ? (size_t)(threads / 16) : (size_t)kExactSumWords;
-}
-
 // Host-side fault injection (ch_fault.cu; armed by ch_set_fault or CH_FAULT).
 enum { kFaultNone = 0, kFaultAlloc = 1, kFaultNan = 2, kFaultTimeout = 3 };
 // Every device allocation of the library goes through here: an armed alloc fault makes

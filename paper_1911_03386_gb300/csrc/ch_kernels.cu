@@ -1166,7 +1166,7 @@ __global__ void __launch_bounds__(256, S == 16 ? 4 : 3) rows_walk_kernel(DevView
 size_t rows_walk_smem(int nr, int nx, int S) {
   const int cpl = S == 16 ? 2 : 4, ns = (nx + 32 * cpl - 1) / (32 * cpl);
   const size_t f = (size_t)(nr + 4) * (nx + 4 * (nx / S)) + ((2 * ns * (nr + 4) + 3) & ~3) + 28;
-  return ((f * sizeof(float) + 15) & ~(size_t)15) + red_doubles(256) * sizeof(double);
+  return ((f * sizeof(float) + 15) & ~(size_t)15) + 16 * sizeof(double);
 }
 
 // -------------------------------------------------------------------------------------
@@ -2534,7 +2534,7 @@ template <typename T>
 size_t rowT_smem_bytes(int nw) {
   size_t b = ((size_t)nw * 32 * 33 + (size_t)nw * 68 + (size_t)2 * nw * 64) * sizeof(T);
   b = (b + 15) & ~(size_t)15;
-  return b + red_doubles(32 * nw) * sizeof(double);
+  return b + (size_t)2 * nw * sizeof(double);
 }
 
 // The segment-form row kernel of one class, one CTA per band: FP32 in one tile, FP64 in two.
