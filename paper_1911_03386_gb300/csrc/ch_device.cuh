@@ -274,7 +274,7 @@ __device__ __noinline__ bool fixed_partials(const MemberParams& P, int nx, int n
   const i64 one = 1ll << 58;
   const FxLimb bx = P.fx_bx, by = P.fx_by;
   const int su = P.fx_su - 2;  // the cubic term from (C^2 - 1) 2^58
-  auto scaled = [](i64 v, int s) { return s >= 0 ? v << s : v >> -s; };
+  auto scaled = [](i64 v, int s) { return s >= 0 ? v << s : v >> min(-s, 63); };
   for (int item = warp; item < nchunk * nstrip; item += nw) {
     const int k = item % nchunk, r0 = (item / nchunk) * hs, r1 = min(nr, r0 + hs);
     if (r0 >= r1) continue;

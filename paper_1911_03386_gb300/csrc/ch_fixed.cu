@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
     RhsFp rhs{P.fx_tall != 0, P.fx_ratio, P.fx_w0};
     band_rhs<NW, -1>(b, Es, Em, top, emax, MuFp{P.a, P.bx, P.by}, rhs, wtop + 4 * NW);
   } else
-    with_shift(2 * (emax - 1022) + 6 - P.fx_su, [&](auto sh) {
+    with_shift(max(-62, 2 * (emax - 1022) + 6 - P.fx_su), [&](auto sh) {  // C^2 vanishes long before -62
       const i64 one = 1ll << (60 - P.fx_su);
       auto fixed = [&](auto mu, auto rhs, auto form) {
         band_rhs<NW, decltype(form)::value>(b, Es, Em, top, emax, mu, rhs, wtop + 4 * NW);
