@@ -547,7 +547,9 @@ typedef struct {
 /*
  * Create a server of one precision whose runs' fields fit in hbm_budget_bytes of device
  * memory (two arenas: fields and row-solve scratch, allocated now) with at most
- * max_members runs in flight.  Errors: CH_EINVAL, CH_ENOMEM, CH_ECUDA.
+ * max_members runs in flight.  Also allocated now, beside the arenas: the runs' parameter, state and
+ * tile tables, the row exponents of CH_FP64 runs (4 bytes per 16 elements of scratch) and the 1 MiB
+ * staging buffer through which CH_FP32 fields are converted.  Errors: CH_EINVAL, CH_ENOMEM, CH_ECUDA.
  */
 int ch_server_create(size_t hbm_budget_bytes, int precision, int max_members, ch_server* out);
 /* Queue a request (non-blocking); *id identifies it.  Errors: CH_EINVAL (bad request),

@@ -1292,21 +1292,21 @@ int ch_series(ch_handle h, int member, double* out, int64_t cap, int64_t* n) {
 }  // extern "C"
 
 namespace chh {
+// Staging buffer of n values for CH_FP32 transfers; false (none) if the device has no room for it.
+bool alloc_stage(ch_ensemble* h, int64_t n) {
+  if (chk::dev_malloc((void**)&h->stage, sizeof(double) * n) != cudaSuccess) h->stage = nullptr;
+  h->stage_points = h->stage ? n : 0;
+  return h->stage != nullptr;
+}
+
 // The fields of members k0 .. k1 - 1, one after another, between host memory (FP64 values) and the
 // device.  Members that follow each other in C move in one piece: FP64 as they are, FP32 through
 // the staging buffer, converted on the device (compensated members: hi + lo).  Synchronises.
 template <bool OUT>
 int move_fields(ch_ensemble* h, int k0, int k1, void* host, const char* what) {
   double* at = static_cast<double*>(host);
-  if (h->precision == CH_FP32 && !h->stage) {
-    const int64_t n = std::min<int64_t>(ch_ensemble::kStage, std::max<int64_t>(h->w_points, h->total_points));
-    if (cudaMalloc(&h->stage, sizeof(double) * n) == cudaSuccess) {
-      h->stage_points = n;
-    } else {  // converted on the host below
-      cudaGetLastError();
-      h->stage = nullptr;
-    }
-  }
+  if (h->precision == CH_FP32 && !h->stage && !alloc_stage(h, std::min(ch_ensemble::kStage, h->total_points)))
+    cudaGetLastError();  // converted on the host below
   std::vector<float> hh, hl;
   auto lo_delta = [&](int k) { return h->hp[k].comp ? h->hp[k].lo_offset - h->hp[k].offset : -1; };
   for (int k = k0; k < k1;) {

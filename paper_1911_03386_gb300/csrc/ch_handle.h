@@ -69,8 +69,9 @@ struct ch_ensemble {
   cudaEvent_t fork = nullptr;
   int aux_used = 0;
 
-  // CH_FP32: staging of FP64 values for field transfers (allocated on first use, kept)
-  static constexpr int64_t kStage = (int64_t)1 << 22;
+  // CH_FP32: staging of FP64 values for field transfers, allocated on first use and kept; a server,
+  // which serves from a fixed budget, allocates a smaller one when it is created
+  static constexpr int64_t kStage = (int64_t)1 << 22, kServerStage = (int64_t)1 << 17;
   double* stage = nullptr;
   int64_t stage_points = 0;
 
@@ -120,6 +121,7 @@ int fx_class(int nx);
 int fx_band(int nx);
 void fx_shape(const MemberParams& p, chk::LaunchShape* sh);
 ch_tuning default_tuning();
+bool alloc_stage(ch_ensemble* h, int64_t n);
 // Tiles and launch shapes for the present members under tuning t.
 int build_tiles(ch_ensemble* h, const ch_tuning& t);
 // Upload tile tables, partial slots and member parameters (synchronises the stream).

@@ -373,6 +373,7 @@ int ch_server_create(size_t hbm_budget_bytes, int precision, int max_members, ch
     cudaFree(h->dcst);
     cudaFree(h->dres);
     cudaFree(h->dpart);
+    cudaFree(h->stage);
     if (h->own) cudaStreamDestroy(h->own);
     delete h;
     delete S;
@@ -399,6 +400,8 @@ int ch_server_create(size_t hbm_budget_bytes, int precision, int max_members, ch
     return cleanup(CH_ECUDA, std::string("server set-up: ") + cudaGetErrorString(e));
   if (int rc = chh::build_tiles(h, h->tuning)) return cleanup(rc, "server tiles");
   if (int rc = chh::upload_tiles(h)) return cleanup(rc, "server tiles");
+  if (precision == CH_FP32 && !chh::alloc_stage(h, std::min(elems, ch_ensemble::kServerStage)))
+    return cleanup(CH_ENOMEM, "server allocation: field staging");
   S->t_created = Clock::now();
   S->worker = std::thread(worker_main, S);
   *out = S;
