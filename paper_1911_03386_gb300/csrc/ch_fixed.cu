@@ -746,12 +746,10 @@ cudaError_t launch_fx_rows(const DevView& v, const LaunchShape& sh, cudaStream_t
     if (n[3] > 0) launch_dependent(fx_rows_kernel<256, 2>, n[3], 256, sm[3], st, v, base, tables_ready);
     return cudaPeekAtLastError();
   }
-  // few tiles: larger CTAs (a sample's sums then take 8 warps instead of 2 or 4)
+  // few tiles of one short class (so none of the next): larger CTAs (a sample's sums then take 8 warps)
   if (n[0] + n[1] > 0 && n[0] + n[1] <= kDependentCtas) {
     launch_dependent(fx_rows_kernel<256, 4>, n[0] + n[1], 256, max(sm[0], sm[1]), st, v, base, tables_ready);
     base += n[0] + n[1];
-    if (n[2] > 0) launch_dependent(fx_rows_kernel<256, 4>, n[2], 256, sm[2], st, v, base, tables_ready);
-    base += n[2];
     if (n[3] > 0) launch_dependent(fx_rows_kernel<256, 2>, n[3], 256, sm[3], st, v, base, tables_ready);
     return cudaPeekAtLastError();
   }
