@@ -1014,7 +1014,7 @@ __device__ __forceinline__ void seg_tile_setup(const DevView& v, const Tile& tl,
 // (28 T), then the FP64 reduction buffer.  PERSIST: a CTA walks the tiles blockIdx.x,
 // + gridDim.x, ... and copies the next tile's C band while it computes the current one.
 template <typename T, int S, bool PERSIST>
-__global__ void __launch_bounds__(256) rows_seg_kernel(DevView v, int base, int ntiles, int ccap, int mcap) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? (S == 16 ? 4 : 3) : 1) rows_seg_kernel(DevView v, int base, int ntiles, int ccap, int mcap) {
   extern __shared__ __align__(16) unsigned char smem[];
   T* Cbuf = reinterpret_cast<T*>(smem);
   T* Ms = Cbuf + (size_t)(PERSIST ? 2 : 1) * ccap;
