@@ -1013,6 +1013,9 @@ __device__ __forceinline__ void seg_tile_setup(const DevView& v, const Tile& tl,
 // when PERSIST), the mu tile (mcap elements), the 24 scan constants and the sample flag
 // (28 T), then the FP64 reduction buffer.  PERSIST: a CTA walks the tiles blockIdx.x,
 // + gridDim.x, ... and copies the next tile's C band while it computes the current one.
+// Launch bounds: CH_FP32 (persistent only) held to 64 (80) registers, which the shared memory of two C
+// tiles and one mu tile leaves room for at bands of 16 rows: 64 x 512^2 112 us per step with the bound
+// and 128 without (116 registers, two CTAs per SM), 256 x 256^2 109 and 128, 16 x 1024^2 166 and 164.
 template <typename T, int S, bool PERSIST>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? (S == 16 ? 4 : 3) : 1) rows_seg_kernel(DevView v, int base, int ntiles, int ccap, int mcap) {
   extern __shared__ __align__(16) unsigned char smem[];
