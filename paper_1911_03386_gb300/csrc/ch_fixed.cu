@@ -93,12 +93,10 @@ struct Fp {
   static constexpr bool kFixed = false;
   static __device__ __forceinline__ State state(i64 y) { return __longlong_as_double(y); }
   static __device__ __forceinline__ i64 value(State s) { return double_bits(s); }
-  static __device__ __forceinline__ double entry(FxLimb m) {  // times 2^58
-    return ldexp((double)(((i64)m.h << 32) + m.l), -58);
-  }
+  // (a table after tab_to_fp64)
   static __device__ __forceinline__ i64 dot(const FxLimb* row, i64 x0, i64 x1, i64 r) {
-    return double_bits(fma(entry(row[0]), __longlong_as_double(x0),
-                           fma(entry(row[1]), __longlong_as_double(x1), __longlong_as_double(r))));
+    const double* m = reinterpret_cast<const double*>(row);
+    return double_bits(fma(m[0], __longlong_as_double(x0), fma(m[1], __longlong_as_double(x1), __longlong_as_double(r))));
   }
   __device__ __forceinline__ void track(i64) {}
 };
@@ -161,7 +159,7 @@ __device__ __forceinline__ void pass_full(A& ar, i64* p, int es, int len, typena
 // segment may be shorter than the others; tab.A[d] = M^(S 2^d), tab.P = M^(length of the last
 // segment), tab.B[l] = M^(S l) P, tab.B[32 + pos] = M^(distance from the line's end) P with P
 // = (I - M^n)^-1, all in shared memory.  (a, b): end state in, start state out.
-struct ScanTab {
+struct alignas(16) ScanTab {
   FxLimb A[5][4], P[4], B[64][4];  // entries / 64, times 2^64, row-major
 };
 // The table into shared memory (16-byte asynchronous copies: Ax, Px, Bx lie like A, P, B).
@@ -169,6 +167,15 @@ __device__ __forceinline__ void load_tab(ScanTab& t, const SegTable& g) {
   static_assert(sizeof(ScanTab) % 16 == 0, "whole pieces");
   for (int k = threadIdx.x; k < (int)(sizeof(ScanTab) / 16); k += blockDim.x)
     copy16(reinterpret_cast<char*>(&t) + 16 * k, reinterpret_cast<const char*>(&g.Ax[0][0]) + 16 * k);
+}
+
+// The table's entries to FP64, in place (the Fp policy; the caller's barriers order it).
+__device__ __forceinline__ void tab_to_fp64(ScanTab& t) {
+  FxLimb* m = &t.A[0][0];
+  for (int k = threadIdx.x; k < (int)(sizeof(ScanTab) / sizeof(FxLimb)); k += blockDim.x) {
+    const double x = ldexp((double)(((i64)m[k].h << 32) + m[k].l), -58);
+    *reinterpret_cast<double*>(m + k) = x;
+  }
 }
 
 // Programmatic dependent launch: a step kernel lets its successor start (its CTAs take the SMs'
@@ -258,7 +265,8 @@ struct RhsFp {
   __device__ __forceinline__ i64 operator()(i64 m_, i64 e_, i64 w_, i64 n_, i64 s_) const {
     const double m = __longlong_as_double(m_), e = __longlong_as_double(e_), w = __longlong_as_double(w_),
                  n = __longlong_as_double(n_), s = __longlong_as_double(s_);
-    return double_bits(fma(w0, m, tall ? fma(ratio, e + w, s + n) : fma(ratio, s + n, e + w)));
+    const double x = e + w, y = s + n, p = tall ? x : y, q = tall ? y : x;
+    return double_bits(fma(w0, m, fma(ratio, p, q)));
   }
 };
 
@@ -449,6 +457,7 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
   __syncthreads();
   int up = 0;  // R' is held times 2^(kmu + up - E)
   if (bad) {
+    tab_to_fp64(tab);
     RhsFp rhs{P.fx_tall != 0, P.fx_ratio, P.fx_w0};
     band_rhs<NW, -1>(b, Es, Em, top, emax, MuFp{P.a, P.bx, P.by}, rhs, wtop + 4 * NW);
   } else
@@ -690,8 +699,14 @@ __global__ void __launch_bounds__(kColThreads, 3) fx_cols_kernel(DevView v, int 
     Fp ar(P.fx_cy, P.p1y, P.p2y);
     double a, b;
     col_first(ar, y, len, S, ws, a, b, [](short2 e, auto f) {
-      f([e](i64 w) { return e.y == kBadRow ? w : double_bits(ldexp((double)w, e.x)); });
+      if (e.y == kBadRow) {
+        f([](i64 w) { return w; });
+      } else {
+        const double unit = pow2(e.x);  // e.x >= -400: no subnormal
+        f([unit](i64 w) { return double_bits(unit * (double)w); });
+      }
     });
+    tab_to_fp64(tab);
     col_solve(ar, y, len, tab, xs, wtop, G, gw, P.fx_lvy, ny % S == 0, cw, 0, a, b);
     col_update(ar, ye, len, Ce, nx, P.fx_kappa, cv, a, b, [](i64 t) { return __longlong_as_double(t); });
   } else {
