@@ -322,14 +322,18 @@ void fx_mu_params(MemberParams* p) {
   p->fx_ratio = p->fx_tall ? (p->hy * p->hy) / (p->hx * p->hx) : p->rho;
   p->fx_w0 = -2.0 * (1.0 + p->fx_ratio);
   p->fx_kappa = p->fx_tall ? p->dt / (p->hy * p->hy * p->cx * p->cy) : p->kappa;
-  // |C| < 2^E: |mu| / 2^E <= 3 + 4 (bx + by) for E <= 1 and |R'| <= 4 (1 + ratio) |mu|, which has
-  // to fit 62 bits (60 where R' takes a product).  The ratio is at most 1 whatever the grid: with
+  // |C| < 2^E: |mu| / 2^E <= max(3, 4^E - 1) + 4 (bx + by) and |R'| <= 4 (1 + ratio) |mu|, which has
+  // to fit 62 bits (60 where R' takes a product).  (C^2 - 1) 2^(60 - su) fits 62 bits if su >= 2 E - 2.  The ratio is at most 1 whatever the grid: with
   // rho = (hx / hy)^2 in its place a tall grid's headroom came out of mu (17 x 600: 39 bits of mu and
   // 94 times the FP64 kernels' error on a separated field).
-  const double bound = 4.0 * (1.0 + p->fx_ratio) * (3.0 + 4.0 * (p->bx + p->by));
-  p->fx_mu = std::isfinite(bound) && bound < 1e9;
+  auto bound = [&](int E) { return 4.0 * (1.0 + p->fx_ratio) * (std::ldexp(1.0, 2 * E) - 1.0 + 4.0 * (p->bx + p->by)); };
+  auto kmu = [&](int E) {
+    return std::min(57 - 2 * E, (p->fx_square ? 62 : 60) - (int)std::ceil(std::log2(bound(E))));
+  };
+  p->fx_mu = std::isfinite(bound(1)) && bound(1) < 1e9;
   if (!p->fx_mu) return;
-  p->fx_kmu = std::min(55, (p->fx_square ? 62 : 60) - (int)std::ceil(std::log2(bound)));
+  p->fx_kmu = kmu(1);
+  for (int E = 2; E <= chk::kFxMaxE; ++E) p->fx_cut[E - 2] = p->fx_kmu - kmu(E);
   p->fx_su = 55 - p->fx_kmu;
   p->fx_bx = fx_limb(std::ldexp(p->bx, p->fx_kmu + 5));
   p->fx_by = fx_limb(std::ldexp(p->by, p->fx_kmu + 5));

@@ -237,6 +237,12 @@ struct SquareSum {
   }
 };
 
+// v / 2^r of a constant, r >= 0, rounded.
+__device__ __forceinline__ FxLimb cut_limb(FxLimb q, int r) {
+  const i64 v = ((i64)q.h << 32) + q.l;
+  return r > 0 ? limbs(shift_down(v, r)) : q;
+}
+
 __device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 
 // Partial sums of the F and dF/dt densities (in thread 0) over nr rows of a field of nx columns in
@@ -267,13 +273,14 @@ __device__ __noinline__ bool fixed_partials(const MemberParams& P, int nx, int n
   __syncthreads();
   const int emax = __reduce_max_sync(kAll, lane < nw ? (int)slots[lane] : 0);
   __syncthreads();
-  if (!P.fx_mu || emax > 1023 || emax < 823) return false;
+  if (!P.fx_mu || emax > 1022 + kFxMaxE || emax < 823) return false;
   if (threadIdx.x < 10) sums[threadIdx.x] = 0;
   __syncthreads();
-  const int E = emax - 1022, sh = 2 * E + 4;
-  const i64 one = 1ll << 58;
-  const FxLimb bx = P.fx_bx, by = P.fx_by;
-  const int su = P.fx_su - 2;  // the cubic term from (C^2 - 1) 2^58
+  const int E = emax - 1022, cut = E > 1 ? P.fx_cut[E - 2] : 0, kmu = P.fx_kmu - cut;
+  const int wb = 60 - 2 * max(E, 1), sh = 2 * E + wb - 54;  // C^2 - 1 is held times 2^wb
+  const i64 one = 1ll << wb;
+  const FxLimb bx = cut_limb(P.fx_bx, cut), by = cut_limb(P.fx_by, cut);
+  const int su = P.fx_su + cut + wb - 60;  // the cubic term from (C^2 - 1) 2^wb
   auto scaled = [](i64 v, int s) { return s >= 0 ? v << s : v >> min(-s, 63); };
   for (int item = warp; item < nchunk * nstrip; item += nw) {
     const int k = item % nchunk, r0 = (item / nchunk) * hs, r1 = min(nr, r0 + hs);
@@ -282,7 +289,7 @@ __device__ __noinline__ bool fixed_partials(const MemberParams& P, int nx, int n
     const bool own = lane >= 1 && lane <= 29 && 29 * k + lane - 1 < nx;
     auto mu_of = [&](i64 c, i64 e, i64 w, i64 n, i64 s, i64& q) {
       const FxLimb cl = limbs(c);
-      q = scaled(mul_top(cl, cl), sh) - one;  // (C^2 - 1) 2^58
+      q = scaled(mul_top(cl, cl), sh) - one;
       const i64 u = mul_top(cl, limbs(scaled(q, -su)));
       return u - mul_top(limbs(e + w - 2 * c), bx) - mul_top(limbs(n + s - 2 * c), by);
     };
@@ -336,8 +343,8 @@ __device__ __noinline__ bool fixed_partials(const MemberParams& P, int nx, int n
     // lane q: sum q: (C^2 - 1)^2 / 4, gamma / 2 of (D+x C)^2 and (D+y C)^2, (D+x mu)^2, (D+y mu)^2
     const int q = min(lane, 4);
     const double hinv = (q & 1) ? P.ihx2 : P.ihy2;
-    const double weight = q == 0 ? pow2(16 - 118) : q < 3 ? 0.5 * P.gamma * pow2(16 + 2 * (E - 59)) * hinv
-                                                          : pow2(16 + 2 * (E - P.fx_kmu)) * hinv;
+    const double weight = q == 0 ? pow2(14 - 2 * wb) : q < 3 ? 0.5 * P.gamma * pow2(16 + 2 * (E - 59)) * hinv
+                                                          : pow2(16 + 2 * (E - kmu)) * hinv;
     const double s = weight * fma((double)sums[2 * q + 1], 18446744073709551616.0, (double)sums[2 * q]);
     sF = s + (__shfl_sync(kAll, s, 1) + __shfl_sync(kAll, s, 2));
     sD = __shfl_sync(kAll, s, 3) + __shfl_sync(kAll, s, 4);

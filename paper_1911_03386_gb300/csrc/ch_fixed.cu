@@ -26,7 +26,7 @@
 // a bound of the recurrence's gain (the l1 norm of its impulse response), and its result is
 // shifted the same way before the backward one.
 //
-// A band whose largest |C| is outside [2^-200, 2), or not finite, is taken through the same
+// A band whose largest |C| is outside [2^-200, 8), or not finite, is taken through the same
 // code in FP64 arithmetic (the Fp policy), its rows marked kBadRow; the columns of a member
 // with such a row run in FP64 too.
 //
@@ -446,7 +446,8 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
   __syncthreads();
   top = __reduce_max_sync(kAll, lane < NW ? wtop[lane] : 0u);
   const int emax = (int)(top >> 20);  // biased exponent of the largest |C|
-  const bool bad = emax > 1023 || emax < 823;
+  const bool bad = emax > 1022 + kFxMaxE || emax < 823;
+  const int cut = !bad && emax > 1023 ? P.fx_cut[emax - 1024] : 0, kmu = P.fx_kmu - cut, su = P.fx_su + cut;
   // the strips' edge columns
   for (int k = threadIdx.x; k < 2 * b.ns * (nr + 4); k += TH) {
     const int e = k / (nr + 4), t = k - e * (nr + 4);
@@ -461,20 +462,21 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
     RhsFp rhs{P.fx_tall != 0, P.fx_ratio, P.fx_w0};
     band_rhs<NW, -1>(b, Es, Em, top, emax, MuFp{P.a, P.bx, P.by}, rhs, wtop + 4 * NW);
   } else
-    with_shift(max(-62, 2 * (emax - 1022) + 6 - P.fx_su), [&](auto sh) {  // C^2 vanishes long before -62
-      const i64 one = 1ll << (60 - P.fx_su);
+    with_shift(max(-62, 2 * (emax - 1022) + 6 - su), [&](auto sh) {  // C^2 vanishes long before -62
+      const i64 one = 1ll << (60 - su);
+      const FxLimb bx = cut_limb(P.fx_bx, cut), by = cut_limb(P.fx_by, cut);
       auto fixed = [&](auto mu, auto rhs, auto form) {
         band_rhs<NW, decltype(form)::value>(b, Es, Em, top, emax, mu, rhs, wtop + 4 * NW);
         up = rhs.up;
       };
       if (P.fx_square)
-        fixed(MuFx<true, decltype(sh)>{P.fx_bx, P.fx_by, one, sh}, RhsFx<0>{P.fx_rl, P.fx_er},
+        fixed(MuFx<true, decltype(sh)>{bx, by, one, sh}, RhsFx<0>{P.fx_rl, P.fx_er},
               std::integral_constant<int, 0>());
       else if (!P.fx_tall)
-        fixed(MuFx<false, decltype(sh)>{P.fx_bx, P.fx_by, one, sh}, RhsFx<1>{P.fx_rl, P.fx_er},
+        fixed(MuFx<false, decltype(sh)>{bx, by, one, sh}, RhsFx<1>{P.fx_rl, P.fx_er},
               std::integral_constant<int, 1>());
       else
-        fixed(MuFx<false, decltype(sh)>{P.fx_bx, P.fx_by, one, sh}, RhsFx<2>{P.fx_rl, P.fx_er},
+        fixed(MuFx<false, decltype(sh)>{bx, by, one, sh}, RhsFx<2>{P.fx_rl, P.fx_er},
               std::integral_constant<int, 2>());
     });
   if (sample)
@@ -491,7 +493,7 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
   else
     row_solve<NW>(seg, len, l, G, gw, P.fx_lvx, full, Fx(P.fx_cx, 0.0, 0.0), tab, P.fx_gainx, top, wtop + NW, e_lsb, e_top);
   if (row < nr && l == 0) {
-    const int eb = emax - 1022 - P.fx_kmu - up;
+    const int eb = emax - 1022 - kmu - up;
     v.wexp[P.fx_wexp + j0 + row] = bad ? make_short2(0, kBadRow) : make_short2((short)(e_lsb + eb), (short)(e_top + eb));
   }
   // W to HBM as whole rows (row_solve ends with a barrier)

@@ -29,6 +29,7 @@ struct FxLimb {
 struct FxCoef {
   FxLimb p1, p2;         // recurrence coefficients / 8, times 2^64
 };
+constexpr int kFxMaxE = 3;        // |C| < 2^E up to here in fixed point
 constexpr int kBadRow = 32767;    // row exponent of a row held in FP64
 constexpr int kFxRowClasses = 4;  // nx <= 64, 128, 512, 1024
 
@@ -74,7 +75,8 @@ struct MemberParams {
   int fx_sx, fx_sy, fx_cw;           // points per segment (powers of two), columns per panel
   int fx_gainx, fx_gainy;            // log2 bound of the recurrences' gain
   int fx_mu;                         // kmu, su, bx, by are set (any precision: the observables' sums)
-  int fx_kmu, fx_su;                 // mu is held times 2^(kmu - E); su = 55 - kmu
+  int fx_kmu, fx_su;                 // mu is held times 2^(kmu - E), |C| < 2^E; su = 55 - kmu
+  int fx_cut[2];                     // kmu less this, su more, for E = 2, 3 (larger cubic term)
   // R' of the fixed-point form, from the second differences dx, dy of mu: dx + ratio dy, or where
   // hy < hx ratio dx + dy (1 / rho times the other form's; kappa times rho), so ratio <= 1
   int fx_er, fx_square, fx_tall;     // ratio product: d << er; square: hx = hy; tall: hy < hx

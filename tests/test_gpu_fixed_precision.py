@@ -102,6 +102,34 @@ def test_no_less_precise_than_fp64_at_any_aspect_ratio(nx, ny, L, start):
     assert fixed[1] <= 2.0 * fp64[1]
 
 
+@pytest.mark.parametrize("scale", [1.9, 2.1, 3.9, 4.1, 7.9])  # the scale's exponents end at 2, 4 and 8
+@pytest.mark.parametrize("nx,ny", [(64, 64), (100, 70), (48, 96)])
+@pytest.mark.parametrize("start", [noise, separated])
+def test_no_less_precise_than_fp64_at_large_values(nx, ny, start, scale):
+    f = start(ny, nx)
+    f *= scale / np.max(np.abs(f))
+    fixed, fp64 = errors(f, nx * TWO_PI / 128, 0.01, 2e-6, 2)
+    assert fixed[0] <= 1.25 * fp64[0]
+    assert fixed[1] <= 2.0 * fp64[1]
+
+
+@pytest.mark.parametrize("scale", [0.9, 2.5, 7.0])
+def test_samples_at_large_values(scale):
+    # F and dF/dt against the FP64 kernels: both round sums of 4096 terms of one sign
+    f = separated(64, 64)
+    f *= scale / np.max(np.abs(f))
+    out = []
+    for t in ({}, dict(split=1)):
+        with ch.Ensemble.create(64, 64, TWO_PI, 0.01, 1e-6, [0.0], 1, ch.CH_FP64) as e:
+            if t:
+                e.set_tuning(**t)
+            e.set_field(0, f)
+            F, D, _ = e.observables()
+            out.append((F[0], D[0]))
+    for a, b in zip(*out):
+        assert abs(a - b) <= 64 * 2.0 ** -53 * abs(b)
+
+
 @pytest.mark.parametrize("nx,ny", [(33, 512), (17, 600)])
 def test_allocation_free_step_of_tall_grids(nx, ny):
     # its stated agreement with the FP64 kernels: 1e-13
