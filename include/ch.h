@@ -181,7 +181,7 @@ int ch_launch_phase(ch_handle h, int phase);
  * Launch shape of a handle's kernels (no effect on results beyond round-off order within
  * a line's recurrence chunks; every choice is checked by the parity tests).  Fields <= 0
  * (split: -1) take the precision's default.  With every field at its default, CH_FP64 members
- * of 16 to 1024 points per axis and gamma dt / h^4 up to about 1e5 run in the fixed-point form,
+ * of 16 to 1024 points per axis and gamma dt / h^4 up to about 5e4 run in the fixed-point form,
  * whose shapes follow from the member's size alone; setting a field (other than the CH_FP32
  * ones, resident and resident_rows, and col_seg = -1, the CH_FP64 default) selects the FP64 kernels
  * described here.  ch_get_tuning reports member 0: defaults (col_seg and resident -1) where it runs

@@ -340,14 +340,15 @@ void fx_mu_params(MemberParams* p) {
 }
 
 // The member's constants of the fixed-point form; false where it does not apply: lines of 16 to
-// 1024 points whose recurrences gain at most 2^9 (s up to about 1e5: above, 64 bits minus the
-// gain's headroom would hold less than FP64).  x, y: its scan tables, filled in where it applies.
+// 1024 points whose recurrences gain at most 2^8 (s up to about 5e4: above, 62 bits minus the gain's
+// headroom hold no more than FP64; at s = 8e4, gain 2^9, a step's error was up to 1.8 times the FP64
+// kernels').  x, y: its scan tables, filled in where it applies.
 bool fx_params(MemberParams* p, chk::SegTable* x, chk::SegTable* y) {
   if (p->nx < 16 || p->ny < 16 || p->nx > 1024 || p->ny > 1024) return false;
   p->fx_gainx = fx_gain(p->p1x, p->p2x);
   const bool alike = p->nx == p->ny && p->p1x == p->p1y && p->p2x == p->p2y;  // both directions
   p->fx_gainy = alike ? p->fx_gainx : fx_gain(p->p1y, p->p2y);
-  if (p->fx_gainx > 9 || p->fx_gainy > 9) return false;
+  if (p->fx_gainx > 8 || p->fx_gainy > 8) return false;
   if (!p->fx_mu) return false;
   int er = 0;
   if (std::frexp(p->fx_ratio, &er) > 1.0 - 1e-9) ++er;  // ratio < 2^er, not by rounding alone

@@ -31,14 +31,17 @@ def laplacian(f, hx, hy):
             + (np.roll(f, -1, 0) - 2 * f + np.roll(f, 1, 0)) / hy ** 2)
 
 
-def solve_rows(R, s):
-    """(I + s D^4)^-1 along axis 1, periodic: D^4 = (z - 2 + 1/z)^2 factored into a forward and a
+def solve_rows(R, s, coefficients=None):
+    """(I + s D^4)^-1 along axis 1, periodic (or the recurrences of given p1, p2, over c): D^4 = (z - 2 + 1/z)^2 factored into a forward and a
     backward recurrence with the characteristic root a inside the unit circle, a + 1/a = 2 + i/sqrt(s)."""
-    s = LD(s)
-    w = np.clongdouble(2) + np.clongdouble(1j) / np.sqrt(s)
-    d = np.sqrt(w * w - 4)
-    a = 2 / (w + d if abs(w + d) >= abs(w - d) else w - d)
-    p1, p2, c = 2 * a.real, -(a.real ** 2 + a.imag ** 2), s / (a.real ** 2 + a.imag ** 2)
+    if coefficients:
+        p1, p2, c = coefficients
+    else:
+        s = LD(s)
+        w = np.clongdouble(2) + np.clongdouble(1j) / np.sqrt(s)
+        d = np.sqrt(w * w - 4)
+        a = 2 / (w + d if abs(w + d) >= abs(w - d) else w - d)
+        p1, p2, c = 2 * a.real, -(a.real ** 2 + a.imag ** 2), s / (a.real ** 2 + a.imag ** 2)
     n, pre = R.shape[1], int(50 / -math.log(math.sqrt(float(-p2)))) + 50  # the wrap has decayed below 1e-21
 
     def forward(r):
@@ -100,6 +103,45 @@ def test_no_less_precise_than_fp64_at_any_aspect_ratio(nx, ny, L, start):
     fixed, fp64 = errors(start(ny, nx), L, 0.01, 5e-4, 2)
     assert fixed[0] <= 1.25 * fp64[0]
     assert fixed[1] <= 2.0 * fp64[1]
+
+
+def step_with_library_coefficients(f, L, gamma, dt):
+    """One step of an n x n field in extended precision with the library's own FP64 coefficients, so
+    that a form's error is its rounding alone (at large s the coefficients' is as large)."""
+    n = f.shape[0]
+    h2 = (L / n) ** 2
+    c, p1, p2, _ = ch.ch_penta_factor(gamma * dt / h2 ** 2)
+    C, a, b = f.astype(LD), LD(1 - 2 * gamma / h2 - 2 * gamma / h2), LD(gamma / h2)
+
+    def around(g):
+        return np.roll(g, 1, 1) + np.roll(g, -1, 1) + np.roll(g, 1, 0) + np.roll(g, -1, 0)
+
+    mu = C * (C * C - a) - b * around(C)
+    W = solve_rows(around(mu) - 4 * mu, None, (LD(p1), LD(p2), LD(1)))
+    return C + LD(dt / (h2 * c * c)) * solve_rows(W.T, None, (LD(p1), LD(p2), LD(1))).T
+
+
+@pytest.mark.parametrize("s", [2e4, 4e4, 8e4])  # gain 2^7.4, 2^7.8, 2^8.3
+@pytest.mark.parametrize("n", [64, 128])
+def test_no_less_precise_than_fp64_at_large_s(n, s):
+    # noise in 8 rows and a hundredth of it elsewhere, so that one band's scale is the whole field's;
+    # the root mean square over 24 fields: each has a few independent long waves, so the two pooled
+    # errors of equal size differ by a few per cent
+    gamma, seeds = 0.01, 24
+    dt = s * (TWO_PI / n) ** 4 / gamma
+    f = np.stack([2 * np.random.default_rng(k).random((n, n)) - 1 for k in range(seeds)])
+    f[:, 8:] *= 0.01
+    total = []
+    for t in ({}, dict(split=1)):
+        with ch.Ensemble.create(n, n, TWO_PI, gamma, dt, [0.0] * seeds, 1, ch.CH_FP64) as e:
+            if t:
+                e.set_tuning(**t)
+            e.set_fields_ptr(f.ctypes.data)
+            e.step(1)
+            total.append([e.field(k) for k in range(seeds)])
+    ref = [step_with_library_coefficients(g, TWO_PI, gamma, dt) for g in f]
+    fixed, fp64 = (sum(float(np.mean((g - r) ** 2)) for g, r in zip(out, ref)) for out in total)
+    assert math.sqrt(fixed / fp64) <= 1.05
 
 
 @pytest.mark.parametrize("scale", [1.9, 2.1, 3.9, 4.1, 7.9])  # the scale's exponents end at 2, 4 and 8
