@@ -23,10 +23,15 @@
  *  - A handle is not thread-safe: use one handle per host thread.  Work is enqueued on the
  *    handle's CUDA stream (its own by default, or the caller's via ch_set_stream); calls
  *    that return host data synchronise that stream only.
- *  - Precision: CH_FP64 keeps fields in FP64 and computes each step with at least FP64's
- *    precision: by default in 64-bit fixed point scaled to the data (59 to 62 significant
- *    bits; lines of 16 to 1024 points), in FP64 for other sizes, for values outside the
- *    scaled range and whenever ch_tuning asks for a kernel shape.  CH_FP32 keeps fields,
+ *  - Precision: CH_FP64 keeps fields in FP64 and computes each step with FP64's precision:
+ *    by default in 64-bit fixed point scaled to the data (lines of 16 to 1024 points,
+ *    gamma dt / h^4 up to about 5e4), in FP64 for other members, for values outside the
+ *    scaled range and whenever ch_tuning asks for a kernel shape.  A step's rounding error
+ *    in fixed point is at most about FP64's relative to the largest |C| of the run (the
+ *    stages hold 62 bits less the recurrences' gain, 2^1 at s = 0.9 and 2^8 at s = 5e4);
+ *    where the field has regions 2^-10 below that (in blocks of 32 columns by 2 rows, bands
+ *    of 8 or 16 rows), where |C| reaches 8 or stays below 2^-200, that part of the run and
+ *    its column solves are computed in FP64, each value to its own relative precision.  CH_FP32 keeps fields,
  *    the stencil and the sweeps in FP32 (sweep coefficients computed in FP64, rounded
  *    once), while the F / dF/dt reductions, beta and its time average stay in FP64.
  */
@@ -548,7 +553,7 @@ typedef struct {
  * Create a server of one precision whose runs' fields fit in hbm_budget_bytes of device
  * memory (two arenas: fields and row-solve scratch, allocated now) with at most
  * max_members runs in flight.  Also allocated now, beside the arenas: the runs' parameter, state and
- * tile tables, the row exponents of CH_FP64 runs (4 bytes per 16 elements of scratch) and the 1 MiB
+ * tile tables, the row exponents of CH_FP64 runs (8 bytes per 16 elements of scratch) and the 1 MiB
  * staging buffer through which CH_FP32 fields are converted.  Errors: CH_EINVAL, CH_ENOMEM, CH_ECUDA.
  */
 int ch_server_create(size_t hbm_budget_bytes, int precision, int max_members, ch_server* out);

@@ -261,8 +261,9 @@ bool fx_tables(double p1, double p2, int S, int n, chk::SegTable* t, int* levels
   const double a = 1.0 - Mn[0], b = -Mn[1], c = -Mn[2], d = 1.0 - Mn[3], det = a * d - b * c;
   const double P[4] = {d / det, -b / det, -c / det, a / det};
   bool ok = true;
-  auto put = [&](chk::FxLimb* to, const double* m) {
+  auto put = [&](chk::FxLimb* to, const double* m, double* fp64 = nullptr) {
     for (int i = 0; i < 4; ++i) {
+      if (fp64) fp64[i] = m[i];
       if (!(std::fabs(m[i]) < 15.0))
         ok = false;
       else
@@ -274,13 +275,13 @@ bool fx_tables(double p1, double p2, int S, int n, chk::SegTable* t, int* levels
   for (int q = 0; q < 5 && (1 << q) < G; ++q) {
     for (double x : Ad)
       if (std::fabs(x) >= 0x1p-62) lv = q + 1;
-    put(t->Ax[q], Ad);
+    put(t->Ax[q], Ad, t->Dx[q]);
     mat2_mul(Ad, Ad, Ad);
   }
-  put(t->Px, ML);
+  put(t->Px, ML, t->Dx[5]);
   double F[4] = {P[0], P[1], P[2], P[3]}, R[4];
   for (int l = 0; l < G; ++l) {
-    put(t->Bx[l], F);
+    put(t->Bx[l], F, t->Dx[6 + l]);
     mat2_mul(MS, F, F);
   }
   put(t->Bx[32], P);
@@ -955,7 +956,7 @@ int create_common(int m, const ch_member_desc* d, int precision, ch_handle* out)
     }
   h->c_points = off;
   h->w_points = h->total_points;
-  const size_t exp_bytes = precision == CH_FP64 ? sizeof(short2) * rows : 0;
+  const size_t exp_bytes = precision == CH_FP64 ? sizeof(chk::RowExp) * rows : 0;
   int rc = build_tiles(h, default_tuning());
   if (rc) {
     delete h;
@@ -1519,14 +1520,14 @@ int ch_debug_row_solve(ch_handle h, int member, double* out) {
   if (h->precision == CH_FP64) {
     if (int rc = copy_out(h, out, static_cast<double*>(h->W) + p.offset, sizeof(double) * np, "read W")) return rc;
     if (p.fx) {  // 64-bit integers with an exponent per row (rows held in FP64: as they are)
-      std::vector<short2> ex(p.ny);
-      if (int rc = copy_out(h, ex.data(), h->view().wexp + p.fx_wexp, sizeof(short2) * ex.size(), "read W")) return rc;
+      std::vector<chk::RowExp> ex(p.ny);
+      if (int rc = copy_out(h, ex.data(), h->view().wexp + p.fx_wexp, sizeof(ex[0]) * ex.size(), "read W")) return rc;
       for (int64_t i = 0; i < np; ++i) {
-        const short2 e = ex[i / p.nx];
-        if (e.y == chk::kBadRow) continue;
+        const chk::RowExp e = ex[i / p.nx];
+        if (e.top == chk::kBadRow) continue;
         long long q;
         std::memcpy(&q, out + i, sizeof q);
-        out[i] = std::ldexp((double)q, e.x);
+        out[i] = std::ldexp((double)q, e.unit);
       }
     }
     for (int64_t i = 0; i < np; ++i) out[i] *= scale;

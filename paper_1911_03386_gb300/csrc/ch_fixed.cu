@@ -28,7 +28,13 @@
 //
 // A band whose largest |C| is outside [2^-200, 8), or not finite, is taken through the same
 // code in FP64 arithmetic (the Fp policy), its rows marked kBadRow; the columns of a member
-// with such a row run in FP64 too.
+// with such a row run in FP64 too.  So do a band in which some block of 32 columns by 2 rows (halo rows
+// included) holds only values below 2^-10 of the band's largest, and the columns of a member whose
+// bands' largest values differ by that much: a value that far below the one that sets its scale would
+// keep fewer bits than in FP64, which shows in regions so quiet beside others (a field grown from a
+// local seed: 1e-12 noise beside it had a relative error of 7e-3 after a step, now FP64's 2e-12).
+// Above that line the error is FP64's or less relative to the run's largest |C|, and within a factor
+// of 16 of it relative to a block's.  Two rows, because one row of a nodal line is no quiet region.
 //
 // Lines of n points are split into G = ceil(n / S) segments of S points (the last one may be
 // shorter), one lane (rows) or warp (columns) per segment.  Each recurrence is a pass from a
@@ -93,7 +99,7 @@ struct Fp {
   static constexpr bool kFixed = false;
   static __device__ __forceinline__ State state(i64 y) { return __longlong_as_double(y); }
   static __device__ __forceinline__ i64 value(State s) { return double_bits(s); }
-  // (a table after tab_to_fp64)
+  // (a table of fp64_tables)
   static __device__ __forceinline__ i64 dot(const FxLimb* row, i64 x0, i64 x1, i64 r) {
     const double* m = reinterpret_cast<const double*>(row);
     return double_bits(fma(m[0], __longlong_as_double(x0), fma(m[1], __longlong_as_double(x1), __longlong_as_double(r))));
@@ -169,13 +175,30 @@ __device__ __forceinline__ void load_tab(ScanTab& t, const SegTable& g) {
     copy16(reinterpret_cast<char*>(&t) + 16 * k, reinterpret_cast<const char*>(&g.Ax[0][0]) + 16 * k);
 }
 
-// The table's entries to FP64, in place (the Fp policy; the caller's barriers order it).
-__device__ __forceinline__ void tab_to_fp64(ScanTab& t) {
-  FxLimb* m = &t.A[0][0];
-  for (int k = threadIdx.x; k < (int)(sizeof(ScanTab) / sizeof(FxLimb)); k += blockDim.x) {
-    const double x = ldexp((double)(((i64)m[k].h << 32) + m[k].l), -58);
-    *reinterpret_cast<double*>(m + k) = x;
+// The Fp policy's tables in place of the fixed-point ones, whose entries are exact to 2^-59: not enough
+// for values that differ by more, which is why a band is in FP64.  Warp 0, lane l segment l; the caller's
+// barriers order it.  Returns the scan's levels.
+__device__ __forceinline__ int fp64_tables(ScanTab& t, const SegTable& g, int G) {
+  if (threadIdx.x < 32) {
+    const int l = threadIdx.x;
+    auto put = [](FxLimb* to, double a, double b, double c, double d) {
+      double* q = reinterpret_cast<double*>(to);
+      q[0] = a;
+      q[1] = b;
+      q[2] = c;
+      q[3] = d;
+    };
+    const double *tail = g.Dx[5], *own = g.Dx[6 + l], *before = g.Dx[6 + max(l - 1, 0)];
+    if (l < 5) put(t.A[l], g.Dx[l][0], g.Dx[l][1], g.Dx[l][2], g.Dx[l][3]);
+    if (l == 5) put(t.P, tail[0], tail[1], tail[2], tail[3]);
+    put(t.B[l], own[0], own[1], own[2], own[3]);
+    if (l == 0)
+      put(t.B[32], own[0], own[1], own[2], own[3]);
+    else  // the last segment's own length, then the others
+      put(t.B[32 + l], fma(tail[0], before[0], tail[1] * before[2]), fma(tail[0], before[1], tail[1] * before[3]),
+          fma(tail[2], before[0], tail[3] * before[2]), fma(tail[2], before[1], tail[3] * before[3]));
   }
+  return 32 - __clz(G - 1);
 }
 
 // Programmatic dependent launch: a step kernel lets its successor start (its CTAs take the SMs'
@@ -387,6 +410,10 @@ __device__ __forceinline__ void row_solve(i64* seg, int len, int l, int G, int g
 // CTA, so that a member's samples do not depend on the CTA size that its company leads to.
 __device__ __forceinline__ int sample_warps(const MemberParams& P) { return P.fx == 1 ? 2 : P.fx == 2 ? 4 : 8; }
 
+// Exponents by which a block's largest |C| may lie below the band's (a band's below the member's) of
+// |C| < 2^E: less where the cubic term takes bits from mu.
+__device__ __forceinline__ int quiet_line(int E) { return 10 - 3 * max(0, E - 1); }
+
 template <int TH, int MINB>
 __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_base) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -434,19 +461,27 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
     }
   }
   asm volatile("cp.async.wait_all;\n" ::: "memory");
-  unsigned top = 0;
+  unsigned top = 0, low = ~0u;  // of the blocks' largest |C|, the largest and the least (high words)
   for (int s = warp; s < b.ns; s += NW) {  // this thread's own copies
     const int i = min(32 * s + lane, nx - 1);
     const int2* col = reinterpret_cast<const int2*>(b.tile + i + (i >> b.ls));
-#pragma unroll 4
-    for (int t = 0; t < nr + 4; ++t) top = max(top, (unsigned)col[t * b.pitch].y & 0x7fffffffu);
+#pragma unroll 2
+    for (int t = 0; t < nr + 4; t += 2) {
+      const int2* at = col + min(t, nr + 2) * b.pitch;
+      const unsigned block = __reduce_max_sync(kAll, (unsigned)max(at[0].y & 0x7fffffff, at[b.pitch].y & 0x7fffffff));
+      top = max(top, block);
+      low = min(low, block);
+    }
   }
-  top = __reduce_max_sync(kAll, top);
-  if (lane == 0) wtop[warp] = top;
+  if (lane == 0) {
+    wtop[warp] = top;
+    wtop[NW + warp] = low;
+  }
   __syncthreads();
   top = __reduce_max_sync(kAll, lane < NW ? wtop[lane] : 0u);
+  low = __reduce_min_sync(kAll, lane < NW ? wtop[NW + lane] : ~0u);
   const int emax = (int)(top >> 20);  // biased exponent of the largest |C|
-  const bool bad = emax > 1022 + kFxMaxE || emax < 823;
+  const bool bad = emax > 1022 + kFxMaxE || emax < 823 || (int)(low >> 20) + quiet_line(emax - 1022) < emax;
   const int cut = !bad && emax > 1023 ? P.fx_cut[emax - 1024] : 0, kmu = P.fx_kmu - cut, su = P.fx_su + cut;
   // the strips' edge columns
   for (int k = threadIdx.x; k < 2 * b.ns * (nr + 4); k += TH) {
@@ -457,8 +492,9 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
   }
   __syncthreads();
   int up = 0;  // R' is held times 2^(kmu + up - E)
+  int levels = P.fx_lvx;
   if (bad) {
-    tab_to_fp64(tab);
+    levels = fp64_tables(tab, v.seg[tl.member], G);
     RhsFp rhs{P.fx_tall != 0, P.fx_ratio, P.fx_w0};
     band_rhs<NW, -1>(b, Es, Em, top, emax, MuFp{P.a, P.bx, P.by}, rhs, wtop + 4 * NW);
   } else
@@ -489,12 +525,13 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
   const bool full = nx % S == 0;
   int e_lsb, e_top;
   if (bad)
-    row_solve<NW>(seg, len, l, G, gw, P.fx_lvx, full, Fp(P.fx_cx, P.p1x, P.p2x), tab, 0, 0u, wtop + NW, e_lsb, e_top);
+    row_solve<NW>(seg, len, l, G, gw, levels, full, Fp(P.fx_cx, P.p1x, P.p2x), tab, 0, 0u, wtop + NW, e_lsb, e_top);
   else
-    row_solve<NW>(seg, len, l, G, gw, P.fx_lvx, full, Fx(P.fx_cx, 0.0, 0.0), tab, P.fx_gainx, top, wtop + NW, e_lsb, e_top);
+    row_solve<NW>(seg, len, l, G, gw, levels, full, Fx(P.fx_cx, 0.0, 0.0), tab, P.fx_gainx, top, wtop + NW, e_lsb, e_top);
   if (row < nr && l == 0) {
     const int eb = emax - 1022 - kmu - up;
-    v.wexp[P.fx_wexp + j0 + row] = bad ? make_short2(0, kBadRow) : make_short2((short)(e_lsb + eb), (short)(e_top + eb));
+    v.wexp[P.fx_wexp + j0 + row] = bad ? RowExp{0, (short)kBadRow, (short)(emax - 1022), 0}
+                                       : RowExp{(short)(e_lsb + eb), (short)(e_top + eb), (short)(emax - 1022), 0};
   }
   // W to HBM as whole rows (row_solve ends with a barrier)
   i64* Wg = static_cast<i64*>(v.W) + P.offset + (int64_t)j0 * nx;
@@ -594,7 +631,7 @@ __device__ __forceinline__ void col_update(const A& ar, const i64* y, int len, d
 // segment.  Rows come in bands of one exponent that start at multiples of 8 (ws: the segment's
 // row exponents).
 template <class A, class Scaled>
-__device__ __forceinline__ void col_first(const A& ar, i64* y, int len, int S, const short2* ws,
+__device__ __forceinline__ void col_first(const A& ar, i64* y, int len, int S, const RowExp* ws,
                                           typename A::State& a, typename A::State& b, const Scaled& scaled) {
   a = A::zero();
   b = A::zero();
@@ -648,15 +685,15 @@ __global__ void __launch_bounds__(kColThreads, 3) fx_cols_kernel(DevView v, int 
   const int64_t base = (int64_t)min(seg, G - 1) * S * nx + tl.start + (cv ? c : 0);
   i64* y = reinterpret_cast<i64*>(smem) + threadIdx.x;
   double* Cg = static_cast<double*>(v.C) + P.offset + base;
-  const short2* we = v.wexp + P.fx_wexp;
-  const short2* ws = we + min(seg, G - 1) * S;
+  const RowExp* we = v.wexp + P.fx_wexp;
+  const RowExp* ws = we + min(seg, G - 1) * S;
   // All of the panel's W in flight in up to 4 groups of rows of every segment (value u of segment g
   // at u 256 + g cw, so a row piece of the panel is contiguous on both sides), in 16-byte pieces
   // where the rows allow it; C on its way to L2 for the update.
-  // the row exponents' maxima, 8 loads ahead of the copies (ny <= 256; the rest below)
-  short2 we8[8];
+  // the bands' exponents (of every eighth row: bands start at multiples of 8), 4 loads ahead of the copies
+  RowExp we4[4];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) we8[k] = we[min(lane + 32 * k, ny - 1)];
+  for (int k = 0; k < 4; ++k) we4[k] = we[min(8 * (lane + 32 * k), ny - 1)];
   {
     i64* Y = reinterpret_cast<i64*>(smem);
     const bool wide = !((nx | tl.count) & 1);
@@ -689,33 +726,38 @@ __global__ void __launch_bounds__(kColThreads, 3) fx_cols_kernel(DevView v, int 
       if (tl.count > 16) prefetch_l2(p + 128);
     }
   }
-  int emax = -32768;
+  int emax = -32768, Emax = -32768, Emin = 32767;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) emax = max(emax, (int)we8[k].y);
-  for (int j = lane + 256; j < ny; j += 32) emax = max(emax, (int)we[j].y);
+  for (int k = 0; k < 4; ++k) {
+    emax = max(emax, (int)we4[k].top);
+    Emax = max(Emax, (int)we4[k].E);
+    Emin = min(Emin, (int)we4[k].E);
+  }
   emax = __reduce_max_sync(kAll, emax);
-  const bool bad = emax == kBadRow;
+  Emax = __reduce_max_sync(kAll, Emax);
+  Emin = __reduce_min_sync(kAll, Emin);
+  const bool bad = emax == kBadRow || Emin + quiet_line(Emax) < Emax;
   i64* const ye = y + max(len - 1, 0) * kColThreads;
   double* const Ce = Cg + (int64_t)max(len - 1, 0) * nx;
   if (bad) {
     Fp ar(P.fx_cy, P.p1y, P.p2y);
     double a, b;
-    col_first(ar, y, len, S, ws, a, b, [](short2 e, auto f) {
-      if (e.y == kBadRow) {
+    col_first(ar, y, len, S, ws, a, b, [](RowExp e, auto f) {
+      if (e.top == kBadRow) {
         f([](i64 w) { return w; });
       } else {
-        const double unit = pow2(e.x);  // e.x >= -400: no subnormal
+        const double unit = pow2(e.unit);  // above -500: no subnormal
         f([unit](i64 w) { return double_bits(unit * (double)w); });
       }
     });
-    tab_to_fp64(tab);
-    col_solve(ar, y, len, tab, xs, wtop, G, gw, P.fx_lvy, ny % S == 0, cw, 0, a, b);
+    const int levels = fp64_tables(tab, v.segy[tl.member], G);
+    col_solve(ar, y, len, tab, xs, wtop, G, gw, levels, ny % S == 0, cw, 0, a, b);
     col_update(ar, ye, len, Ce, nx, P.fx_kappa, cv, a, b, [](i64 t) { return __longlong_as_double(t); });
   } else {
     Fx ar(P.fx_cy, 0.0, 0.0);
     FxLimb a, b;
     const int up = 62 - gain - emax;
-    col_first(ar, y, len, S, ws, a, b, [up](short2 e, auto f) { with_shift(max(-62, min(62, up + (int)e.x)), f); });
+    col_first(ar, y, len, S, ws, a, b, [up](RowExp e, auto f) { with_shift(max(-62, min(62, up + (int)e.unit)), f); });
     const int sl = col_solve(ar, y, len, tab, xs, wtop, G, gw, P.fx_lvy, ny % S == 0, cw, gain, a, b);
     col_update(ar, ye, len, Ce, nx, P.fx_kappa * ldexp(1.0, -up - sl), cv, a, b, [](i64 t) { return (double)t; });
   }

@@ -93,7 +93,7 @@ struct ch_ensemble {
     v.segy = dsegy;
     v.colseg_tiles = dcst;
     v.res_tiles = dres;
-    v.wexp = reinterpret_cast<short2*>(static_cast<char*>(W) + elt * w_points);
+    v.wexp = reinterpret_cast<chk::RowExp*>(static_cast<char*>(W) + elt * w_points);
     v.m = m;
     return v;
   }

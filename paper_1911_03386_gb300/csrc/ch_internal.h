@@ -10,7 +10,7 @@
 //   col_tiles   Tile[]            one CTA of the column kernel per tile (a column panel);
 //   partials    double2[]         FP64 (sum F density, sum dF/dt density) per row band;
 //   series      double[m][cap][4] ring of (t, F, dF/dt, beta) samples per member;
-//   wexp        short2[]          row exponents of W (fixed-point form, behind W).
+//   wexp        RowExp[]          row exponents of W (fixed-point form, behind W).
 #pragma once
 
 #include <cstdint>
@@ -30,7 +30,12 @@ struct FxCoef {
   FxLimb p1, p2;         // recurrence coefficients / 8, times 2^64
 };
 constexpr int kFxMaxE = 3;        // |C| < 2^E up to here in fixed point
-constexpr int kBadRow = 32767;    // row exponent of a row held in FP64
+constexpr int kBadRow = 32767;    // RowExp::top of a row held in FP64
+// Exponents of a row of W in fixed point: of its unit, of its largest value, and E of its band (its
+// largest |C| is in [2^(E-1), 2^E)).
+struct alignas(8) RowExp {
+  short unit, top, E, pad;
+};
 constexpr int kFxRowClasses = 4;  // nx <= 64, 128, 512, 1024
 
 struct MemberParams {
@@ -105,16 +110,21 @@ struct SegTable {
     double B[64][4];     // up to 64 segments: columns over a CTA pair (rows use at most 32)
     FxLimb Bx[64][4];
   };
-  float Af[5][4];        // the same rounded to FP32
-  float Bf[64][4];
-  float Pf[4];
-  // Closed-form responses of one segment of S <= 32 points (cluster-resident column
-  // kernel), FP32: Hf[u] = (g1_u, g2_u, k1_u, k2_u) where, on a segment with start states
-  // s = (y_-1, y_-2) of the forward and t = (x_S, x_S+1) of the backward recurrence,
-  // x_u = G0(F0(r))_u + g1_u s_0 + g2_u s_1 + k1_u t_0 + k2_u t_1 (F0, G0: the forward and
-  // backward recurrences from zero states; g = G0 of the forward homogeneous responses,
-  // k = the backward homogeneous responses).
-  float Hf[32][4];
+  union {
+    struct {
+      float Af[5][4];        // the same rounded to FP32
+      float Bf[64][4];
+      float Pf[4];
+      // Closed-form responses of one segment of S <= 32 points (cluster-resident column
+      // kernel), FP32: Hf[u] = (g1_u, g2_u, k1_u, k2_u) where, on a segment with start states
+      // s = (y_-1, y_-2) of the forward and t = (x_S, x_S+1) of the backward recurrence,
+      // x_u = G0(F0(r))_u + g1_u s_0 + g2_u s_1 + k1_u t_0 + k2_u t_1 (F0, G0: the forward and
+      // backward recurrences from zero states; g = G0 of the forward homogeneous responses,
+      // k = the backward homogeneous responses).
+      float Hf[32][4];
+    };
+    double Dx[38][4];    // fixed-point form: Ax (5), Px and Bx (the first 32) in FP64, for bands out of its range
+  };
 };
 
 struct MemberState {
@@ -151,7 +161,7 @@ struct DevView {
   const SegTable* segy;  // [m] scan tables of the y recurrence (segment form of the column kernel)
   const Tile* colseg_tiles;  // CTAs of the segment-form column kernel
   const Tile* res_tiles;     // one per member of the cluster-resident form (FP32)
-  short2* wexp;              // fixed-point form: per row of W, the exponent of its unit and of its largest value
+  RowExp* wexp;              // fixed-point form: per row of W
   int m;
 };
 

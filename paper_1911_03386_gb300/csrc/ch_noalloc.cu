@@ -55,7 +55,7 @@ struct FixedTables {
   chk::SegTable seg, segy;
   chk::Tile rows[128], cols[128];
   double2 partials[128];
-  short2 wexp[1024];
+  chk::RowExp wexp[1024];
 };
 static __device__ FixedTables g_noalloc_fixed;
 

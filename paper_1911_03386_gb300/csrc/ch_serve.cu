@@ -384,7 +384,7 @@ int ch_server_create(size_t hbm_budget_bytes, int precision, int max_members, ch
     return cleanup(CH_ECUDA, std::string("stream: ") + cudaGetErrorString(e));
   h->stream = h->own;
   h->w_points = elems;
-  const size_t exp_bytes = precision == CH_FP64 ? sizeof(short2) * (elems / kRowElems) : 0;
+  const size_t exp_bytes = precision == CH_FP64 ? sizeof(chk::RowExp) * (elems / kRowElems) : 0;
   if ((e = chk::dev_malloc(&h->C, elt * elems)) != cudaSuccess ||
       (e = chk::dev_malloc(&h->W, elt * elems + exp_bytes)) != cudaSuccess ||
       (e = chk::dev_malloc((void**)&h->dmp, sizeof(MemberParams) * max_members)) != cudaSuccess ||

@@ -155,6 +155,34 @@ def test_no_less_precise_than_fp64_at_large_values(nx, ny, start, scale):
     assert fixed[1] <= 2.0 * fp64[1]
 
 
+# the active part: a quarter of the box, some columns, some rows
+@pytest.mark.parametrize("part", [(slice(0, 0.5), slice(0, 0.5)), (slice(0, 1), slice(0.25, 0.5)), (slice(0.5, 0.75), slice(0, 1))])
+@pytest.mark.parametrize("nx,ny,s", [(128, 128, 0.9), (256, 200, 0.9), (130, 97, 0.5), (64, 64, 0.05), (600, 48, 10.0)])
+def test_quiet_regions_keep_their_own_precision(nx, ny, s, part):
+    # 1e-12 of the rest: relative error there against the FP64 kernels'.  Both forms carry the active
+    # part's tail there in FP64 with a relative error that grows by a rounding per point, along one
+    # recurrence (the FP64 kernels) or in segments and their matrices' powers: factors of 2 and 4 for that
+    L = TWO_PI
+    dt = s * (L / max(nx, ny)) ** 4 / 0.01
+    rows, cols = (slice(round(p.start * n), round(p.stop * n)) for p, n in zip(part, (ny, nx)))
+    f = 1e-12 * (2 * np.random.default_rng(nx).random((ny, nx)) - 1)
+    f[rows, cols] = separated(ny, nx)[rows, cols]
+    ref = steps_extended(f, L, 0.01, dt, 1)
+    quiet = np.abs(ref) < 1e-10
+    assert np.any(quiet)
+    rel = []
+    for t in ({}, dict(split=1)):
+        with ch.Ensemble.create(nx, ny, L, 0.01, dt, [0.0], 1, ch.CH_FP64) as e:
+            if t:
+                e.set_tuning(**t)
+            e.set_field(0, f)
+            e.step(1)
+            r = np.abs(e.field(0) - ref)[quiet] / 1e-12
+            rel.append((float(np.sqrt(np.mean(r * r))), float(np.max(r))))
+    assert rel[0][0] <= 2.0 * rel[1][0]
+    assert rel[0][1] <= 4.0 * rel[1][1]
+
+
 @pytest.mark.parametrize("scale", [0.9, 2.5, 7.0])
 def test_samples_at_large_values(scale):
     # F and dF/dt against the FP64 kernels: both round sums of 4096 terms of one sign
