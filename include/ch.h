@@ -188,10 +188,9 @@ int ch_launch_phase(ch_handle h, int phase);
  * (split: -1) take the precision's default.  With every field at its default, CH_FP64 members
  * of 16 to 1024 points per axis and gamma dt / h^4 up to about 5e4 run in the fixed-point form,
  * whose shapes follow from the member's size alone; setting a field (other than the CH_FP32
- * ones, resident and resident_rows, and col_seg = -1, the CH_FP64 default) selects the FP64 kernels
- * described here.  ch_get_tuning reports member 0: defaults (col_seg and resident -1) where it runs
- * in the fixed-point form, which passing them back keeps, else the shape in effect, which passing
- * back makes explicit for every member.
+ * ones, resident and resident_rows) selects the FP64 kernels described here.  ch_get_tuning
+ * reports these kernels' shape, also where members run in the fixed-point form, which has no
+ * field; on a handle with such members a request that equals its report changes nothing.
  *   split       1: stencil and row sweep as separate kernels (default for CH_FP64: all
  *               threads of the stencil kernel do FP64 work, the sweeps run as many
  *               independent recurrences per SM); 0: one fused row kernel (default for

@@ -621,7 +621,7 @@ int build_tiles(ch_ensemble* h, const ch_tuning& t) {
   };
   // fixed-point form (CH_FP64): every member it applies to, unless the tuning asks for a shape
   // of the other forms
-  const bool fx_on = f64 && (t.split < 0 || h->fx_fused) && t.stream < 0 && t.persist <= 0 && t.row_seg == 0 && t.col_seg <= 0 &&
+  const bool fx_on = f64 && (t.split < 0 || h->fx_fused) && t.stream < 0 && t.persist <= 0 && t.row_seg == 0 && t.col_seg == 0 &&
                      t.rows_band == 0 && t.rows_p == 0 && t.sweep_band == 0 && t.cols_panel == 0 && t.cols_p == 0 &&
                      t.threads == 0 && t.preroll_head == 0;
   int cwarps[4] = {8, 8, max_wp, max_wp};  // warps per CTA of each class
@@ -1428,6 +1428,10 @@ int ch_set_tuning(ch_handle h, const ch_tuning* t) {
     return fail(CH_EINVAL, "resident_rows must be 0, 32 or 64");
   if (req.preroll_head < -1 || req.preroll_head > 0) return fail(CH_EINVAL, "preroll_head must be -1 or 0");
   CH_CUDA(cudaStreamSynchronize(h->stream), "synchronise");
+  // with members in the fixed-point form, which has no field: the report of ch_get_tuning passed back
+  // keeps the shape in effect
+  ch_tuning now;
+  if (h->shape.fx_tiles > 0 && ch_get_tuning(h, &now) == CH_OK && std::memcmp(&now, &req, sizeof now) == 0) return CH_OK;
   const std::vector<MemberParams> saved = h->hp;
   const ch_tuning old = h->tuning;
   if (int rc = build_tiles(h, req)) {
@@ -1442,14 +1446,6 @@ int ch_set_tuning(ch_handle h, const ch_tuning* t) {
 int ch_get_tuning(ch_handle h, ch_tuning* t) {
   if (int rc = check_handle(h)) return rc;
   if (!t) return fail(CH_EINVAL, "t is NULL");
-  if (h->hp[0].fx) {
-    // fixed-point form: it has no fields of its own and runs under the defaults, so these are what a
-    // caller can pass back to keep it (col_seg -1 and 0 are the same request for CH_FP64)
-    *t = default_tuning();
-    t->persist = 0;
-    t->col_seg = t->resident = -1;
-    return CH_OK;
-  }
   // the shape in effect, with per-member values of member 0
   t->split = h->shape.split;
   t->rows_band = h->rt.empty() ? 0 : h->rt[0].count;
