@@ -29,7 +29,7 @@
  *    scaled range and whenever ch_tuning asks for a kernel shape.  A step's rounding error
  *    in fixed point is at most about FP64's relative to the largest |C| of the run (the
  *    stages hold 62 bits less the recurrences' gain, 2^1 at s = 0.9 and 2^8 at s = 5e4);
- *    where the field has regions 2^-10 below that (in blocks of 32 columns by 2 rows, bands
+ *    where the field has regions 2^-10 below that (in blocks of 32 columns by 4 rows, bands
  *    of 8 or 16 rows), where |C| reaches 8 or stays below 2^-200, that part of the run and
  *    its column solves are computed in FP64, each value to its own relative precision.  CH_FP32 keeps fields,
  *    the stencil and the sweeps in FP32 (sweep coefficients computed in FP64, rounded

@@ -28,13 +28,14 @@
 //
 // A band whose largest |C| is outside [2^-200, 8), or not finite, is taken through the same
 // code in FP64 arithmetic (the Fp policy), its rows marked kBadRow; the columns of a member
-// with such a row run in FP64 too.  So do a band in which some block of 32 columns by 2 rows (halo rows
+// with such a row run in FP64 too.  So do a band in which some block of 32 columns by 4 rows (halo rows
 // included) holds only values below 2^-10 of the band's largest, and the columns of a member whose
 // bands' largest values differ by that much: a value that far below the one that sets its scale would
 // keep fewer bits than in FP64, which shows in regions so quiet beside others (a field grown from a
 // local seed: 1e-12 noise beside it had a relative error of 7e-3 after a step, now FP64's 2e-12).
 // Above that line the error is FP64's or less relative to the run's largest |C|, and within a factor
-// of 16 of it relative to a block's.  Two rows, because one row of a nodal line is no quiet region.
+// of 16 of it relative to a block's.  Four rows: a nodal line of one or two rows is no quiet region, and the
+// two rows next to an active one take its flux within the step.
 //
 // Lines of n points are split into G = ceil(n / S) segments of S points (the last one may be
 // shorter), one lane (rows) or warp (columns) per segment.  Each recurrence is a pass from a
@@ -177,8 +178,8 @@ __device__ __forceinline__ void load_tab(ScanTab& t, const SegTable& g) {
 
 // The Fp policy's tables in place of the fixed-point ones, whose entries are exact to 2^-59: not enough
 // for values that differ by more, which is why a band is in FP64.  Warp 0, lane l segment l; the caller's
-// barriers order it.  Returns the scan's levels.
-__device__ __forceinline__ int fp64_tables(ScanTab& t, const SegTable& g, int G) {
+// barriers order it.  The scans take all levels: no power vanishes.
+__device__ __forceinline__ void fp64_tables(ScanTab& t, const SegTable& g) {
   if (threadIdx.x < 32) {
     const int l = threadIdx.x;
     auto put = [](FxLimb* to, double a, double b, double c, double d) {
@@ -198,8 +199,8 @@ __device__ __forceinline__ int fp64_tables(ScanTab& t, const SegTable& g, int G)
       put(t.B[32 + l], fma(tail[0], before[0], tail[1] * before[2]), fma(tail[0], before[1], tail[1] * before[3]),
           fma(tail[2], before[0], tail[3] * before[2]), fma(tail[2], before[1], tail[3] * before[3]));
   }
-  return 32 - __clz(G - 1);
 }
+__device__ __forceinline__ int all_levels(int G) { return 32 - __clz(G - 1); }
 
 // Programmatic dependent launch: a step kernel lets its successor start (its CTAs take the SMs'
 // free slots, read their constant tables and wait) and waits itself until its predecessor has
@@ -466,9 +467,12 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
     const int i = min(32 * s + lane, nx - 1);
     const int2* col = reinterpret_cast<const int2*>(b.tile + i + (i >> b.ls));
 #pragma unroll 2
-    for (int t = 0; t < nr + 4; t += 2) {
-      const int2* at = col + min(t, nr + 2) * b.pitch;
-      const unsigned block = __reduce_max_sync(kAll, (unsigned)max(at[0].y & 0x7fffffff, at[b.pitch].y & 0x7fffffff));
+    for (int t = 0; t < nr + 4; t += 4) {
+      const int2* at = col + min(t, nr) * b.pitch;  // the last block may overlap the one before
+      unsigned block = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) block = max(block, (unsigned)at[q * b.pitch].y & 0x7fffffffu);
+      block = __reduce_max_sync(kAll, block);
       top = max(top, block);
       low = min(low, block);
     }
@@ -482,7 +486,7 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
   low = __reduce_min_sync(kAll, lane < NW ? wtop[NW + lane] : ~0u);
   const int emax = (int)(top >> 20);  // biased exponent of the largest |C|
   const bool bad = emax > 1022 + kFxMaxE || emax < 823 || (int)(low >> 20) + quiet_line(emax - 1022) < emax;
-  const int cut = !bad && emax > 1023 ? P.fx_cut[emax - 1024] : 0, kmu = P.fx_kmu - cut, su = P.fx_su + cut;
+  auto cut_bits = [&] { return emax > 1023 ? P.fx_cut[emax - 1024] : 0; };  // (in range)
   // the strips' edge columns
   for (int k = threadIdx.x; k < 2 * b.ns * (nr + 4); k += TH) {
     const int e = k / (nr + 4), t = k - e * (nr + 4);
@@ -492,12 +496,12 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
   }
   __syncthreads();
   int up = 0;  // R' is held times 2^(kmu + up - E)
-  int levels = P.fx_lvx;
   if (bad) {
-    levels = fp64_tables(tab, v.seg[tl.member], G);
+    fp64_tables(tab, v.seg[tl.member]);
     RhsFp rhs{P.fx_tall != 0, P.fx_ratio, P.fx_w0};
     band_rhs<NW, -1>(b, Es, Em, top, emax, MuFp{P.a, P.bx, P.by}, rhs, wtop + 4 * NW);
-  } else
+  } else {
+    const int cut = cut_bits(), su = P.fx_su + cut;
     with_shift(max(-62, 2 * (emax - 1022) + 6 - su), [&](auto sh) {  // C^2 vanishes long before -62
       const i64 one = 1ll << (60 - su);
       const FxLimb bx = cut_limb(P.fx_bx, cut), by = cut_limb(P.fx_by, cut);
@@ -515,6 +519,7 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
         fixed(MuFx<false, decltype(sh)>{bx, by, one, sh}, RhsFx<2>{P.fx_rl, P.fx_er},
               std::integral_constant<int, 2>());
     });
+  }
   if (sample)
     band_partials_field<double>(v, tl, nx, nr, P, v.partials + P.partial_base + tl.index, red, sample_warps(P));
 
@@ -525,11 +530,11 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
   const bool full = nx % S == 0;
   int e_lsb, e_top;
   if (bad)
-    row_solve<NW>(seg, len, l, G, gw, levels, full, Fp(P.fx_cx, P.p1x, P.p2x), tab, 0, 0u, wtop + NW, e_lsb, e_top);
+    row_solve<NW>(seg, len, l, G, gw, all_levels(G), full, Fp(P.fx_cx, P.p1x, P.p2x), tab, 0, 0u, wtop + NW, e_lsb, e_top);
   else
-    row_solve<NW>(seg, len, l, G, gw, levels, full, Fx(P.fx_cx, 0.0, 0.0), tab, P.fx_gainx, top, wtop + NW, e_lsb, e_top);
+    row_solve<NW>(seg, len, l, G, gw, P.fx_lvx, full, Fx(P.fx_cx, 0.0, 0.0), tab, P.fx_gainx, top, wtop + NW, e_lsb, e_top);
   if (row < nr && l == 0) {
-    const int eb = emax - 1022 - kmu - up;
+    const int eb = bad ? 0 : emax - 1022 - P.fx_kmu + cut_bits() - up;
     v.wexp[P.fx_wexp + j0 + row] = bad ? RowExp{0, (short)kBadRow, (short)(emax - 1022), 0}
                                        : RowExp{(short)(e_lsb + eb), (short)(e_top + eb), (short)(emax - 1022), 0};
   }
@@ -750,8 +755,8 @@ __global__ void __launch_bounds__(kColThreads, 3) fx_cols_kernel(DevView v, int 
         f([unit](i64 w) { return double_bits(unit * (double)w); });
       }
     });
-    const int levels = fp64_tables(tab, v.segy[tl.member], G);
-    col_solve(ar, y, len, tab, xs, wtop, G, gw, levels, ny % S == 0, cw, 0, a, b);
+    fp64_tables(tab, v.segy[tl.member]);
+    col_solve(ar, y, len, tab, xs, wtop, G, gw, all_levels(G), ny % S == 0, cw, 0, a, b);
     col_update(ar, ye, len, Ce, nx, P.fx_kappa, cv, a, b, [](i64 t) { return __longlong_as_double(t); });
   } else {
     Fx ar(P.fx_cy, 0.0, 0.0);

@@ -101,6 +101,7 @@ GRIDS = [(33, 512, TWO_PI), (17, 600, TWO_PI), (17, 1000, TWO_PI), (140, 513, 51
 @pytest.mark.parametrize("nx,ny,L", GRIDS)
 def test_no_less_precise_than_fp64_at_any_aspect_ratio(nx, ny, L, start):
     fixed, fp64 = errors(start(ny, nx), L, 0.01, 5e-4, 2)
+    assert fixed != fp64  # another form ran
     assert fixed[0] <= 1.25 * fp64[0]
     assert fixed[1] <= 2.0 * fp64[1]
 
@@ -151,6 +152,7 @@ def test_no_less_precise_than_fp64_at_large_values(nx, ny, start, scale):
     f = start(ny, nx)
     f *= scale / np.max(np.abs(f))
     fixed, fp64 = errors(f, nx * TWO_PI / 128, 0.01, 2e-6, 2)
+    assert fixed != fp64
     assert fixed[0] <= 1.25 * fp64[0]
     assert fixed[1] <= 2.0 * fp64[1]
 
