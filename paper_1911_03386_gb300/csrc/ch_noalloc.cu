@@ -80,14 +80,18 @@ __global__ void noalloc_fixed_setup(FixedSetup s, FixedTables* t, int band) {
   if (k * cw < nx) t->cols[k] = chk::Tile{0, k * cw, min(cw, nx - k * cw), k, 0, 0};
 }
 
+cudaError_t scratch_address(double** out);
+
 // nsteps steps of the fixed-point kernels; false where the form does not apply.
-bool step_fixed(double* C, double* W, const ch_member_desc& d, int64_t nsteps, cudaStream_t st, int* rc) {
+bool step_fixed(double* C, const ch_member_desc& d, int64_t nsteps, cudaStream_t st, int* rc) {
   FixedSetup s;
   if (chh::fill_params(d, CH_FP64, &s.mp) != CH_OK || !chh::fx_params(&s.mp, &s.seg, &s.segy)) return false;
   if (s.mp.fx_gainx > 6 || s.mp.fx_gainy > 6) return false;
   *rc = CH_ECUDA;
+  double* W = nullptr;
   FixedTables* t = nullptr;
-  if (cudaGetSymbolAddress(reinterpret_cast<void**>(&t), g_noalloc_fixed) != cudaSuccess ||
+  if (scratch_address(&W) != cudaSuccess ||
+      cudaGetSymbolAddress(reinterpret_cast<void**>(&t), g_noalloc_fixed) != cudaSuccess ||
       chk::set_fx_smem_limits() != cudaSuccess)
     return true;
   s.mp.every = INT_MAX;
@@ -270,8 +274,6 @@ extern "C" int ch_step_field_noalloc(double* C, int nx, int ny, double L, double
     return na_fail(CH_EINVAL, "ch_step_field_noalloc: nx*ny exceeds the 1048576-point (1024x1024) scratch limit");
   if (!(L > 0.0) || !(gamma > 0.0) || !(dt > 0.0) || !(L < 1e300) || !(gamma < 1e300) || !(dt < 1e300))
     return na_fail(CH_EINVAL, "L, gamma and dt must be finite and > 0");
-  double* W = nullptr;
-  if (scratch_address(&W) != cudaSuccess) return na_fail(CH_ECUDA, "scratch set-up failed");
   {
     ch_member_desc d{};
     d.nx = nx;
@@ -280,7 +282,7 @@ extern "C" int ch_step_field_noalloc(double* C, int nx, int ny, double L, double
     d.gamma = gamma;
     d.dt = dt;
     int rc = CH_OK;
-    if (step_fixed(C, W, d, nsteps, static_cast<cudaStream_t>(stream), &rc))
+    if (step_fixed(C, d, nsteps, static_cast<cudaStream_t>(stream), &rc))
       return rc == CH_OK ? CH_OK : na_fail(rc, "ch_step_field_noalloc: launch failed");
   }
   StepConsts P;
@@ -308,6 +310,8 @@ extern "C" int ch_step_field_noalloc(double* C, int nx, int ny, double L, double
   if (rows_smem > kSmemMax || cols_smem > kSmemMax) return na_fail(CH_EINVAL, "grid line too long");
   P.br = br;
   P.bc = bc;
+  double* W = nullptr;
+  if (scratch_address(&W) != cudaSuccess) return na_fail(CH_ECUDA, "scratch set-up failed");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int row_blocks = (ny + br - 1) / br, col_blocks = (nx + bc - 1) / bc;
   // Launch errors are read with cudaPeekAtLastError, which leaves the error state as it
