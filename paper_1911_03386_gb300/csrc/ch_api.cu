@@ -324,9 +324,9 @@ void fx_mu_params(MemberParams* p) {
   p->fx_w0 = -2.0 * (1.0 + p->fx_ratio);
   p->fx_kappa = p->fx_tall ? p->dt / (p->hy * p->hy * p->cx * p->cy) : p->kappa;
   // |C| < 2^E: |mu| / 2^E <= max(3, 4^E - 1) + 4 (bx + by) and |R'| <= 4 (1 + ratio) |mu|, which has
-  // to fit 62 bits (60 where R' takes a product).  (C^2 - 1) 2^(60 - su) fits 62 bits if su >= 2 E - 2.  The ratio is at most 1 whatever the grid: with
-  // rho = (hx / hy)^2 in its place a tall grid's headroom came out of mu (17 x 600: 39 bits of mu and
-  // 94 times the FP64 kernels' error on a separated field).
+  // to fit 62 bits (60 where R' takes a product); (C^2 - 1) 2^(60 - su) fits 62 bits if su >= 2 E - 2.
+  // The ratio is at most 1 whatever the grid: with rho = (hx / hy)^2 in its place a tall grid's headroom
+  // came out of mu (17 x 600: 39 bits of mu and 94 times the FP64 kernels' error on a separated field).
   auto bound = [&](int E) { return 4.0 * (1.0 + p->fx_ratio) * (std::ldexp(1.0, 2 * E) - 1.0 + 4.0 * (p->bx + p->by)); };
   auto kmu = [&](int E) {
     return std::min(57 - 2 * E, (p->fx_square ? 62 : 60) - (int)std::ceil(std::log2(bound(E))));

@@ -4,38 +4,40 @@
 // costs a warp 38 SM clocks; the same step in 64-bit fixed point (six 32 x 32 -> 64 bit
 // multiply-adds and a few adds) costs 8.7 (measured, 16 or more warps per SM).  The step of a
 // CH_FP64 member is therefore formed in 64-bit integers with power-of-two scales taken from
-// the data, which hold 59 to 63 significant bits where FP64 holds 53; the fields stay FP64 in
-// memory and the update C += kappa Z is one FP64 FMA.
+// the data: C enters with 59 bits below its band's scale, the solves hold 62 bits less the
+// recurrences' gain (2^1 at s = 0.9, 2^5 at s = 900, 2^8 at s = 5e4), where FP64 holds 53; the
+// fields stay FP64 in memory and the update C += kappa Z is one FP64 FMA.
 //
 //   fx_rows_kernel   a band of rows: C -> mu -> R' -> both row recurrences -> W (64-bit
 //                    integers, one exponent per row)
 //   fx_cols_kernel   a panel of up to 32 columns: both column recurrences of W, C += kappa Z
 //
-// Measured (us per step of a whole ensemble, the FP64 kernels before): 256 x 256^2 rows 219 +
-// columns 136 = 0.347 ms (stencil 0.334 + rows 0.196 + columns 0.241 = 0.762 ms); 16 x 1024^2
-// 0.406 ms (1.43 ms); 64^2 alone 14.6 us (70 us).  At 256^2 a point takes about 290 instructions of
-// the row kernel and 170 of the column kernel; both are bound by issue slots and the integer
-// multiply pipe (56 % and 44 % of the issue slots used), not by HBM (40 bytes per point, 0.1 ms).
+// Measured (a step of a whole ensemble; in brackets the FP64 kernels): 256 x 256^2 rows 212 + columns
+// 138 us, 0.352 ms (0.650 ms), 16 x 1024^2 0.402 ms (1.16 ms), 64^2 alone 14.7 us (58 us).  At 256^2 a
+// point takes 331 instructions of the row kernel and 175 of the column kernel; both are bound by issue
+// slots and the integer multiply pipe (65 % and 53 % of the issue slots, 59 % and 52 % of that pipe),
+// not by HBM (40 bytes per point, 0.1 ms).  Oblong grids (hx != hy) pay 2 % for the precision of R'.
 //
 // Scales.  x = C / 2^E with 2^E just above the band's largest |C| (E from an integer maximum
-// over the loaded values); C enters as x 2^59, mu as mu 2^(kmu - E), where kmu leaves room
-// for the largest R' the stencil can form from such a band (so mu's unit is a few bits below
-// the rounding of the FP64 formula, whose terms 4 (bx + by) C are as large), R' is formed
-// from mu exactly where hx = hy.  Each recurrence y_i = r_i + p1 y_{i-1} + p2 y_{i-2} then
-// runs on r shifted so that its row's (or panel's) largest value sits g bits below 2^62, 2^g
-// a bound of the recurrence's gain (the l1 norm of its impulse response), and its result is
-// shifted the same way before the backward one.
+// over the loaded values); C enters as x 2^59, mu as mu 2^(kmu - E), where kmu leaves room for
+// the largest R' the stencil can form from such a band (so mu's unit is a few bits below the
+// rounding of the FP64 formula, whose terms 4 (bx + by) C are as large), R' is formed in units
+// of the closer spacing, from mu exactly where hx = hy.  Each recurrence y_i = r_i + p1 y_{i-1}
+// + p2 y_{i-2} then runs on r shifted so that its row's (or panel's) largest value sits g bits
+// below 2^62, 2^g a bound of the recurrence's gain (the l1 norm of its impulse response), and
+// its result is shifted the same way before the backward one.
 //
-// A band whose largest |C| is outside [2^-200, 8), or not finite, is taken through the same
-// code in FP64 arithmetic (the Fp policy), its rows marked kBadRow; the columns of a member
-// with such a row run in FP64 too.  So do a band in which some block of 32 columns by 4 rows (halo rows
-// included) holds only values below 2^-10 of the band's largest, and the columns of a member whose
-// bands' largest values differ by that much: a value that far below the one that sets its scale would
-// keep fewer bits than in FP64, which shows in regions so quiet beside others (a field grown from a
-// local seed: 1e-12 noise beside it had a relative error of 7e-3 after a step, now FP64's 2e-12).
-// Above that line the error is FP64's or less relative to the run's largest |C|, and within a factor
-// of 16 of it relative to a block's.  Four rows: a nodal line of one or two rows is no quiet region, and the
-// two rows next to an active one take its flux within the step.
+// A band whose largest |C| is outside [2^-200, 8), or not finite, is taken through the same code
+// in FP64 arithmetic (the Fp policy: 0.91 ms per step of 256 x 256^2 where every band is,
+// FP64 kernels 0.65; 16 x 1024^2 1.01 and 1.15; 64^2 alone 24 and 55 us), its rows marked kBadRow; the columns of a member with such a row run in FP64
+// too.  So do a band in which some block of 32 columns by 4 rows (halo rows included) holds only
+// values below 2^-10 of the band's largest, and the columns of a member whose bands' largest
+// values differ by that much: a value that far below the one that sets its scale would keep
+// fewer bits than in FP64, which shows in regions so quiet beside others (a field grown from a
+// local seed: 1e-12 noise beside it had a relative error of 7e-3 after a step, now FP64's
+// 2e-12). Above that line the error is FP64's or less relative to the run's largest |C|, and
+// within a factor of 16 of it relative to a block's.  Four rows: a nodal line of one or two rows
+// is no quiet region, and the two rows next to an active one take its flux within the step.
 //
 // Lines of n points are split into G = ceil(n / S) segments of S points (the last one may be
 // shorter), one lane (rows) or warp (columns) per segment.  Each recurrence is a pass from a
@@ -206,7 +208,7 @@ __device__ __forceinline__ int all_levels(int G) { return 32 - __clz(G - 1); }
 // free slots, read their constant tables and wait) and waits itself until its predecessor has
 // finished and its writes are visible.  What is read before the wait -- the tiles and the scan
 // tables -- must therefore not come from the predecessor (tables_ready, launch_fx_rows).  64^2 alone:
-// 20.2 us per step without it, 16.5 with it.
+// 20.2 us per step without it, 14.7 with it.
 __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;\n" ::: "memory");
 }
@@ -779,7 +781,7 @@ cudaError_t rows_limit() {
 // A step kernel; as a dependent launch up to one CTA per SM (above, CTAs that start in the slots their
 // predecessor happens to leave free are spread unevenly: 64 x 128^2 51 us per step with it, 39
 // without, 8 x 512^2 76 and 68).
-constexpr int kDependentCtas = 152;
+constexpr int kDependentCtas = 152;  // the GPU's SMs
 
 template <class K>
 void launch_dependent(K kernel, int grid, int block, size_t smem, cudaStream_t st, const DevView& v, int base, bool ready) {

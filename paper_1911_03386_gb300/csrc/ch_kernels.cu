@@ -1755,14 +1755,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(sizeof(T) == 4 ? 102
 //           operations, so it updates its halo rows -- its neighbours' boundary rows --
 //           itself, bit for bit as the neighbours update them: no halo exchange.
 // Bound by latencies: shared memory, the cluster barrier, the serial chains.  us per step of
-// 256 x 256^2 / 32 x 256^2 / 256 x 128^2: 59.2 / 8.2 / 24.7; with the walks and the adjacent rows
-// 55.8 / 7.7 / 24.5; turns in the last wave (res_turns) 54.6 / 7.7 / 22.5; two FP32 values per
-// instruction 53.5 / 7.6 / 22.5; the combination in two serial walks instead of four 51.1 / 7.2 /
-// 22.3; built for the column segments there are (KMAX, FULL) 48.2 / 6.8 / 16.8.
+// 256 x 256^2 / 32 x 256^2 / 256 x 128^2: 48.2 / 6.8 / 16.8, and 59.2 / 8.2 / 24.7 without the walks
+// and adjacent rows, the turns of res_turns, two FP32 values per instruction, the combination in two
+// serial walks and its loops built for the segments there are.
 // The end states are double-buffered by step parity (a CTA may start the next step while
-// others still read this step's).  Sample steps add the FP64 partial sums of the F and
-// dF/dt densities (mu recomputed in FP64 from the stored field, as in the other FP32
-// kernels); rank 0 sums the CTAs' partials in rank order and finalises the sample.  mu and
+// others still read this step's).  Sample steps add the exact partial sums of the F and
+// dF/dt densities (fixed_partials; in FP64 where the range does not fit, mu recomputed from the
+// stored field); rank 0 sums the CTAs' partials in rank order and finalises the sample.  mu and
 // R' are formed in the operation order of the segment-form kernels.
 // -------------------------------------------------------------------------------------
 // NR rows of the field per CTA (32 or 64) with 8 NR threads: every thread owns 2 rows in the
@@ -1989,7 +1988,10 @@ struct ResRun {
   int base, width, pos, parts, nsteps;
 };
 
-// KMAX: column segments (ny / (NX / 8)) at most, or exactly (FULL).
+// KMAX: column segments (ny / (NX / 8)) at most, or exactly (FULL: the tallest members of a form, ny =
+// 256, and 128 at 128 columns; the combination's loops lose their guards: 256 x 256^2 51.1 -> 48.2 us per
+// step).  Heights between keep the guards: 256 members of 256 x 224 46.2 us, 256 x 192 36.7, which
+// per point is 9 % and 1 % more than 256 x 256; 256 x 128 21.9, 9 % less.
 template <int NX, int NR, bool COMP, bool OBS, int KMAX, bool FULL>
 __global__ void __launch_bounds__(8 * NR, NR == 32 ? 2 : 1) res_kernel(DevView v, ResRun run) {
   constexpr int TH = 8 * NR;      // threads per CTA
