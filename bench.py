@@ -239,6 +239,8 @@ def kernel_name(phase, t, elt, nx=256):
     if phase == "rowsweep":
         return ("rowstream_kernel<%s>" if t["stream"] else "rowsweep_kernel<%s>") % ty
     if phase == "rows":
+        if t["row_seg"] in (16, 32) and elt == 4 and not t["persist"] & 2:
+            return "rows_walk_kernel<%d, %d>" % (t["row_seg"], 2 if t["row_seg"] == 16 else 4)
         if t["row_seg"] in (16, 32):
             return "rows_seg_kernel<%s, %d, %s>" % (ty, t["row_seg"], "true" if t["persist"] & 2 else "false")
         return "rowsT_kernel<%s>" % ty if t["row_seg"] == 1 else "rows_kernel<%s, false>" % ty
@@ -594,7 +596,7 @@ def value_estimate(res):
 #   stream64    the same in the FP64 split form: stencil_kernel, rowstream_kernel,
 #               colstream_kernel per step
 #   segment32   FP32 with the resident form off, the whole ensemble (134 MB):
-#               rows_seg_kernel, colseg_kernel per step
+#               rows_walk_kernel, colseg_kernel per step
 # name: (precision, ch_tuning.resident, members, workload)
 KERNEL_CASES = {"resident32": ("fp32", 0, 32, "ensemble"), "fixed64": ("fp64", 0, 256, "ensemble"), "stream64": ("fp64", -1, 256, "ensemble"),
                 "segment32": ("fp32", -1, 256, "ensemble"), "long16": ("fp32", -1, 16, "long")}
