@@ -12,6 +12,7 @@ import numpy as np
 import pytest
 
 import paper_1911_03386_gb300 as ch
+from oracle.oracle import get as get_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -200,6 +201,21 @@ def test_samples_at_large_values(scale):
             out.append((F[0], D[0]))
     for a, b in zip(*out):
         assert abs(a - b) <= 64 * 2.0 ** -53 * abs(b)
+
+
+@pytest.mark.parametrize("scale", [0.9, 2.5, 7.0, 9.0])
+@pytest.mark.parametrize("n", [64, 128])  # tiled, cluster-resident
+def test_fp32_samples_at_large_values(n, scale):
+    # the same sums of CH_FP32 fields against the oracle's FP64 ones, n^2 terms of one sign each: its
+    # n^2 roundings
+    f = separated(n, n)
+    f *= scale / np.max(np.abs(f))
+    with ch.Ensemble.create(n, n, TWO_PI, 0.01, 1e-6, [0.0], 1, ch.CH_FP32) as e:
+        e.set_field(0, f)
+        F, D, _ = e.observables()
+        want = get_oracle().field_observables(e.field(0), TWO_PI, 0.01)
+    for a, b in zip((F[0], D[0]), want):
+        assert abs(a - b) <= n * n * 2.0 ** -53 * abs(b)
 
 
 @pytest.mark.parametrize("nx,ny", [(33, 512), (17, 600)])
