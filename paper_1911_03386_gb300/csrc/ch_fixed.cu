@@ -28,16 +28,17 @@
 // its result is shifted the same way before the backward one.
 //
 // A band whose largest |C| is outside [2^-200, 8), or not finite, is taken through the same code
-// in FP64 arithmetic (the Fp policy: 0.91 ms per step of 256 x 256^2 where every band is,
-// FP64 kernels 0.65; 16 x 1024^2 1.01 and 1.15; 64^2 alone 24 and 55 us), its rows marked kBadRow; the columns of a member with such a row run in FP64
-// too.  So do a band in which some block of 32 columns by 4 rows (halo rows included) holds only
-// values below 2^-10 of the band's largest, and the columns of a member whose bands' largest
-// values differ by that much: a value that far below the one that sets its scale would keep
-// fewer bits than in FP64, which shows in regions so quiet beside others (a field grown from a
-// local seed: 1e-12 noise beside it had a relative error of 7e-3 after a step, now FP64's
-// 2e-12). Above that line the error is FP64's or less relative to the run's largest |C|, and
-// within a factor of 16 of it relative to a block's.  Four rows: a nodal line of one or two rows
-// is no quiet region, and the two rows next to an active one take its flux within the step.
+// in FP64 arithmetic (the Fp policy: 0.91 ms per step of 256 x 256^2 where every band is, FP64
+// kernels 0.65; 16 x 1024^2 1.01 and 1.15; 64^2 alone 24 and 55 us), its rows marked kBadRow;
+// the columns of a member with such a row run in FP64 too.  So do a band in which some block of
+// 32 columns (16 to 32 at the end of a row) by 4 rows (halo rows included) holds only values
+// below 2^-10 of the band's largest, and the columns of a member whose bands' largest values
+// differ by that much: a value that far below the one that sets its scale would keep fewer bits
+// than in FP64, which shows in regions so quiet beside others (a field grown from a local seed:
+// 1e-12 noise beside it had a relative error of 7e-3 after a step, now FP64's 2e-12). Above that
+// line the error is FP64's or less relative to the run's largest |C|, and within a factor of 16
+// of it relative to a block's.  Four rows: a nodal line of one or two rows is no quiet region,
+// and the two rows next to an active one take its flux within the step.
 //
 // Lines of n points are split into G = ceil(n / S) segments of S points (the last one may be
 // shorter), one lane (rows) or warp (columns) per segment.  Each recurrence is a pass from a
@@ -468,6 +469,7 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
   for (int s = warp; s < b.ns; s += NW) {  // this thread's own copies
     const int i = min(32 * s + lane, nx - 1);
     const int2* col = reinterpret_cast<const int2*>(b.tile + i + (i >> b.ls));
+    const bool wide = 32 * s + 16 <= nx;  // a last strip of a few columns may lie along a nodal line
 #pragma unroll 2
     for (int t = 0; t < nr + 4; t += 4) {
       const int2* at = col + min(t, nr) * b.pitch;  // the last block may overlap the one before
@@ -476,7 +478,7 @@ __global__ void __launch_bounds__(TH, MINB) fx_rows_kernel(DevView v, int tile_b
       for (int q = 0; q < 4; ++q) block = max(block, (unsigned)at[q * b.pitch].y & 0x7fffffffu);
       block = __reduce_max_sync(kAll, block);
       top = max(top, block);
-      low = min(low, block);
+      if (wide) low = min(low, block);
     }
   }
   if (lane == 0) {
