@@ -253,8 +253,10 @@ __device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + 
 // of the step's mu, sums of squares of 128 bits per strip and lane added exactly, so the result does
 // not depend on the CTA's size) it costs about one.  A warp takes 29 columns (lanes 0, 30 and 31 are their neighbours) of a
 // strip of 4 or 8 rows.  sums: 80 bytes of shared memory; ends with every thread past a barrier;
-// false (nothing summed) where the values' range does not fit, the same in every thread.
-template <class Load, class Conv, class Mag>
+// false (nothing summed) where the values' range does not fit, the same in every thread.  MAXE: |C| <
+// 2^MAXE fits, 1 for CH_FP32 (with the exponents of the CH_FP64 step the resident kernel around it took
+// 48.6 us per step of 256 x 256^2 instead of 47.5, samples or not).
+template <int MAXE, class Load, class Conv, class Mag>
 __device__ __noinline__ bool fixed_partials(const MemberParams& P, int nx, int nr, unsigned long long* sums, Load load,
                                             Conv conv, Mag mag, double& sF, double& sD) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -273,15 +275,15 @@ __device__ __noinline__ bool fixed_partials(const MemberParams& P, int nx, int n
   __syncthreads();
   const int emax = __reduce_max_sync(kAll, lane < nw ? (int)slots[lane] : 0);
   __syncthreads();
-  if (!P.fx_mu || emax > 1022 + kFxMaxE || emax < 823) return false;
+  if (!P.fx_mu || emax > 1022 + MAXE || emax < 823) return false;
   if (threadIdx.x < 10) sums[threadIdx.x] = 0;
   __syncthreads();
-  const int E = emax - 1022, cut = E > 1 ? P.fx_cut[E - 2] : 0, kmu = P.fx_kmu - cut;
-  const int wb = 60 - 2 * max(E, 1), sh = 2 * E + wb - 54;  // C^2 - 1 is held times 2^wb
+  const int E = emax - 1022, cut = MAXE > 1 && E > 1 ? P.fx_cut[E - 2] : 0;
+  const int wb = MAXE > 1 ? 60 - 2 * max(E, 1) : 58, sh = max(2 * E + wb - 54, -63);  // C^2 - 1 is held times 2^wb
   const i64 one = 1ll << wb;
   const FxLimb bx = cut_limb(P.fx_bx, cut), by = cut_limb(P.fx_by, cut);
   const int su = P.fx_su + cut + wb - 60;  // the cubic term from (C^2 - 1) 2^wb
-  auto scaled = [](i64 v, int s) { return s >= 0 ? v << s : v >> min(-s, 63); };
+  auto scaled = [](i64 v, int s) { return s >= 0 ? v << s : v >> -s; };
   for (int item = warp; item < nchunk * nstrip; item += nw) {
     const int k = item % nchunk, r0 = (item / nchunk) * hs, r1 = min(nr, r0 + hs);
     if (r0 >= r1) continue;
@@ -344,7 +346,7 @@ __device__ __noinline__ bool fixed_partials(const MemberParams& P, int nx, int n
     const int q = min(lane, 4);
     const double hinv = (q & 1) ? P.ihx2 : P.ihy2;
     const double weight = q == 0 ? pow2(14 - 2 * wb) : q < 3 ? 0.5 * P.gamma * pow2(16 + 2 * (E - 59)) * hinv
-                                                          : pow2(16 + 2 * (E - kmu)) * hinv;
+                                                          : pow2(16 + 2 * (E - P.fx_kmu + cut)) * hinv;
     const double s = weight * fma((double)sums[2 * q + 1], 18446744073709551616.0, (double)sums[2 * q]);
     sF = s + (__shfl_sync(kAll, s, 1) + __shfl_sync(kAll, s, 2));
     sD = __shfl_sync(kAll, s, 3) + __shfl_sync(kAll, s, 4);
@@ -368,7 +370,7 @@ __device__ void band_partials_field(const DevView& v, const Tile& tl, int nx, in
     return (int64_t)j * nx + i;
   };
   double sF, sD;
-  const bool ok = fixed_partials(
+  const bool ok = fixed_partials<sizeof(T) == 8 ? kFxMaxE : 1>(
       P, nx, nr, reinterpret_cast<unsigned long long*>(red),
       [=](int r, int i) {
         const int64_t k = index(r, i);

@@ -1956,7 +1956,7 @@ __device__ __forceinline__ void res_partials(const float* Ct, const float* Lt, c
 template <int NX, int NR, bool COMP>
 __device__ __forceinline__ void res_sample(const float* Ct, const float* Lt, const MemberParams& P, double* red,
                                            double& sF, double& sD) {
-  const bool ok = fixed_partials(
+  const bool ok = fixed_partials<1>(
       P, NX, NR, reinterpret_cast<unsigned long long*>(red),
       [=](int r, int i) {
         const int k = (r + 2) * NX + i;
